@@ -32,24 +32,29 @@ size_t dtype_bytes(int dt) { return dt == DT_F64 ? 8 : (dt == DT_F32 ? 4 : 2); }
 // tw x th chunks); kind 1 / 2 / 3 / 4: TMA-staged D2Q9 kernel with node
 // pairs (V = 2) in the large-tile / small-tile / wide-CTA / deep-ring
 // geometry (smem_tile_nodes variant kind - 1), tile width per instance.
+// Kind 0 with V = 1 is the FP64 kernel with one node per thread (warps of 32
+// consecutive nodes: tw = 32, th = 1).
 struct Shape {
     int V, tw, th;
     int kind = 0;
+    bool flat() const { return kind == 0 && V == 1; }
 };
 
 Shape default_shape(int lattice, int storage) {
     if (lattice == 1) return {storage == DT_F64 ? 2 : 4, 128, 1};
-    if (storage == DT_F64) return {2, 16, 8};
+    if (storage == DT_F64) return {1, 32, 1};
     if (storage == DT_F32) return {4, 16, 8};
     return {8, 8, 16};
 }
 
 // Launch-shape candidates of the autotuner.  D2Q9 with FP32 arithmetic: the
 // TMA-staged kernel in its four geometries and the default register-chunk
-// shape (which wins only on small, cache-resident lattices).  D1Q3 and the
-// FP64 path: register-chunk shapes, V = the compiled widths of the storage
-// type, tiles of 128 or 256 threads.
-std::vector<Shape> candidate_shapes(int lattice, int storage, int64_t max_nx, int64_t max_ny) {
+// shape (which wins only on small, cache-resident lattices).  D2Q9 in FP64:
+// one node per thread (measured ahead of every register-chunk shape from
+// 800 x 4 to 2048^2 nodes, so nothing is timed).  D1Q3: register-chunk
+// shapes, V = the compiled widths of the storage type, tiles of 128 or 256
+// threads.
+std::vector<Shape> candidate_shapes(int lattice, int storage, int64_t max_nx) {
     std::vector<Shape> out;
     if (lattice == 2 && storage != DT_F64) {
         out.push_back({2, 0, 0, 1});  // TMA-staged kernel, node pairs, large tiles
@@ -59,23 +64,18 @@ std::vector<Shape> candidate_shapes(int lattice, int storage, int64_t max_nx, in
         out.push_back(default_shape(lattice, storage));
         return out;
     }
+    if (lattice == 2) {
+        out.push_back(default_shape(lattice, storage));
+        return out;
+    }
     std::vector<int> vs;
     if (storage == DT_F64) vs = {2};
     else if (storage == DT_F32) vs = {2, 4};
     else vs = {4, 8};
     for (int V : vs) {
         for (int block : {128, 256}) {
-            if (lattice == 1) {
-                if ((int64_t)block * V > 2 * std::max<int64_t>(max_nx, 8) && block > 128) continue;
-                out.push_back({V, block, 1});
-                continue;
-            }
-            for (int tw : {8, 16, 32}) {
-                const int th = block / tw;
-                if (th > max_ny && tw < 32) continue;
-                if ((int64_t)tw * V > 2 * std::max<int64_t>(max_nx, 8) && tw > 8) continue;
-                out.push_back({V, tw, th});
-            }
+            if ((int64_t)block * V > 2 * std::max<int64_t>(max_nx, 8) && block > 128) continue;
+            out.push_back({V, block, 1});
         }
     }
     return out;
@@ -208,6 +208,7 @@ struct lbm_ctx {
     bool post = false;  // stored field is post-collision
     int64_t steps = 0;
     Shape shape{};
+    int flat_nodes = 0;  // one-node-per-thread kernel: nodes per tile-table entry
     const void* kern = nullptr;
     int grid = 0;
     size_t smem = 0;  // dynamic shared memory of the step kernel
@@ -259,6 +260,27 @@ AuxArgs aux_args(const lbm_ctx* ctx) {
     return a;
 }
 
+// One-node-per-thread kernel: colliding nodes of an instance, nodes per
+// tile-table entry (the fewest, from one warp up, whose entries fit the
+// table) and CTA size.
+int64_t flat_fluid(int64_t nx, int64_t ny, int bc) {
+    return bc == LBM_BC_CAVITY ? (nx - 2) * (ny - 2) : nx * ny;
+}
+int flat_nodes(const lbm_ctx* ctx) {
+    for (int e = 32;; e *= 2) {
+        int64_t n = 0;
+        for (const InstDesc& in : ctx->layout.inst) {
+            const int64_t fluid = flat_fluid(in.nx, in.ny, ctx->bc);
+            n += (fluid + e - 1) / e + ((int64_t)in.nx * in.ny - fluid + e - 1) / e;
+        }
+        if (n <= ctx->layout.max_tiles) return e;
+    }
+}
+int block_threads(const lbm_ctx* ctx, const Shape& s) {
+    if (s.kind >= 1) return smem_block_threads(s.kind - 1);
+    return s.flat() ? std::min(ctx->flat_nodes, FLAT_MAX_THREADS) : s.tw * s.th;
+}
+
 std::vector<TileDesc> build_tiles(const lbm_ctx* ctx, const Shape& s) {
     std::vector<TileDesc> t;
     if (s.kind >= 1) {
@@ -272,6 +294,20 @@ std::vector<TileDesc> build_tiles(const lbm_ctx* ctx, const Shape& s) {
                 for (int64_t x0 = 0; x0 < in.nx; x0 += X)
                     t.push_back({(int32_t)i, (int32_t)x0, (int32_t)y0, (int32_t)X});
         }
+        return t;
+    }
+    if (s.flat()) {
+        // flat_nodes consecutive nodes per entry: the fluid nodes of every
+        // instance, then the rings of the cavities
+        for (int part = 0; part < 2; ++part)
+            for (int i = 0; i < ctx->count; ++i) {
+                const InstDesc& in = ctx->layout.inst[i];
+                const int64_t n = (int64_t)in.nx * in.ny, fluid = flat_fluid(in.nx, in.ny, ctx->bc);
+                const int64_t end = part == 0 ? fluid : n;
+                for (int64_t k = part == 0 ? 0 : fluid; k < end; k += ctx->flat_nodes)
+                    t.push_back({(int32_t)i, (int32_t)k,
+                                 (int32_t)std::min<int64_t>(k + ctx->flat_nodes, end), 0});
+            }
         return t;
     }
     for (int i = 0; i < ctx->count; ++i) {
@@ -307,30 +343,24 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
         const int rc = build_tensor_maps(ctx, var);
         if (rc != LBM_OK) return rc;
     } else {
+        if (s.flat() && (s.tw != 32 || s.th != 1)) return LBM_ERR_ARG;
         k = find_step_kernel(ctx->lattice, ctx->storage, ctx->collision, s.V);
     }
     if (!k) return LBM_ERR_ARG;
+    if (s.flat()) ctx->flat_nodes = flat_nodes(ctx);
     std::vector<TileDesc> t = build_tiles(ctx, s);
     if ((int64_t)t.size() > ctx->layout.max_tiles) return LBM_ERR_ARG;
-    // the instance table records each instance's tile range
-    int32_t idx = 0;
-    for (int i = 0; i < ctx->count; ++i) {
-        ctx->layout.inst[i].tile0 = idx;
-        int32_t n = 0;
-        while (idx + n < (int32_t)t.size() && t[idx + n].inst == i) ++n;
-        ctx->layout.inst[i].ntiles = n;
-        idx += n;
-    }
     LBM_CK(cudaMemcpyAsync(ctx->d_tiles, t.data(), sizeof(TileDesc) * t.size(),
                            cudaMemcpyHostToDevice, ctx->stream));
     LBM_CK(cudaMemcpyAsync(ctx->d_inst, ctx->layout.inst.data(), sizeof(InstDesc) * ctx->count,
                            cudaMemcpyHostToDevice, ctx->stream));
     LBM_CK(cudaStreamSynchronize(ctx->stream));
-    const int block = s.kind >= 1 ? smem_block_threads(s.kind - 1) : s.tw * s.th;
+    const int block = block_threads(ctx, s);
     int per_sm = 0;
     LBM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
     per_sm = std::max(per_sm, 1);
-    const int64_t g = std::min<int64_t>((int64_t)per_sm * ctx->num_sms, (int64_t)t.size());
+    const int64_t g = s.flat() ? (int64_t)t.size() * (ctx->flat_nodes / block)
+                               : std::min<int64_t>((int64_t)per_sm * ctx->num_sms, (int64_t)t.size());
     ctx->tiles.swap(t);
     ctx->shape = s;
     ctx->kern = k;
@@ -403,7 +433,7 @@ StepArgs step_args(const lbm_ctx* ctx, int src) {
     a.inst = ctx->d_inst;
     a.tiles = ctx->d_tiles;
     a.ntiles = (int32_t)ctx->tiles.size();
-    a.tw = ctx->shape.tw;
+    a.tw = ctx->shape.flat() ? ctx->flat_nodes : ctx->shape.tw;
     a.tw_log2 = ctx->shape.tw > 0 ? ilog2(ctx->shape.tw) : 0;
     a.th = ctx->shape.th;
     a.rho0 = ctx->rho0;
@@ -414,17 +444,18 @@ StepArgs step_args(const lbm_ctx* ctx, int src) {
     a.error = ctx->d_error;
     a.spin_limit = ctx->spin_limit;
     a.lost_tile = ctx->lost_tile;
+    a.inplace = 0;
     return a;
 }
 
 // One step launch.  It is a programmatic dependent launch: the kernel may be
 // scheduled while the previous kernel in the stream drains, and waits for its
 // completion (griddepcontrol.wait) before touching device state.
-cudaError_t launch_step(lbm_ctx* ctx, int src, cudaStream_t s) {
+cudaError_t launch_step(lbm_ctx* ctx, int src, cudaStream_t s, bool inplace = false) {
     StepArgs a = step_args(ctx, src);
+    a.inplace = inplace ? 1 : 0;  // one-node-per-thread kernel only
     void* params[] = {&a};
-    const int block = ctx->shape.kind >= 1 ? smem_block_threads(ctx->shape.kind - 1)
-                                           : ctx->shape.tw * ctx->shape.th;
+    const int block = block_threads(ctx, ctx->shape);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -569,8 +600,8 @@ int autotune(lbm_ctx* ctx) {
     const std::string key = tune_key(ctx);
     Shape cached;
     if (tune_lookup(key, &cached) && apply_shape(ctx, cached) == LBM_OK) return LBM_OK;
-    std::vector<Shape> cands = candidate_shapes(ctx->lattice, ctx->storage, ctx->layout.max_nx,
-                                                ctx->layout.max_ny);
+    std::vector<Shape> cands = candidate_shapes(ctx->lattice, ctx->storage, ctx->layout.max_nx);
+    if (cands.size() == 1) return apply_shape(ctx, cands[0]);
     cudaEvent_t ev[6];
     for (int i = 0; i < 6; ++i) LBM_CK(cudaEventCreate(&ev[i]));
     float best = 1e30f;
@@ -1032,9 +1063,13 @@ int lbm_step(lbm_ctx* ctx, int64_t n) {
     if (!ctx->initialized) return LBM_ERR_STATE;
     if (n == 0) return LBM_OK;
     if (!ctx->post) {
-        AuxArgs a = aux_args(ctx);
-        LBM_CK(run_aux(AuxOp::CollideInPlace, a, ctx->buf[ctx->cur], ctx->buf[1 - ctx->cur],
-                       nullptr, nullptr, nullptr, nullptr, nullptr, nullptr));
+        if (ctx->shape.flat()) {
+            LBM_CK(launch_step(ctx, ctx->cur, ctx->stream, true));
+        } else {
+            AuxArgs a = aux_args(ctx);
+            LBM_CK(run_aux(AuxOp::CollideInPlace, a, ctx->buf[ctx->cur], ctx->buf[1 - ctx->cur],
+                           nullptr, nullptr, nullptr, nullptr, nullptr, nullptr));
+        }
         ctx->cur = 1 - ctx->cur;
         ctx->post = true;
         ctx->steps += 1;

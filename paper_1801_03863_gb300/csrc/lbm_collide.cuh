@@ -44,6 +44,7 @@
 // one rounding (Num<T>::mad).
 #pragma once
 #include "lbm_common.cuh"
+#include "lbm_f64.cuh"
 #include "lbm_num.cuh"
 
 namespace lbm {
@@ -76,7 +77,9 @@ __device__ __forceinline__ typename Num<T>::Pred finite_nonneg(const T (&out)[Q]
                                                                const double (&w)[Q], T rho0) {
     using N = Num<T>;
     typename N::Pred ok;
-    if constexpr (N::LANES == 1) {
+    if constexpr (std::is_same<T, double>::value) {
+        ok = finite_nonneg_f64<Q>(out, w, rho0);
+    } else if constexpr (N::LANES == 1) {
         ok = true;
 #pragma unroll
         for (int a = 0; a < Q; ++a) ok = ok && (out[a] >= -T(w[a]) * rho0);
@@ -146,33 +149,6 @@ __device__ __forceinline__ uint32_t plain_status(const T (&out)[Q], const double
     }
 }
 
-// 4x4 symmetric positive definite solve A x = b by an LDL^T factorisation:
-// A = L D L^T with unit lower-triangular L, then L z = b, x = L^-T D^-1 z.
-// Four reciprocals (of the pivots) and 32 multiply-adds; A is given as its
-// 10 unique entries, unknown order (1, 2, 3, 4).
-template <typename T>
-__device__ __forceinline__ void spd4_solve(T a11, T a21, T a22, T a31, T a32, T a33, T a41, T a42,
-                                           T a43, T a44, T b1, T b2, T b3, T b4, T& x1, T& x2,
-                                           T& x3, T& x4) {
-    using N = Num<T>;
-    const T r1 = N::rcp(a11);
-    const T l21 = a21 * r1, l31 = a31 * r1, l41 = a41 * r1;
-    const T r2 = N::rcp(N::mad(-l21, a21, a22));
-    const T t32 = N::mad(-l31, a21, a32), t42 = N::mad(-l41, a21, a42);
-    const T l32 = t32 * r2, l42 = t42 * r2;
-    const T r3 = N::rcp(N::mad(-l32, t32, N::mad(-l31, a31, a33)));
-    const T t43 = N::mad(-l42, t32, N::mad(-l41, a31, a43));
-    const T l43 = t43 * r3;
-    const T r4 = N::rcp(N::mad(-l43, t43, N::mad(-l42, t42, N::mad(-l41, a41, a44))));
-    const T z2 = N::mad(-l21, b1, b2);
-    const T z3 = N::mad(-l32, z2, N::mad(-l31, b1, b3));
-    const T z4 = N::mad(-l43, z3, N::mad(-l42, z2, N::mad(-l41, b1, b4)));
-    x4 = z4 * r4;
-    x3 = N::mad(-l43, x4, z3 * r3);
-    x2 = N::mad(-l42, x4, N::mad(-l32, x3, z2 * r2));
-    x1 = N::mad(-l41, x4, N::mad(-l31, x3, N::mad(-l21, x2, b1 * r1)));
-}
-
 #ifndef LBM_MX4_LOGP
 #define LBM_MX4_LOGP 1  // FP32 MinxEnt4: logarithms of pair products / quotients (7 instead of 9)
 #endif
@@ -219,8 +195,7 @@ __device__ __forceinline__ uint32_t minxent_d2q9(const T (&d)[9], T rho0, const 
                                                  T (&out)[9]) {
     static_assert(NFREE == 4 || NFREE == 2, "MinxEnt4 or MinxEnt2");
     using N = Num<T>;
-    constexpr bool FP64 = std::is_same<T, double>::value;
-    static_assert(!(YFORM && FP64), "the direct form is for 2-byte storage with FP32 arithmetic");
+    static_assert(!std::is_same<T, double>::value, "FP64 nodes collide in minxent_f64");
     const T omega = r.omega;
     constexpr double W[9] = {4.0 / 9.0,  1.0 / 9.0,  1.0 / 9.0,  1.0 / 9.0, 1.0 / 9.0,
                              1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0};
@@ -306,20 +281,14 @@ __device__ __forceinline__ uint32_t minxent_d2q9(const T (&d)[9], T rho0, const 
         cp = C1 + sp;
         cm = C1 + sm;
     }
-    // FP64: the exact test of reading C-NEG.  FP32: see the Newton-step test below.
-    typename N::Pred ok{};
-    if constexpr (FP64) {
-        const T mn = N::vmin(N::vmin(N::vmin(y[0], y[1]), N::vmin(y[2], y[3])),
-                             N::vmin(N::vmin(y[4], y[5]), N::vmin(N::vmin(y[6], y[7]), y[8])));
-        ok = N::gt(mn, T(0.0));
-    }
+    typename N::Pred ok{};  // set where some lane skips its step, see the Newton-step test below
 
     // q_a = W_a / p_a = 1 / y_a.  FP32: opposite populations share one
     // reciprocal of their product (each result within ~2 ulp); with
     // LBM_SHARED_RCP the four products and y_0 share a single one.
     T q[9];
     T p13 = T(0.0), p24 = T(0.0), p57 = T(0.0), p68 = T(0.0), pa = T(0.0), pd = T(0.0);
-    if constexpr (!FP64) {
+    {
         p13 = y[1] * y[3]; p24 = y[2] * y[4]; p57 = y[5] * y[7]; p68 = y[6] * y[8];
         T r13, r24, r57, r68;
         if constexpr (LBM_SHARED_RCP) {
@@ -339,9 +308,6 @@ __device__ __forceinline__ uint32_t minxent_d2q9(const T (&d)[9], T rho0, const 
         q[2] = y[4] * r24; q[4] = y[2] * r24;
         q[5] = y[7] * r57; q[7] = y[5] * r57;
         q[6] = y[8] * r68; q[8] = y[6] * r68;
-    } else {
-#pragma unroll
-        for (int a = 0; a < 9; ++a) q[a] = N::rcp(y[a]);
     }
 
     // Gradient terms ln(p/W) (natural or base-2 logs, see Num::LOG_SCALE):
@@ -351,7 +317,7 @@ __device__ __forceinline__ uint32_t minxent_d2q9(const T (&d)[9], T rho0, const 
     // and diagonal products (3 instead of 9).  FP32 MinxEnt4 with
     // LBM_MX4_LOGP takes the differences as logarithms of the quotients
     // y_a q_opp(a) as well (7 instead of 9).
-    constexpr bool LOGP = !FP64 && (NFREE == 2 || LBM_MX4_LOGP);
+    constexpr bool LOGP = NFREE == 2 || LBM_MX4_LOGP;
     T L0, La, Ld, D31 = T(0.0), D42 = T(0.0), l57 = T(0.0), l68 = T(0.0);
     if constexpr (LOGP) {
         if constexpr (!LBM_SHARED_RCP) {
@@ -418,14 +384,7 @@ __device__ __forceinline__ uint32_t minxent_d2q9(const T (&d)[9], T rho0, const 
     }
     // a node whose start point is not positive keeps p^start (reading C-NEG)
     bool rare = false;  // some lane skipped its Newton step (FP32 paths)
-    if constexpr (FP64) {
-        se = N::sel(ok, se, T(0.0));
-        sps = N::sel(ok, sps, T(0.0));
-        if constexpr (NFREE == 4) {
-            sx_ = N::sel(ok, sx_, T(0.0));
-            sy_ = N::sel(ok, sy_, T(0.0));
-        }
-    } else {
+    {
         // FP32: a start probability <= 0 gives log2 = NaN or -inf, which the
         // solve carries into every component of the step; a step that is not
         // finite (this, or an overflowing solve) is skipped.  chk = c - c is
@@ -529,14 +488,10 @@ __device__ __forceinline__ uint32_t minxent_d2q9(const T (&d)[9], T rho0, const 
             const T wa = T(W[a]);
             out[a] = N::mad(-rs, t[a], N::mad(wa * rho, del[a], wa * drho));
         }
-        if constexpr (FP64) {
-            return lane_status<T>(ok, finite_nonneg<T, 9>(out, W, rho0));
-        } else {
-            if (rare) return lane_status<T>(ok, finite_nonneg<T, 9>(out, W, rho0));
-            // every step was finite, and so are the populations: only the sign of
-            // f^post = W rho0 + out remains to test (OR of the sign bits)
-            return sign_status<T, 9>(out, W, rho0);
-        }
+        if (rare) return lane_status<T>(ok, finite_nonneg<T, 9>(out, W, rho0));
+        // every step was finite, and so are the populations: only the sign of
+        // f^post = W rho0 + out remains to test (OR of the sign bits)
+        return sign_status<T, 9>(out, W, rho0);
     }
 }
 
@@ -681,15 +636,19 @@ template <class Lat, int COLL, typename T, int SB = 8> struct Collide;
 template <typename T, int SB> struct Collide<D2Q9, COLL_MINXENT4, T, SB> {
     __device__ static __forceinline__ uint32_t run(const T (&d)[9], T rho0, const Rates<T>& r,
                                                    T (&o)[9]) {
-        return minxent_d2q9<T, 4, LBM_YFORM && SB == 2 && !std::is_same<T, double>::value>(
-            d, rho0, r, o);
+        if constexpr (std::is_same<T, double>::value)
+            return minxent_f64<4>(d, rho0, r.omega, r.omega2, o);
+        else
+            return minxent_d2q9<T, 4, LBM_YFORM && SB == 2>(d, rho0, r, o);
     }
 };
 template <typename T, int SB> struct Collide<D2Q9, COLL_MINXENT2, T, SB> {
     __device__ static __forceinline__ uint32_t run(const T (&d)[9], T rho0, const Rates<T>& r,
                                                    T (&o)[9]) {
-        return minxent_d2q9<T, 2, LBM_YFORM && SB == 2 && !std::is_same<T, double>::value>(
-            d, rho0, r, o);
+        if constexpr (std::is_same<T, double>::value)
+            return minxent_f64<2>(d, rho0, r.omega, r.omega2, o);
+        else
+            return minxent_d2q9<T, 2, LBM_YFORM && SB == 2>(d, rho0, r, o);
     }
 };
 template <typename T, int SB> struct Collide<D2Q9, COLL_SRT, T, SB> {

@@ -102,14 +102,15 @@ struct alignas(16) InstDesc {
     double lid_dev[9];  // f^eq_a(rho0, (u_lid, 0)) - W_a rho0, FP64
     float lid_dev_f[9]; // the same rounded to FP32
     float rates_f[4];   // omega, omega2, s_e, s_eps rounded to FP32
-    int32_t tile0, ntiles;  // this instance's tiles in the tile table
+    int32_t pad[2];
 };
 static_assert(sizeof(InstDesc) % 16 == 0, "bulk copies move multiples of 16 bytes");
 
 struct TileDesc {
     int32_t inst;  // instance index
-    int32_t cx0;   // first thread chunk (units of V nodes) in x
-    int32_t y0;    // first row
+    int32_t cx0;   // first thread chunk (units of V nodes) in x, node in x (TMA kernel), or
+                   // first node in row-major order (one-node-per-thread kernel)
+    int32_t y0;    // first row (one-node-per-thread kernel: end of the node range)
     int32_t pad;
 };
 
@@ -125,7 +126,8 @@ struct StepArgs {
     const InstDesc* inst;
     const TileDesc* tiles;
     int32_t ntiles;
-    int32_t tw;       // tile width in chunks (power of two)
+    int32_t tw;       // tile width in chunks (power of two; one-node-per-thread
+                      // kernel: nodes of a tile-table entry)
     int32_t tw_log2;
     int32_t th;       // tile height in rows
     double rho0;
@@ -136,7 +138,13 @@ struct StepArgs {
     unsigned int* error;         // device error word (bounded waits that ran out)
     int32_t spin_limit;          // polls of one bounded mbarrier wait (TMA kernel)
     int32_t lost_tile;           // test hook: tile whose copies are never issued (-1: none)
+    int32_t inplace;             // FP64 one-node-per-thread kernel: collide without streaming
 };
+
+// Most threads of a CTA of the one-node-per-thread kernel.
+#ifndef FLAT_MAX_THREADS
+#define FLAT_MAX_THREADS 32
+#endif
 
 __host__ __device__ inline int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
 

@@ -1,7 +1,7 @@
 // lbm_num.cuh -- arithmetic types of the collision kernels.
 //
 // The collision rules are written once over a number type T:
-//   double  FP64 path: IEEE division, library log1p.
+//   double  FP64 path: Newton reciprocal (below) and table logarithm (lbm_f64.cuh).
 //   float   FP32 path, one node per value.
 //   F2      FP32 path, two nodes per value: the packed FP32x2 instructions of
 //           sm_100+ (__fadd2_rn, __fmul2_rn, __ffma2_rn) do both nodes in one
@@ -34,6 +34,20 @@ __device__ __forceinline__ float lg2_approx(float x) {
     float r;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
+}
+
+// 1 / x in FP64: the 20-bit hardware seed and one third-order Newton step,
+// r (1 + e + e^2) with e = 1 - x r (error e^3 < 2^-60, then one rounding):
+// 3 FP64 instructions instead of an IEEE division's 8.  Operands near the
+// ends of the exponent range, zeros, infinities and NaN take the division.
+__device__ __noinline__ static double rcp_f64_slow(double x) { return 1.0 / x; }
+__device__ __forceinline__ double rcp_f64(double x) {
+    const uint32_t ex = ((uint32_t)__double2hiint(x) >> 20) & 0x7ffu;
+    if (ex - 64u >= 1920u) return rcp_f64_slow(x);
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
 struct F2 {
@@ -76,14 +90,8 @@ template <typename T> struct Num;
 template <> struct Num<double> {
     using Pred = bool;
     static constexpr int LANES = 1;
-    static constexpr double LOG_SCALE = 1.0;  // log returns natural logs
     __device__ static __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
-    __device__ static __forceinline__ double rcp(double x) { return 1.0 / x; }
-    // ln(1 + delta), given delta and y = 1 + delta
-    __device__ static __forceinline__ double lnp(double delta, double) { return log1p(delta); }
-    __device__ static __forceinline__ double vmin(double a, double b) { return fmin(a, b); }
-    __device__ static __forceinline__ Pred gt(double a, double b) { return a > b; }
-    __device__ static __forceinline__ double sel(Pred p, double a, double b) { return p ? a : b; }
+    __device__ static __forceinline__ double rcp(double x) { return rcp_f64(x); }
     __device__ static __forceinline__ double lane(double v, int) { return v; }
     __device__ static __forceinline__ void set_lane(double& v, int, double x) { v = x; }
 };
@@ -141,5 +149,32 @@ template <> struct Num<F2> {
 template <typename T> struct LaneOf { using type = T; };
 template <> struct LaneOf<F2> { using type = float; };
 template <> struct LaneOf<F1> { using type = float; };
+
+// 4x4 symmetric positive definite solve A x = b by an LDL^T factorisation:
+// A = L D L^T with unit lower-triangular L, then L z = b, x = L^-T D^-1 z.
+// Four reciprocals (of the pivots) and 32 multiply-adds; A is given as its
+// 10 unique entries, unknown order (1, 2, 3, 4).
+template <typename T>
+__device__ __forceinline__ void spd4_solve(T a11, T a21, T a22, T a31, T a32, T a33, T a41, T a42,
+                                           T a43, T a44, T b1, T b2, T b3, T b4, T& x1, T& x2,
+                                           T& x3, T& x4) {
+    using N = Num<T>;
+    const T r1 = N::rcp(a11);
+    const T l21 = a21 * r1, l31 = a31 * r1, l41 = a41 * r1;
+    const T r2 = N::rcp(N::mad(-l21, a21, a22));
+    const T t32 = N::mad(-l31, a21, a32), t42 = N::mad(-l41, a21, a42);
+    const T l32 = t32 * r2, l42 = t42 * r2;
+    const T r3 = N::rcp(N::mad(-l32, t32, N::mad(-l31, a31, a33)));
+    const T t43 = N::mad(-l42, t32, N::mad(-l41, a31, a43));
+    const T l43 = t43 * r3;
+    const T r4 = N::rcp(N::mad(-l43, t43, N::mad(-l42, t42, N::mad(-l41, a41, a44))));
+    const T z2 = N::mad(-l21, b1, b2);
+    const T z3 = N::mad(-l32, z2, N::mad(-l31, b1, b3));
+    const T z4 = N::mad(-l43, z3, N::mad(-l42, z2, N::mad(-l41, b1, b4)));
+    x4 = z4 * r4;
+    x3 = N::mad(-l43, x4, z3 * r3);
+    x2 = N::mad(-l42, x4, N::mad(-l32, x3, z2 * r2));
+    x1 = N::mad(-l41, x4, N::mad(-l31, x3, N::mad(-l21, x2, b1 * r1)));
+}
 
 }  // namespace lbm

@@ -313,6 +313,121 @@ __global__ void __launch_bounds__(256) step_kernel(const StepArgs args) {
     }
 }
 
+// ---------------------------------------------------------------------------
+// The FP64 D2Q9 step with one node per thread and one warp per CTA.
+//
+// FP64 arithmetic bounds this step on GB300 (lbm_f64.cuh): a warp
+// instruction holds its scheduler's FP64 unit for 64 cycles, whatever the
+// number of active lanes, so what counts is that every scheduler gets the
+// same number of full warps, down to the smallest lattices.  Nodes are
+// numbered linearly, without tile padding; in a cavity the fluid nodes come
+// first and the outer ring (walls and lid, which do not collide) after them,
+// and the tile table lists the ring entries of all instances behind the
+// fluid ones, so that the colliding CTAs go to the SMs in turn.  An entry
+// covers up to args.tw nodes, [cx0, y0) of one instance in that numbering,
+// and args.tw / blockDim.x CTAs.  CTAs are single warps: with 64 or 128
+// threads whole CTAs are dealt to the SMs and the last round fills worse
+// (257 x 257: 42.6 us a step with one warp, 52.8 with two or four; 17 x 17
+// lattices alike within 1 %).
+//
+// Measured, MinxEnt4, per step, against the register-chunk kernel with log1p
+// and IEEE divisions: 120 lattices of 17 x 17: 122.5 -> 18.9 us; 257 x 257:
+// 110 -> 37.1 us; 800 x 4: 50 -> 12-16 us; 2048 x 2048: 3680 -> 1903 us (250
+// FP64 instructions per node against 485; 0.88 of the FP64 issue rate).
+//
+// inplace: the first step after a state was loaded collides f(x, t_n) itself,
+// without streaming.
+// ---------------------------------------------------------------------------
+template <int COLL>
+__global__ void __launch_bounds__(FLAT_MAX_THREADS) step_flat_kernel(const StepArgs args) {
+    constexpr int Q = 9;
+    const double* __restrict__ src = static_cast<const double*>(args.src);
+    double* __restrict__ dst = static_cast<double*>(args.dst);
+    const uint32_t per = (uint32_t)args.tw / blockDim.x;  // CTAs per entry, a power of two
+    const TileDesc tile = args.tiles[blockIdx.x / per];
+    const InstDesc& in = args.inst[tile.inst];
+    const uint32_t nx = (uint32_t)in.nx, ny = (uint32_t)in.ny;
+    const int bc = in.bc;
+    const uint32_t k = (uint32_t)tile.cx0 + (blockIdx.x & (per - 1u)) * blockDim.x + threadIdx.x;
+    const bool active = k < (uint32_t)tile.y0;
+    uint32_t x, y;
+    bool ring = false;
+    if (bc == BC_CAVITY) {
+        const uint32_t mx = nx - 2u, fluid = mx * (ny - 2u);
+        if (k < fluid) {
+            const uint32_t r = k / mx;
+            y = 1u + r;
+            x = 1u + k - r * mx;
+        } else {
+            // ring: bottom row, top row, then the two sides, row by row
+            const uint32_t j = k - fluid;
+            ring = true;
+            if (j < 2u * nx) {
+                y = j < nx ? 0u : ny - 1u;
+                x = j < nx ? j : j - nx;
+            } else {
+                const uint32_t s = j - 2u * nx;
+                y = 1u + (s >> 1);
+                x = (s & 1u) ? nx - 1u : 0u;
+            }
+        }
+    } else {
+        y = k / nx;
+        x = k - y * nx;
+    }
+    wait_previous_grid();
+    allow_next_grid();
+    if (!active) return;
+
+    const int64_t pitch = in.pitch, plane = in.plane;
+    const double* base = src + in.off;
+    double d[Q];
+    if (args.inplace) {
+        const double* p = base + (int64_t)y * pitch + x;
+#pragma unroll
+        for (int a = 0; a < Q; ++a) d[a] = p[a * plane];
+    } else {
+        // columns x - 1, x + 1 and rows y - 1, y + 1 under the boundary rule;
+        // a cavity node pulls deviation 0 from outside the lattice
+        const bool cav = bc == BC_CAVITY;
+        const bool l = x > 0u, r = x + 1u < nx, b = y > 0u, t = y + 1u < ny;
+        const uint32_t wrap_l = bc == BC_PERIODIC ? nx - 1u : 0u, wrap_r = bc == BC_PERIODIC ? 0u : nx - 1u;
+        const uint32_t xs[3] = {l ? x - 1u : wrap_l, x, r ? x + 1u : wrap_r};
+        const uint32_t ys[3] = {b ? y - 1u : ny - 1u, y, t ? y + 1u : 0u};
+        const bool xok[3] = {l || !cav, true, r || !cav}, yok[3] = {b || !cav, true, t || !cav};
+#pragma unroll
+        for (int a = 0; a < Q; ++a) {
+            const int i = 1 - D2Q9::vx(a), j = 1 - D2Q9::vy(a);
+            d[a] = (xok[i] && yok[j]) ? __ldg(base + a * plane + (int64_t)ys[j] * pitch + xs[i]) : 0.0;
+        }
+    }
+    double o[Q];
+    double* op = dst + in.off + (int64_t)y * pitch + x;
+    if (ring) {
+        const bool lid = y == ny - 1u && x > 0u && x < nx - 1u;
+#pragma unroll
+        for (int a = 0; a < Q; ++a) op[a * plane] = lid ? in.lid_dev[a] : d[D2Q9::opp(a)];
+        return;
+    }
+    const Rates<double> rates{in.omega, in.omega2, in.s_e, in.s_eps};
+    const uint32_t st = Collide<D2Q9, COLL, double, 8>::run(d, args.rho0, rates, o);
+#pragma unroll
+    for (int a = 0; a < Q; ++a) op[a * plane] = o[a];
+    if (st & ST_NEWTON_SKIPPED) atomicAdd(args.status + 2 * tile.inst + 0, 1ull);
+    if (st & ST_UNSTABLE) atomicAdd(args.status + 2 * tile.inst + 1, 1ull);
+}
+
+inline const void* pick_step_flat_kernel(int collision) {
+    switch (collision) {
+        case COLL_MINXENT4: return (const void*)&step_flat_kernel<COLL_MINXENT4>;
+        case COLL_SRT: return (const void*)&step_flat_kernel<COLL_SRT>;
+        case COLL_MINXENT2: return (const void*)&step_flat_kernel<COLL_MINXENT2>;
+        case COLL_MRT:
+        case COLL_TRT: return (const void*)&step_flat_kernel<COLL_MRT>;
+    }
+    return nullptr;
+}
+
 // The __global__ function for (lattice, collision rule) with storage S,
 // arithmetic T and V nodes per thread.  TRT shares the MRT kernel (its rates
 // come from the instance table); on D1Q3 every rule is BGK.

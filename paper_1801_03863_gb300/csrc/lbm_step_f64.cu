@@ -5,6 +5,7 @@
 namespace lbm {
 
 const void* step_kernel_f64(int lattice, int collision, int V) {
+    if (V == 1) return lattice == 2 ? pick_step_flat_kernel(collision) : nullptr;
     if (V == 2) return pick_step_kernel<double, double, 2>(lattice, collision);
     return nullptr;
 }
