@@ -275,9 +275,10 @@ int lbm_conservation_noalloc(lbm_ctx* ctx, double* out);
 int lbm_status(lbm_ctx* ctx, int64_t* counters);
 int lbm_status_instance(lbm_ctx* ctx, int32_t instance, int64_t* counters);
 
-/* Launch shape in use: out[0] = nodes per thread (1: the FP64 D2Q9 kernel
- * with one node per thread, warps of 32 consecutive nodes, tw = 32, th = 1), out[1] = tile width in
- * thread chunks, out[2] = tile height in rows, out[3] = grid size (CTAs),
+/* Launch shape in use: out[0] = nodes per thread (1 on D2Q9: the FP64 kernel
+ * with one node per thread, warps of 32 consecutive nodes, tw = 32, th = 1;
+ * on D1Q3 nodes per lane of the tube kernel, tw x th = threads of a CTA, both
+ * following from the sizes), out[1] = tile width in thread chunks, out[2] = tile height in rows, out[3] = grid size (CTAs),
  * out[4] = kernel kind (0: register-chunk kernel; 1 to 4: the TMA-staged
  * D2Q9 kernel, whose CTAs have one warp that only moves tiles in and out
  * besides the colliding warps.  1: large tiles, 8-warp CTAs, 1792 nodes for

@@ -32,52 +32,30 @@ size_t dtype_bytes(int dt) { return dt == DT_F64 ? 8 : (dt == DT_F32 ? 4 : 2); }
 // tw x th chunks); kind 1 / 2 / 3 / 4: TMA-staged D2Q9 kernel with node
 // pairs (V = 2) in the large-tile / small-tile / wide-CTA / deep-ring
 // geometry (smem_tile_nodes variant kind - 1), tile width per instance.
-// Kind 0 with V = 1 is the FP64 kernel with one node per thread (warps of 32
-// consecutive nodes: tw = 32, th = 1).
+// Kind 0 with V = 1 on D2Q9 is the FP64 kernel with one node per thread
+// (warps of 32 consecutive nodes: tw = 32, th = 1).  On D1Q3 kind 0 is the
+// tube kernel: V nodes per lane, tw x th threads per CTA.
 struct Shape {
     int V, tw, th;
     int kind = 0;
-    bool flat() const { return kind == 0 && V == 1; }
 };
 
-Shape default_shape(int lattice, int storage) {
-    if (lattice == 1) return {storage == DT_F64 ? 2 : 4, 128, 1};
+Shape default_shape_d2q9(int storage) {
     if (storage == DT_F64) return {1, 32, 1};
     if (storage == DT_F32) return {4, 16, 8};
     return {8, 8, 16};
 }
 
-// Launch-shape candidates of the autotuner.  D2Q9 with FP32 arithmetic: the
+// Launch-shape candidates of the autotuner on D2Q9.  FP32 arithmetic: the
 // TMA-staged kernel in its four geometries and the default register-chunk
-// shape (which wins only on small, cache-resident lattices).  D2Q9 in FP64:
-// one node per thread (measured ahead of every register-chunk shape from
-// 800 x 4 to 2048^2 nodes, so nothing is timed).  D1Q3: register-chunk
-// shapes, V = the compiled widths of the storage type, tiles of 128 or 256
-// threads.
-std::vector<Shape> candidate_shapes(int lattice, int storage, int64_t max_nx) {
+// shape (which wins only on small, cache-resident lattices).  FP64: one node
+// per thread (measured ahead of every register-chunk shape from 800 x 4 to
+// 2048^2 nodes, so nothing is timed).
+std::vector<Shape> candidate_shapes(int storage) {
     std::vector<Shape> out;
-    if (lattice == 2 && storage != DT_F64) {
-        out.push_back({2, 0, 0, 1});  // TMA-staged kernel, node pairs, large tiles
-        out.push_back({2, 0, 0, 2});  // TMA-staged kernel, node pairs, small tiles
-        out.push_back({2, 0, 0, 3});  // TMA-staged kernel, node pairs, wide CTAs
-        out.push_back({2, 0, 0, 4});  // TMA-staged kernel, node pairs, deep ring
-        out.push_back(default_shape(lattice, storage));
-        return out;
-    }
-    if (lattice == 2) {
-        out.push_back(default_shape(lattice, storage));
-        return out;
-    }
-    std::vector<int> vs;
-    if (storage == DT_F64) vs = {2};
-    else if (storage == DT_F32) vs = {2, 4};
-    else vs = {4, 8};
-    for (int V : vs) {
-        for (int block : {128, 256}) {
-            if ((int64_t)block * V > 2 * std::max<int64_t>(max_nx, 8) && block > 128) continue;
-            out.push_back({V, block, 1});
-        }
-    }
+    if (storage != DT_F64)
+        for (int kind = 1; kind <= 4; ++kind) out.push_back({2, 0, 0, kind});
+    out.push_back(default_shape_d2q9(storage));
     return out;
 }
 
@@ -209,6 +187,7 @@ struct lbm_ctx {
     int64_t steps = 0;
     Shape shape{};
     int flat_nodes = 0;  // one-node-per-thread kernel: nodes per tile-table entry
+    int halo = 0;        // tube kernel: halo nodes of a segment, steps per launch
     const void* kern = nullptr;
     int grid = 0;
     size_t smem = 0;  // dynamic shared memory of the step kernel
@@ -276,9 +255,59 @@ int flat_nodes(const lbm_ctx* ctx) {
         if (n <= ctx->layout.max_tiles) return e;
     }
 }
+bool is_flat(const lbm_ctx* ctx, const Shape& s) {
+    return ctx->lattice == 2 && s.kind == 0 && s.V == 1;
+}
 int block_threads(const lbm_ctx* ctx, const Shape& s) {
     if (s.kind >= 1) return smem_block_threads(s.kind - 1);
-    return s.flat() ? std::min(ctx->flat_nodes, FLAT_MAX_THREADS) : s.tw * s.th;
+    if (ctx->lattice == 1) return std::max(32, std::min(s.tw * s.th, 256) / 32 * 32);
+    return is_flat(ctx, s) ? std::min(ctx->flat_nodes, FLAT_MAX_THREADS) : s.tw * s.th;
+}
+
+// Tube kernel: nodes per lane V and halo (= steps per launch) of a context,
+// the pair with the least modelled time per step
+//     latency + (ceil(segments / schedulers) - 1) x throughput + launch / halo.
+// A long halo spares launches and memory traffic, which is what single tubes
+// are bound by, and costs redundant nodes, which ensembles are bound by; a
+// small V spreads a short tube over more schedulers.  The constants (us per
+// step of one segment alone on its scheduler / of one segment among many,
+// and per launch) are fits of measurements, V and halo swept over single
+// tubes of 800 to 20000 nodes and ensembles of 200 to 4096 tubes:
+//   800 nodes FP64: V 1, halo 12: 0.76 us a step (V 2, halo 8: 1.45);
+//   800 nodes FP32: V 2, halo 24: 0.19 us (V 4, halo 8: 0.43);
+//   4096 tubes (18.0 M nodes) FP32: V 8, halo 8..16: 21.7 us (V 2: 32.2).
+// V_pinned != 0 (LBM_SHAPE) fixes V.
+void tube_plan(const lbm_ctx* ctx, int V_pinned, int* V, int* halo) {
+    struct Cost {
+        int V;
+        double latency, throughput;
+    };
+    static const Cost f64[] = {{1, 0.62, 0.50}, {2, 1.22, 1.0}, {4, 2.4, 2.0}};
+    static const Cost f32[] = {{2, 0.12, 0.045}, {4, 0.17, 0.079}, {8, 0.31, 0.151}};
+    static const Cost b16[] = {{4, 0.20, 0.090}, {8, 0.36, 0.175}};
+    const Cost* costs = ctx->storage == DT_F64 ? f64 : ctx->storage == DT_F32 ? f32 : b16;
+    const int n = ctx->storage == DT_F64 || ctx->storage == DT_F32 ? 3 : 2;
+    const double copy_us = 6.0 * dtype_bytes(ctx->storage) * ctx->layout.total_nodes / 6.8e6;
+    double best = 1e30;
+    *V = V_pinned;
+    *halo = std::max(V_pinned, 8);
+    for (int c = 0; c < n; ++c) {
+        if (V_pinned && costs[c].V != V_pinned) continue;
+        const int v = costs[c].V;
+        for (int h = std::max(v, 4); h <= 48 && 32 * v - 2 * h >= 8; h += v) {
+            const int64_t u = 32 * v - 2 * h;
+            int64_t segs = 0;
+            for (const InstDesc& in : ctx->layout.inst) segs += (in.nx + u - 1) / u;
+            const double rounds = std::ceil((double)segs / (4.0 * ctx->num_sms));
+            const double t = costs[c].latency + (rounds - 1.0) * costs[c].throughput +
+                             (1.7 + 0.27 * copy_us) / h;
+            if (t < best) {
+                best = t;
+                *V = v;
+                *halo = h;
+            }
+        }
+    }
 }
 
 std::vector<TileDesc> build_tiles(const lbm_ctx* ctx, const Shape& s) {
@@ -296,7 +325,13 @@ std::vector<TileDesc> build_tiles(const lbm_ctx* ctx, const Shape& s) {
         }
         return t;
     }
-    if (s.flat()) {
+    if (ctx->lattice == 1) {
+        const int u = 32 * s.V - 2 * ctx->halo;
+        for (int i = 0; i < ctx->count; ++i)
+            for (int32_t x = 0; x < ctx->layout.inst[i].nx; x += u) t.push_back({(int32_t)i, x, 0, 0});
+        return t;
+    }
+    if (is_flat(ctx, s)) {
         // flat_nodes consecutive nodes per entry: the fluid nodes of every
         // instance, then the rings of the cavities
         for (int part = 0; part < 2; ++part)
@@ -343,11 +378,11 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
         const int rc = build_tensor_maps(ctx, var);
         if (rc != LBM_OK) return rc;
     } else {
-        if (s.flat() && (s.tw != 32 || s.th != 1)) return LBM_ERR_ARG;
+        if (is_flat(ctx, s) && (s.tw != 32 || s.th != 1)) return LBM_ERR_ARG;
         k = find_step_kernel(ctx->lattice, ctx->storage, ctx->collision, s.V);
     }
     if (!k) return LBM_ERR_ARG;
-    if (s.flat()) ctx->flat_nodes = flat_nodes(ctx);
+    if (is_flat(ctx, s)) ctx->flat_nodes = flat_nodes(ctx);
     std::vector<TileDesc> t = build_tiles(ctx, s);
     if ((int64_t)t.size() > ctx->layout.max_tiles) return LBM_ERR_ARG;
     LBM_CK(cudaMemcpyAsync(ctx->d_tiles, t.data(), sizeof(TileDesc) * t.size(),
@@ -359,8 +394,9 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
     int per_sm = 0;
     LBM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
     per_sm = std::max(per_sm, 1);
-    const int64_t g = s.flat() ? (int64_t)t.size() * (ctx->flat_nodes / block)
-                               : std::min<int64_t>((int64_t)per_sm * ctx->num_sms, (int64_t)t.size());
+    const int64_t g = ctx->lattice == 1 ? ((int64_t)t.size() * 32 + block - 1) / block
+                      : is_flat(ctx, s) ? (int64_t)t.size() * (ctx->flat_nodes / block)
+                                        : std::min<int64_t>((int64_t)per_sm * ctx->num_sms, (int64_t)t.size());
     ctx->tiles.swap(t);
     ctx->shape = s;
     ctx->kern = k;
@@ -433,7 +469,7 @@ StepArgs step_args(const lbm_ctx* ctx, int src) {
     a.inst = ctx->d_inst;
     a.tiles = ctx->d_tiles;
     a.ntiles = (int32_t)ctx->tiles.size();
-    a.tw = ctx->shape.flat() ? ctx->flat_nodes : ctx->shape.tw;
+    a.tw = is_flat(ctx, ctx->shape) ? ctx->flat_nodes : ctx->shape.tw;
     a.tw_log2 = ctx->shape.tw > 0 ? ilog2(ctx->shape.tw) : 0;
     a.th = ctx->shape.th;
     a.rho0 = ctx->rho0;
@@ -445,15 +481,20 @@ StepArgs step_args(const lbm_ctx* ctx, int src) {
     a.spin_limit = ctx->spin_limit;
     a.lost_tile = ctx->lost_tile;
     a.inplace = 0;
+    a.steps = 1;
+    a.halo = ctx->halo;
     return a;
 }
 
 // One step launch.  It is a programmatic dependent launch: the kernel may be
 // scheduled while the previous kernel in the stream drains, and waits for its
 // completion (griddepcontrol.wait) before touching device state.
-cudaError_t launch_step(lbm_ctx* ctx, int src, cudaStream_t s, bool inplace = false) {
+// inplace: the (first) step collides without streaming (one-node-per-thread
+// and tube kernels only); steps: time steps of the launch (tube kernel only).
+cudaError_t launch_step(lbm_ctx* ctx, int src, cudaStream_t s, bool inplace = false, int steps = 1) {
     StepArgs a = step_args(ctx, src);
-    a.inplace = inplace ? 1 : 0;  // one-node-per-thread kernel only
+    a.inplace = inplace ? 1 : 0;
+    a.steps = steps;
     void* params[] = {&a};
     const int block = block_threads(ctx, ctx->shape);
     cudaLaunchAttribute attr[1];
@@ -600,12 +641,12 @@ int autotune(lbm_ctx* ctx) {
     const std::string key = tune_key(ctx);
     Shape cached;
     if (tune_lookup(key, &cached) && apply_shape(ctx, cached) == LBM_OK) return LBM_OK;
-    std::vector<Shape> cands = candidate_shapes(ctx->lattice, ctx->storage, ctx->layout.max_nx);
+    std::vector<Shape> cands = candidate_shapes(ctx->storage);
     if (cands.size() == 1) return apply_shape(ctx, cands[0]);
     cudaEvent_t ev[6];
     for (int i = 0; i < 6; ++i) LBM_CK(cudaEventCreate(&ev[i]));
     float best = 1e30f;
-    Shape best_s = default_shape(ctx->lattice, ctx->storage);
+    Shape best_s = default_shape_d2q9(ctx->storage);
     int rc = LBM_OK;
     std::vector<float> t(cands.size(), -1.f);
     for (size_t c = 0; c < cands.size(); ++c) {
@@ -988,11 +1029,18 @@ int lbm_create_batch(lbm_ctx** out, lbm_lattice lat, int32_t count, const int64_
             return fail(LBM_ERR_CUDA);
     }
     Shape s;
-    if (parse_shape_env(&s)) rc = apply_shape(ctx, s);
+    if (lat == 1) {
+        // nothing to time: the plan follows from the sizes (LBM_SHAPE pins V
+        // and the CTA size)
+        int V = 0;
+        const bool pinned = parse_shape_env(&s);
+        tube_plan(ctx, pinned ? s.V : 0, &V, &ctx->halo);
+        rc = apply_shape(ctx, pinned ? s : Shape{V, 128, 1});
+    } else if (parse_shape_env(&s)) rc = apply_shape(ctx, s);
     else if (o.autotune && !getenv("LBM_NO_AUTOTUNE")) rc = autotune(ctx);
-    else rc = apply_shape(ctx, default_shape(lat, o.storage));
+    else rc = apply_shape(ctx, default_shape_d2q9(o.storage));
     if (rc != LBM_OK) return fail(rc);
-    rc = capture_graphs(ctx);
+    if (lat == 2) rc = capture_graphs(ctx);  // the tube kernel takes several steps per launch
     if (rc != LBM_OK) return fail(rc);
     *out = ctx;
     return LBM_OK;
@@ -1062,8 +1110,19 @@ int lbm_step(lbm_ctx* ctx, int64_t n) {
     if (ctx->failed) return LBM_ERR_CUDA;
     if (!ctx->initialized) return LBM_ERR_STATE;
     if (n == 0) return LBM_OK;
+    if (ctx->lattice == 1) {
+        while (n > 0) {
+            const int k = (int)std::min<int64_t>(n, ctx->halo);
+            LBM_CK(launch_step(ctx, ctx->cur, ctx->stream, !ctx->post, k));
+            ctx->cur = 1 - ctx->cur;
+            ctx->post = true;
+            ctx->steps += k;
+            n -= k;
+        }
+        return LBM_OK;
+    }
     if (!ctx->post) {
-        if (ctx->shape.flat()) {
+        if (is_flat(ctx, ctx->shape)) {
             LBM_CK(launch_step(ctx, ctx->cur, ctx->stream, true));
         } else {
             AuxArgs a = aux_args(ctx);

@@ -448,11 +448,11 @@ cudaError_t collide_inplace_dispatch(const AuxArgs& a, const void* src, void* ds
     return cudaGetLastError();
 }
 
-// TRT shares the MRT kernel; on D1Q3 every rule is BGK.
+// TRT shares the MRT kernel.  D1Q3 collides in its step kernel.
 template <class Lat, typename S, typename T>
 cudaError_t collide_inplace_by_rule(const AuxArgs& a, const void* src, void* dst) {
     if constexpr (Lat::Q == 3) {
-        return collide_inplace_dispatch<Lat, S, T, COLL_MINXENT4>(a, src, dst);
+        return cudaErrorInvalidValue;
     } else {
         switch (a.collision) {
             case COLL_MINXENT4: return collide_inplace_dispatch<Lat, S, T, COLL_MINXENT4>(a, src, dst);

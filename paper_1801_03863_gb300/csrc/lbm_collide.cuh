@@ -603,8 +603,8 @@ __device__ __forceinline__ uint32_t mrt_d2q9(const T (&d)[9], T rho0, const Rate
 // constraints, so both rules reduce to f + omega (f^eq - f).
 // ---------------------------------------------------------------------------
 template <typename T>
-__device__ __forceinline__ uint32_t bgk_d1q3(const T (&d)[3], T rho0, const Rates<T>& r,
-                                             T (&out)[3]) {
+__device__ __forceinline__ uint32_t bgk_d1q3_f32(const T (&d)[3], T rho0, const Rates<T>& r,
+                                                 T (&out)[3]) {
     using N = Num<T>;
     const T omega = r.omega;
     constexpr double W[3] = {2.0 / 3.0, 1.0 / 6.0, 1.0 / 6.0};
@@ -626,6 +626,30 @@ __device__ __forceinline__ uint32_t bgk_d1q3(const T (&d)[3], T rho0, const Rate
     if constexpr (N::LANES == 1) all = true;
     else all = {true, true};
     return lane_status<T>(all, finite_nonneg<T, 3>(out, W, rho0));
+}
+
+template <typename T>
+__device__ __forceinline__ uint32_t bgk_d1q3(const T (&d)[3], T rho0, const Rates<T>& r,
+                                             T (&out)[3]) {
+    using N = Num<T>;
+    if constexpr (std::is_same<T, double>::value) {
+        // f^eq_1 - f_1 = f^eq_2 - f_2 = X / 2 and f^eq_0 - f_0 = -X with
+        // X = j u + drho / 3 - (d_1 + d_2) (the rule moves one moment and
+        // conserves the others): 13 FP64 instructions with the reciprocal
+        // instead of 26 (FP64 issue bounds this path; the FP32 paths keep
+        // the form below, whose rounding their results are pinned to)
+        constexpr double W[3] = {2.0 / 3.0, 1.0 / 6.0, 1.0 / 6.0};
+        const double n = d[1] + d[2], drho = d[0] + n, j = d[1] - d[2];
+        const double u = j * N::rcp(rho0 + drho);
+        const double X = fma(j, u, fma(1.0 / 3.0, drho, -n));
+        const double h = 0.5 * r.omega;
+        out[0] = fma(-r.omega, X, d[0]);
+        out[1] = fma(h, X, d[1]);
+        out[2] = fma(h, X, d[2]);
+        return finite_nonneg_f64<3>(out, W, rho0) ? 0u : ST_UNSTABLE;
+    } else {
+        return bgk_d1q3_f32<T>(d, rho0, r, out);
+    }
 }
 
 // Dispatch by lattice, rule, number type and storage bytes SB (the MinxEnt

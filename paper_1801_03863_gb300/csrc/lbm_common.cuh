@@ -108,7 +108,7 @@ static_assert(sizeof(InstDesc) % 16 == 0, "bulk copies move multiples of 16 byte
 
 struct TileDesc {
     int32_t inst;  // instance index
-    int32_t cx0;   // first thread chunk (units of V nodes) in x, node in x (TMA kernel), or
+    int32_t cx0;   // first thread chunk (units of V nodes) in x, node in x (TMA and tube kernels), or
                    // first node in row-major order (one-node-per-thread kernel)
     int32_t y0;    // first row (one-node-per-thread kernel: end of the node range)
     int32_t pad;
@@ -138,7 +138,9 @@ struct StepArgs {
     unsigned int* error;         // device error word (bounded waits that ran out)
     int32_t spin_limit;          // polls of one bounded mbarrier wait (TMA kernel)
     int32_t lost_tile;           // test hook: tile whose copies are never issued (-1: none)
-    int32_t inplace;             // FP64 one-node-per-thread kernel: collide without streaming
+    int32_t inplace;             // collide without streaming (tube kernel: the first step)
+    int32_t steps;               // tube kernel: time steps of this launch, at most halo
+    int32_t halo;                // tube kernel: nodes carried along at either end of a segment
 };
 
 // Most threads of a CTA of the one-node-per-thread kernel.

@@ -428,12 +428,160 @@ inline const void* pick_step_flat_kernel(int collision) {
     return nullptr;
 }
 
-// The __global__ function for (lattice, collision rule) with storage S,
-// arithmetic T and V nodes per thread.  TRT shares the MRT kernel (its rates
-// come from the instance table); on D1Q3 every rule is BGK.
+// ---------------------------------------------------------------------------
+// D1Q3: several time steps per launch, one warp per segment of a tube.
+//
+// A warp holds 32 V consecutive nodes in registers (V per lane) and advances
+// them args.steps <= args.halo steps: streaming is a register shift within a
+// lane and one shuffle per moving plane between lanes, so a step needs no
+// memory and no barrier.  Each step the outermost node on either side of the
+// segment loses its neighbour, so the outer `halo` nodes are carried along
+// only to feed the inner ones and the segment's 32 V - 2 halo inner nodes
+// are written back.  One step per launch moved 24 bytes a node and step (FP32)
+// and was bound by HBM on ensembles and by the launch on single tubes; with a
+// halo of 8 steps the traffic falls to 3 bytes and the arithmetic bounds it.
+//
+// Node i of a lane sits in half i / NP of pair i % NP (NP = V / 2 pairs), so
+// that shifting by one node is taking the neighbouring pair, and only the
+// end pairs are put together from two registers.
+//
+// Tube ends: a periodic segment loads its nodes modulo nx; at a zero-gradient
+// end the entering population is the end node's own (the nodes beyond are
+// never read by the lattice).  Each node's arithmetic is that of one step per
+// launch, rounding to the storage type included.
+// ---------------------------------------------------------------------------
+template <typename CT, typename S> __device__ __forceinline__ CT round_to_storage(CT v) {
+    if constexpr (std::is_same<S, double>::value || std::is_same<S, float>::value) {
+        return v;
+    } else {
+        using N = Num<CT>;
+#pragma unroll
+        for (int l = 0; l < N::LANES; ++l)
+            N::set_lane(v, l, Store<S>::to_f32(Store<S>::from(N::lane(v, l))));
+        return v;
+    }
+}
+
 template <typename S, typename T, int V>
-const void* pick_step_kernel(int lattice, int collision) {
-    if (lattice == 1) return (const void*)&step_kernel<D1Q3, S, T, V, COLL_MINXENT4>;
+__global__ void __launch_bounds__(256) step_tube_kernel(const StepArgs args) {
+    using CT = typename std::conditional<std::is_same<T, float>::value, F2, T>::type;
+    using N = Num<CT>;
+    using LT = typename LaneOf<CT>::type;
+    constexpr int P = N::LANES, NP = V / P;
+    static_assert(V % P == 0, "whole pairs per lane");
+    const int t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+    const int lane = (int)(threadIdx.x & 31u);
+    const bool some = t < args.ntiles;  // the same for the whole warp
+    const TileDesc tile = args.tiles[some ? t : 0];
+    const InstDesc& in = args.inst[tile.inst];
+    const int nx = in.nx, halo = args.halo;
+    const bool periodic = in.bc == BC_PERIODIC;
+    const int x = tile.cx0 - halo + lane * V;  // first node of this lane
+    const Rates<CT> rates{CT((LT)in.omega), CT((LT)in.omega2), CT((LT)in.s_e), CT((LT)in.s_eps)};
+    const CT rho0 = CT((LT)args.rho0);
+    wait_previous_grid();
+    allow_next_grid();
+    if (!some) return;
+
+    // populations of node p + l NP: lane l of f[a][p]
+    CT f[3][NP];
+    const S* src = static_cast<const S*>(args.src) + in.off;
+    const bool whole = x >= 0 && x + V <= nx;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        Chunk<S, V> c;
+        if (whole) {
+            c.load(src + a * in.plane + x);
+        } else {
+            c.zero();
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                int xi = x + i;
+                if (periodic) {
+                    xi %= nx;
+                    if (xi < 0) xi += nx;
+                }
+                if (xi >= 0 && xi < nx) c.set(i, ldg_elem<S>(src + a * in.plane + xi));
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < NP; ++p)
+#pragma unroll
+            for (int l = 0; l < P; ++l) N::set_lane(f[a][p], l, to_compute<T, S>(c.get(p + l * NP)));
+    }
+
+    const bool mine = lane * V >= halo && lane * V < 32 * V - halo;  // lanes written back
+    const bool left_end = !periodic && x == 0;  // x = 0 is the first node of its lane
+    // warp-uniform: the segment holds the last node of a zero-gradient tube
+    const bool has_right = !periodic && tile.cx0 - halo < nx && tile.cx0 - halo + 32 * V >= nx;
+    uint32_t n_unst = 0;
+    for (int s = 0; s < args.steps; ++s) {
+        CT from_l[NP], from_r[NP];  // plane 1 pulled from x - 1, plane 2 from x + 1
+        if (s > 0 || !args.inplace) {
+            const LT in_l = __shfl_up_sync(0xffffffffu, N::lane(f[1][NP - 1], P - 1), 1);
+            const LT in_r = __shfl_down_sync(0xffffffffu, N::lane(f[2][0], 0), 1);
+#pragma unroll
+            for (int p = 1; p < NP; ++p) from_l[p] = f[1][p - 1];
+#pragma unroll
+            for (int p = 0; p < NP - 1; ++p) from_r[p] = f[2][p + 1];
+            N::set_lane(from_l[0], 0, left_end ? N::lane(f[1][0], 0) : in_l);
+            if constexpr (P == 2) N::set_lane(from_l[0], 1, N::lane(f[1][NP - 1], 0));
+            if constexpr (P == 2) N::set_lane(from_r[NP - 1], 0, N::lane(f[2][0], 1));
+            N::set_lane(from_r[NP - 1], P - 1, in_r);
+            if (has_right) {
+#pragma unroll
+                for (int p = 0; p < NP; ++p)
+#pragma unroll
+                    for (int l = 0; l < P; ++l)
+                        if (x + p + l * NP == nx - 1) N::set_lane(from_r[p], l, N::lane(f[2][p], l));
+            }
+        } else {
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                from_l[p] = f[1][p];
+                from_r[p] = f[2][p];
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < NP; ++p) {
+            const CT d[3] = {f[0][p], from_l[p], from_r[p]};
+            CT o[3];
+            const uint32_t st = Collide<D1Q3, COLL_MINXENT4, CT, (int)sizeof(S)>::run(d, rho0, rates, o);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) f[a][p] = round_to_storage<CT, S>(o[a]);
+            if (st && mine) {  // rare: a population is negative or not finite
+#pragma unroll
+                for (int l = 0; l < P; ++l)
+                    if (x + p + l * NP < nx) n_unst += ((st >> (2 * l)) & ST_UNSTABLE) >> 1;
+            }
+        }
+    }
+
+    if (!mine || x >= nx) return;
+    S* dst = static_cast<S*>(args.dst) + in.off + x;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        Chunk<S, V> c;
+        c.zero();
+#pragma unroll
+        for (int p = 0; p < NP; ++p)
+#pragma unroll
+            for (int l = 0; l < P; ++l) c.set(p + l * NP, Store<S>::from(N::lane(f[a][p], l)));
+        if (whole) {
+            c.store(dst + a * in.plane);
+        } else {
+#pragma unroll
+            for (int i = 0; i < V; ++i)
+                if (x + i < nx) dst[a * in.plane + i] = c.get(i);
+        }
+    }
+    if (n_unst) atomicAdd(args.status + 2 * tile.inst + 1, (unsigned long long)n_unst);
+}
+
+// The D2Q9 register-chunk kernel for a collision rule with storage S,
+// arithmetic T and V nodes per thread.  TRT shares the MRT kernel (its rates
+// come from the instance table).
+template <typename S, typename T, int V> const void* pick_step_kernel(int collision) {
     switch (collision) {
         case COLL_MINXENT4: return (const void*)&step_kernel<D2Q9, S, T, V, COLL_MINXENT4>;
         case COLL_SRT: return (const void*)&step_kernel<D2Q9, S, T, V, COLL_SRT>;

@@ -6,8 +6,13 @@
 namespace lbm {
 
 const void* step_kernel_bf16(int lattice, int collision, int V) {
-    if (V == 4) return pick_step_kernel<__nv_bfloat16, float, 4>(lattice, collision);
-    if (V == 8) return pick_step_kernel<__nv_bfloat16, float, 8>(lattice, collision);
+    if (lattice == 1) {
+        if (V == 4) return (const void*)&step_tube_kernel<__nv_bfloat16, float, 4>;
+        if (V == 8) return (const void*)&step_tube_kernel<__nv_bfloat16, float, 8>;
+        return nullptr;
+    }
+    if (V == 4) return pick_step_kernel<__nv_bfloat16, float, 4>(collision);
+    if (V == 8) return pick_step_kernel<__nv_bfloat16, float, 8>(collision);
     return nullptr;
 }
 

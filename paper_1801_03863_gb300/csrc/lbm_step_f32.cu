@@ -6,8 +6,14 @@
 namespace lbm {
 
 const void* step_kernel_f32(int lattice, int collision, int V) {
-    if (V == 2) return pick_step_kernel<float, float, 2>(lattice, collision);
-    if (V == 4) return pick_step_kernel<float, float, 4>(lattice, collision);
+    if (lattice == 1) {
+        if (V == 2) return (const void*)&step_tube_kernel<float, float, 2>;
+        if (V == 4) return (const void*)&step_tube_kernel<float, float, 4>;
+        if (V == 8) return (const void*)&step_tube_kernel<float, float, 8>;
+        return nullptr;
+    }
+    if (V == 2) return pick_step_kernel<float, float, 2>(collision);
+    if (V == 4) return pick_step_kernel<float, float, 4>(collision);
     return nullptr;
 }
 

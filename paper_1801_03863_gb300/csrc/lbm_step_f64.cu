@@ -5,8 +5,14 @@
 namespace lbm {
 
 const void* step_kernel_f64(int lattice, int collision, int V) {
-    if (V == 1) return lattice == 2 ? pick_step_flat_kernel(collision) : nullptr;
-    if (V == 2) return pick_step_kernel<double, double, 2>(lattice, collision);
+    if (lattice == 1) {
+        if (V == 1) return (const void*)&step_tube_kernel<double, double, 1>;
+        if (V == 2) return (const void*)&step_tube_kernel<double, double, 2>;
+        if (V == 4) return (const void*)&step_tube_kernel<double, double, 4>;
+        return nullptr;
+    }
+    if (V == 1) return pick_step_flat_kernel(collision);
+    if (V == 2) return pick_step_kernel<double, double, 2>(collision);
     return nullptr;
 }
 
