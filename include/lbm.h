@@ -206,7 +206,7 @@ int lbm_moments_batch_device(lbm_ctx* ctx, int32_t instance, double* rho, double
 int lbm_stream_function(lbm_ctx* ctx, double* psi);
 
 /* lbm_stream_function into a DEVICE FP64 array, ordered on the stream, no
- * sync and no status check (uses the context's staging area for u). */
+ * sync and no status check. */
 int lbm_stream_function_device(lbm_ctx* ctx, double* psi);
 
 /* lbm_stream_function of ONE instance (Sec. IV.I) into a host FP64 array

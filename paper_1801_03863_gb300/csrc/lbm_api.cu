@@ -229,6 +229,8 @@ AuxArgs aux_args(const lbm_ctx* ctx) {
     a.collision = ctx->collision;
     a.count = ctx->count;
     a.max_nodes = ctx->layout.max_nodes;
+    a.max_ny = ctx->layout.max_ny;
+    a.total_nodes = ctx->layout.total_nodes;
     a.inst = ctx->d_inst;
     a.rho0 = ctx->rho0;
     a.pulled = ctx->post;
@@ -813,7 +815,8 @@ AuxArgs aux_args_instance(const lbm_ctx* ctx, int i) {
     const InstDesc& in = ctx->layout.inst[i];
     a.inst = ctx->d_inst + i;
     a.count = 1;
-    a.max_nodes = (int64_t)in.nx * in.ny;
+    a.max_nodes = a.total_nodes = (int64_t)in.nx * in.ny;
+    a.max_ny = in.ny;
     a.node_base = in.node0;
     return a;
 }
@@ -1167,20 +1170,16 @@ int lbm_stream_function_device(lbm_ctx* ctx, double* psi) {
     if (ctx->Q != 9) return LBM_ERR_ARG;
     if (ctx->failed) return LBM_ERR_CUDA;
     if (!ctx->initialized) return LBM_ERR_STATE;
-    const size_t n = (size_t)ctx->layout.total_nodes;
     AuxArgs a = aux_args(ctx);
-    // u_y of f(t_n) into the staging area (rho and u_x beside it), then the
-    // row integrals
-    LBM_CK(run_aux(AuxOp::Moments, a, ctx->buf[ctx->cur], nullptr, nullptr, nullptr, nullptr,
-                   ctx->d_stage, ctx->d_stage + n, ctx->d_stage + 2 * n));
-    LBM_CK(stream_function(a, ctx->layout.max_ny, ctx->d_stage + 2 * n, psi));
+    LBM_CK(run_aux(AuxOp::StreamFunction, a, ctx->buf[ctx->cur], nullptr, nullptr, nullptr, nullptr, psi,
+                   nullptr, nullptr));
     return LBM_OK;
 }
 
 int lbm_stream_function(lbm_ctx* ctx, double* psi) {
     if (!ctx || !psi) return LBM_ERR_ARG;
     const size_t n = (size_t)ctx->layout.total_nodes;
-    double* dpsi = ctx->d_stage + 3 * n;
+    double* dpsi = ctx->d_stage;
     int rc = lbm_stream_function_device(ctx, dpsi);
     if (rc != LBM_OK) return rc;
     LBM_CK(cudaMemcpyAsync(psi, dpsi, n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
@@ -1370,11 +1369,9 @@ int lbm_stream_function_batch(lbm_ctx* ctx, int32_t instance, double* psi) {
     const InstDesc& in = ctx->layout.inst[instance];
     const size_t n = (size_t)in.nx * in.ny;
     AuxArgs a = aux_args_instance(ctx, instance);
-    LBM_CK(run_aux(AuxOp::Moments, a, ctx->buf[ctx->cur], nullptr, nullptr, nullptr, nullptr,
-                   ctx->d_stage, ctx->d_stage + n, ctx->d_stage + 2 * n));
-    LBM_CK(stream_function(a, in.ny, ctx->d_stage + 2 * n, ctx->d_stage + 3 * n));
-    LBM_CK(cudaMemcpyAsync(psi, ctx->d_stage + 3 * n, n * sizeof(double), cudaMemcpyDeviceToHost,
-                           ctx->stream));
+    LBM_CK(run_aux(AuxOp::StreamFunction, a, ctx->buf[ctx->cur], nullptr, nullptr, nullptr, nullptr,
+                   ctx->d_stage, nullptr, nullptr));
+    LBM_CK(cudaMemcpyAsync(psi, ctx->d_stage, n * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
     LBM_CK(cudaStreamSynchronize(ctx->stream));
     return instance_status(ctx, instance);
 }

@@ -1,8 +1,19 @@
 // lbm_aux.cu -- the kernels around the time step: initial equilibrium,
 // the first (in-place) collision after a state is loaded, moments and
-// population read-out, population load, and the FP64 conservation
-// reduction.  One thread per node, grid = (blocks, instance); none of these
-// is on the per-step hot path.
+// population read-out, population load, the stream function and the FP64
+// conservation reduction.
+//
+// Their results are FP64 and GB300's FP64 pipe issues one warp instruction
+// per scheduler in 64 cycles, so FP64 instructions, not bytes, bound what is
+// written plainly: moments of 33 M nodes took 2.26 ms where their 42 bytes a
+// node take 0.21 ms.  Conversions between FP64 and the storage types are
+// done on the integer pipe (exactly), sums of FP16 values exactly in FP32 or
+// integers, and 1 / rho by three FP64 instructions.
+//
+// One thread per node; a block takes `per` consecutive nodes of one instance
+// (grid = (blocks of the largest instance, instance)).
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "lbm_aux.h"
@@ -13,98 +24,247 @@ namespace {
 
 constexpr int AUX_THREADS = 256;
 
+// ---------------------------------------------------------------------------
+// Conversions without the FP64 pipe.  Zeros and normal numbers are converted
+// by their bits; what is left (FP32 subnormals and overflow, infinities, NaN)
+// goes through the conversion instruction.
+// ---------------------------------------------------------------------------
+__device__ __noinline__ double widen_slow(float v) { return (double)v; }
+__device__ __noinline__ float narrow_slow(double v) { return (float)v; }
+__device__ __noinline__ __half half_slow(double v) { return __double2half(v); }
+__device__ __noinline__ __nv_bfloat16 bf16_slow(double v) { return __double2bfloat16(v); }
+
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u)  // normal
+        return __hiloint2double((int)((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(b << 29));
+    if (m == 0u) return __hiloint2double((int)b, 0);
+    return widen_slow(v);
+}
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(__half v) { return widen(__half2float(v)); }
+__device__ __forceinline__ double widen(__nv_bfloat16 v) { return widen(__bfloat162float(v)); }
+
+// |v| of a double in FP32's normal range, as FP32 bits with `up` added below
+// the kept bits first (rounding), or -1 outside the range
+__device__ __forceinline__ bool in_f32_range(uint32_t hi) {
+    return ((hi >> 20) & 0x7ffu) - 897u < 1150u - 897u;
+}
+// FP32 nearest to v, ties to even
+__device__ __forceinline__ float narrow(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    if (in_f32_range(hi)) {
+        const uint64_t u = ((uint64_t)(hi & 0x7fffffffu) << 32) | lo;
+        const uint64_t r = u + 0x0fffffffull + ((u >> 29) & 1ull);
+        return __uint_as_float((hi & 0x80000000u) | ((uint32_t)(r >> 29) - 0x38000000u * 8u));
+    }
+    if (((hi & 0x7fffffffu) | lo) == 0u) return __uint_as_float(hi);
+    return narrow_slow(v);
+}
+// v to FP32 rounded to odd (truncated, with a sticky last bit), so that a
+// second rounding to 16 bits rounds as once
+__device__ __forceinline__ float narrow_odd(uint32_t hi, uint32_t lo) {
+    const uint32_t m = (hi << 3) | (lo >> 29);  // the low 32 bits of |v| >> 29
+    const uint32_t bits = (m - 0xc0000000u) & 0x7fffffffu;
+    return __uint_as_float((hi & 0x80000000u) | bits | ((lo & 0x1fffffffu) != 0u ? 1u : 0u));
+}
+template <typename S> __device__ __forceinline__ S to_storage(double v);
+template <> __device__ __forceinline__ double to_storage<double>(double v) { return v; }
+template <> __device__ __forceinline__ float to_storage<float>(double v) { return narrow(v); }
+template <> __device__ __forceinline__ __half to_storage<__half>(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    if (in_f32_range(hi)) return __float2half_rn(narrow_odd(hi, lo));
+    if (((hi >> 20) & 0x7ffu) < 897u) return __ushort_as_half((unsigned short)((hi >> 16) & 0x8000u));
+    return half_slow(v);
+}
+template <> __device__ __forceinline__ __nv_bfloat16 to_storage<__nv_bfloat16>(double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
+    if (in_f32_range(hi)) return __float2bfloat16_rn(narrow_odd(hi, lo));
+    if (((hi & 0x7fffffffu) | lo) == 0u) return __ushort_as_bfloat16((unsigned short)(hi >> 16));
+    return bf16_slow(v);
+}
+
+// ---------------------------------------------------------------------------
+// Populations of one node.
+// ---------------------------------------------------------------------------
 template <class Lat, typename S>
 __device__ __forceinline__ const S* elem_ptr(const S* base, const InstDesc& in, int a, int x, int y) {
     return base + in.off + (int64_t)a * in.plane + (int64_t)y * in.pitch + x;
 }
 
-// Deviations of f(x, t_n) at one node, FP64.  pulled = true: the stored field
-// is post-collision and the node pulls f_a from x - v_a with the boundary
-// rules of the step; pulled = false: the stored field is f(x, t_n) itself.
+template <typename S> __device__ __forceinline__ S zero_value() { return S(0.0f); }
+
+// Stored deviations of f(x, t_n) at one node.  pulled = true: the stored
+// field is post-collision and the node pulls f_a from x - v_a with the
+// boundary rules of the step; pulled = false: the stored field is f(x, t_n).
 template <class Lat, typename S>
-__device__ void node_state(const S* base, const InstDesc& in, int x, int y, bool pulled,
-                           double (&d)[Lat::Q]) {
+__device__ __forceinline__ void node_state(const S* src, const InstDesc& in, int x, int y, bool pulled,
+                                           S (&d)[Lat::Q]) {
+    if (!pulled) {
+#pragma unroll
+        for (int a = 0; a < Lat::Q; ++a) d[a] = *elem_ptr<Lat, S>(src, in, a, x, y);
+        return;
+    }
+    const bool cav = in.bc == BC_CAVITY, per = in.bc == BC_PERIODIC;
+    const int nx = in.nx, ny = in.ny;
+    const bool l = x > 0, r = x + 1 < nx, b = y > 0, t = y + 1 < ny;
+    const int xs[3] = {l ? x - 1 : (per ? nx - 1 : 0), x, r ? x + 1 : (per ? 0 : nx - 1)};
+    const int ys[3] = {b ? y - 1 : ny - 1, y, t ? y + 1 : 0};
+    const bool xok[3] = {l || !cav, true, r || !cav}, yok[3] = {b || !cav, true, t || !cav};
 #pragma unroll
     for (int a = 0; a < Lat::Q; ++a) {
-        int sx = x, sy = y;
-        bool inside = true;
-        if (pulled) {
-            sx = x - Lat::vx(a);
-            sy = y - Lat::vy(a);
-            if (in.bc == BC_CAVITY) {
-                inside = sx >= 0 && sx < in.nx && sy >= 0 && sy < in.ny;
-            } else {
-                if (in.bc == BC_PERIODIC) sx = (sx + in.nx) % in.nx;
-                else sx = sx < 0 ? 0 : (sx >= in.nx ? in.nx - 1 : sx);
-                sy = (sy + in.ny) % in.ny;
-            }
-        }
-        d[a] = inside ? Store<S>::to_f64(*elem_ptr<Lat, S>(base, in, a, sx, sy)) : 0.0;
+        const int i = 1 - Lat::vx(a), j = 1 - Lat::vy(a);
+        d[a] = (xok[i] && yok[j]) ? *elem_ptr<Lat, S>(src, in, a, xs[i], ys[j]) : zero_value<S>();
     }
 }
 
-// f^eq(rho, u) - W rho0 in FP64 (Eq. numerical-plyeqm):
-//   W_a (rho - rho0) + W_a rho (3 v.u + 9/2 (v.u)^2 - 3/2 u^2),
-// with the even and odd parts in v shared by opposite velocities.
-template <class Lat>
-__device__ void eq_dev(double rho, double ux, double uy, double rho0, double (&d)[Lat::Q]) {
-    const double dr = rho - rho0;
-    const double b0 = -1.5 * (ux * ux + uy * uy);
+// sum d, sum d v_x, sum d v_y in the number type V (float or double)
+template <class Lat, typename V>
+__device__ __forceinline__ void moment_sums(const V (&d)[Lat::Q], V& m, V& jx, V& jy) {
+    if constexpr (Lat::Q == 9) {
+        const V a57 = d[5] - d[7], a86 = d[8] - d[6];
+        m = (d[0] + ((d[1] + d[3]) + (d[2] + d[4]))) + ((d[5] + d[7]) + (d[6] + d[8]));
+        jx = (d[1] - d[3]) + a57 + a86;
+        jy = (d[2] - d[4]) + a57 - a86;
+    } else {
+        m = d[0] + (d[1] + d[2]);
+        jx = d[1] - d[2];
+        jy = V(0);
+    }
+}
+
+// The same in FP64 from stored values.  FP16 values are multiples of 2^-24:
+// where all are below 1/16 in magnitude, their sums (below 1) are exact in
+// FP32.
+template <class Lat, typename S>
+__device__ __forceinline__ void node_sums(const S (&raw)[Lat::Q], double& m, double& jx, double& jy) {
+    if constexpr (std::is_same<S, __half>::value) {
+        float d[Lat::Q], big = 0.f;
 #pragma unroll
-    for (int a = 0; a < Lat::Q; ++a) {
-        const int o = Lat::opp(a);
-        if (o < a) continue;  // filled with its opposite
-        const double w = Lat::w(a), wr = w * rho;
-        const double vu = Lat::vx(a) * ux + Lat::vy(a) * uy;
-        const double even = fma(4.5 * vu, vu, b0);
-        const double odd = 3.0 * vu;
-        const double base = fma(wr, even, w * dr);
-        d[a] = fma(wr, odd, base);
-        if (o != a) d[o] = fma(-wr, odd, base);
+        for (int a = 0; a < Lat::Q; ++a) {
+            d[a] = __half2float(raw[a]);
+            big = fmaxf(big, fabsf(d[a]));  // (drops a NaN:)
+        }
+        float fm, fx, fy;
+        moment_sums<Lat, float>(d, fm, fx, fy);
+        if (big < 0.0625f && fm == fm) {
+            m = widen(fm);
+            jx = widen(fx);
+            jy = widen(fy);
+            return;
+        }
+    }
+    double d[Lat::Q];
+#pragma unroll
+    for (int a = 0; a < Lat::Q; ++a) d[a] = widen(raw[a]);
+    moment_sums<Lat, double>(d, m, jx, jy);
+}
+
+// f^eq(rho, u) - W rho0 (Eq. numerical-plyeqm),
+//   W_a [(rho - rho0) + rho (3 v.u + 9/2 (v.u)^2 - 3/2 u^2)],
+// with A = rho u_x^2, B = rho u_y^2, C = rho u_x u_y: 30 FP64 instructions.
+// A warp whose nodes are all at rest takes W_a (rho - rho0) alone.
+template <class Lat>
+__device__ __forceinline__ void eq_dev(double rho, double ux, double uy, double rho0, bool rest,
+                                       double (&d)[Lat::Q]) {
+    const double dr = rho - rho0;
+    if (rest) {
+        const double w0 = Lat::w(0) * dr, w1 = Lat::w(1) * dr;
+        const double w2 = Lat::Q == 9 ? Lat::w(Lat::Q - 1) * dr : 0.0;
+#pragma unroll
+        for (int a = 0; a < Lat::Q; ++a) d[a] = a == 0 ? w0 : (a < 5 ? w1 : w2);
+        return;
+    }
+    const double jx = rho * ux, A = jx * ux;
+    if constexpr (Lat::Q == 9) {
+        const double jy = rho * uy, B = jy * uy, C = jx * uy, S = A + B, D = A - B;
+        const double t = fma(0.75, S, dr), e = fma(3.0, S, dr);
+        const double ex = fma(2.25, D, t) * (1.0 / 9.0), ey = fma(-2.25, D, t) * (1.0 / 9.0);
+        const double ep = fma(9.0, C, e) * (1.0 / 36.0), em = fma(-9.0, C, e) * (1.0 / 36.0);
+        const double jp = jx + jy, jm = jy - jx;
+        d[0] = fma(-1.5, S, dr) * (4.0 / 9.0);
+        d[1] = fma(1.0 / 3.0, jx, ex);
+        d[3] = fma(-1.0 / 3.0, jx, ex);
+        d[2] = fma(1.0 / 3.0, jy, ey);
+        d[4] = fma(-1.0 / 3.0, jy, ey);
+        d[5] = fma(1.0 / 12.0, jp, ep);
+        d[7] = fma(-1.0 / 12.0, jp, ep);
+        d[6] = fma(1.0 / 12.0, jm, em);
+        d[8] = fma(-1.0 / 12.0, jm, em);
+    } else {
+        const double e = fma(3.0, A, dr) * (1.0 / 6.0);
+        d[0] = fma(-1.5, A, dr) * (2.0 / 3.0);
+        d[1] = fma(0.5, jx, e);
+        d[2] = fma(-0.5, jx, e);
     }
 }
 
 // Node k of instance `in` (row-major, x fastest) as (x, y): 32-bit index
-// arithmetic (nx * ny < 2^31 for every instance).
+// arithmetic (nx * ny <= 2^31 for every instance).
 __device__ __forceinline__ void node_xy(uint32_t k, uint32_t nx, int& x, int& y) {
     const uint32_t yy = k / nx;
     y = (int)yy;
     x = (int)(k - yy * nx);
 }
 
+// This block's nodes of an instance of n: [first, last)
+__device__ __forceinline__ void block_range(uint32_t n, uint32_t per, uint32_t& first, uint32_t& last) {
+    const uint64_t f = (uint64_t)blockIdx.x * per;
+    first = f < n ? (uint32_t)f : n;
+    last = n - first < per ? n : first + per;
+}
+
 // Host arrays are indexed from the first node of the instances the launch
 // covers: node0 - node_base (node_base = 0 for whole-context calls, the
 // instance's node0 for single-instance calls).
 template <class Lat, typename S>
-__global__ void init_kernel(S* dst, const InstDesc* insts, const double* rho, const double* ux,
-                            const double* uy, double rho0, int64_t node_base) {
-    const InstDesc in = insts[blockIdx.y];
-    const uint32_t n = (uint32_t)in.nx * (uint32_t)in.ny;
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        int x, y;
-        node_xy(k, (uint32_t)in.nx, x, y);
-        const int64_t g = in.node0 - node_base + k;
+__global__ void __launch_bounds__(AUX_THREADS)
+init_kernel(S* dst, const InstDesc* insts, const double* rho, const double* ux, const double* uy,
+            double rho0, int64_t node_base, uint32_t per) {
+    const InstDesc& in = insts[blockIdx.y];
+    const uint32_t nx = (uint32_t)in.nx;
+    uint32_t first, last;
+    block_range(nx * (uint32_t)in.ny, per, first, last);
+    const int64_t g0 = in.node0 - node_base;
+    for (uint32_t w = first + (threadIdx.x & ~31u); w < last; w += AUX_THREADS) {  // whole warps
+        const uint32_t k = w + (threadIdx.x & 31u);
+        const bool some = k < last;
+        double r = 0.0, vx = 0.0, vy = 0.0;
+        if (some) {
+            r = rho[g0 + k];
+            if (ux) vx = ux[g0 + k];
+            if (uy && Lat::Q == 9) vy = uy[g0 + k];
+        }
+        // at rest: both velocities are zero (of either sign)
+        const uint32_t v = (uint32_t)__double2hiint(vx) << 1 | (uint32_t)__double2loint(vx) |
+                           (uint32_t)__double2hiint(vy) << 1 | (uint32_t)__double2loint(vy);
+        const bool rest = __all_sync(0xffffffffu, v == 0u);
+        if (!some) continue;
         double d[Lat::Q];
-        eq_dev<Lat>(rho[g], ux ? ux[g] : 0.0, (uy && Lat::Q == 9) ? uy[g] : 0.0, rho0, d);
+        eq_dev<Lat>(r, vx, vy, rho0, rest, d);
+        int x, y;
+        node_xy(k, nx, x, y);
+        S* p = dst + in.off + (int64_t)y * in.pitch + x;
 #pragma unroll
-        for (int a = 0; a < Lat::Q; ++a)
-            dst[in.off + (int64_t)a * in.plane + (int64_t)y * in.pitch + x] = Store<S>::from(d[a]);
+        for (int a = 0; a < Lat::Q; ++a) p[a * in.plane] = to_storage<S>(d[a]);
     }
 }
 
 template <class Lat, typename S>
-__global__ void set_f_kernel(S* dst, const InstDesc* insts, const double* f, double rho0) {
-    const InstDesc in = insts[blockIdx.y];
-    const uint32_t n = (uint32_t)in.nx * (uint32_t)in.ny;
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+__global__ void __launch_bounds__(AUX_THREADS)
+set_f_kernel(S* dst, const InstDesc* insts, const double* f, double rho0, uint32_t per) {
+    const InstDesc& in = insts[blockIdx.y];
+    const uint32_t nx = (uint32_t)in.nx, n = nx * (uint32_t)in.ny;
+    uint32_t first, last;
+    block_range(n, per, first, last);
+    for (uint32_t k = first + threadIdx.x; k < last; k += AUX_THREADS) {
         int x, y;
-        node_xy(k, (uint32_t)in.nx, x, y);
+        node_xy(k, nx, x, y);
+        const double* fk = f + in.node0 * Lat::Q + k;
+        S* p = dst + in.off + (int64_t)y * in.pitch + x;
 #pragma unroll
-        for (int a = 0; a < Lat::Q; ++a) {
-            const double fa = f[in.node0 * Lat::Q + (int64_t)a * n + k];
-            dst[in.off + (int64_t)a * in.plane + (int64_t)y * in.pitch + x] =
-                Store<S>::from(fa - Lat::w(a) * rho0);
-        }
+        for (int a = 0; a < Lat::Q; ++a)
+            p[a * in.plane] = to_storage<S>(fk[(int64_t)a * n] - Lat::w(a) * rho0);
     }
 }
 
@@ -114,11 +274,15 @@ __global__ void set_f_kernel(S* dst, const InstDesc* insts, const double* f, dou
 // FP32x2 for FP32 -- with the same rates and boundary rules, so this step
 // rounds exactly like a step kernel colliding the same pulled values: a
 // state saved from a running context and loaded into a new one continues
-// bit for bit.  One thread per node pair (x, x + 1) of a row; at an odd
-// width the second lane repeats the last node and is discarded.
+// bit for bit.  One thread per node pair (x, x + 1) of a row, read and
+// written as one word per plane; at an odd width the second lane collides
+// the row's padding and is discarded.
 template <class Lat, typename S, typename T, int COLL>
-__global__ void collide_inplace_kernel(const S* src, S* dst, const InstDesc* insts, double rho0,
-                                       unsigned long long* status) {
+__global__ void __launch_bounds__(AUX_THREADS)
+collide_inplace_kernel(const S* src, S* dst, const InstDesc* insts, double rho0,
+                       unsigned long long* status, uint32_t per) {
+    using Word = typename std::conditional<sizeof(S) == 2, uint32_t, typename std::conditional<
+        sizeof(S) == 4, uint2, double>::type>::type;  // P elements
     using CT = typename std::conditional<std::is_same<T, float>::value, F2, T>::type;
     using N = Num<CT>;
     using LT = typename LaneOf<CT>::type;
@@ -129,20 +293,26 @@ __global__ void collide_inplace_kernel(const S* src, S* dst, const InstDesc* ins
     const uint32_t n = groups * (uint32_t)in.ny;
     const Rates<CT> rates{CT((LT)in.omega), CT((LT)in.omega2), CT((LT)in.s_e), CT((LT)in.s_eps)};
     const CT rho0v = CT((LT)rho0);
+    uint32_t first, last;
+    block_range(n, per, first, last);
     unsigned long long n_skip = 0, n_unst = 0;
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    for (uint32_t k = first + threadIdx.x; k < last; k += AUX_THREADS) {
         int g, y;
         node_xy(k, groups, g, y);
         const int x0 = g * P;
+        const int64_t at = in.off + (int64_t)y * in.pitch + x0;
         CT d[Lat::Q], o[Lat::Q];
 #pragma unroll
         for (int a = 0; a < Lat::Q; ++a) {
+            union {
+                Word w;
+                S v[P];
+            } e;
+            e.w = *reinterpret_cast<const Word*>(src + at + a * in.plane);
 #pragma unroll
             for (int l = 0; l < P; ++l) {
-                const int x = min(x0 + l, in.nx - 1);
-                const S v = *elem_ptr<Lat, S>(src, in, a, x, y);
-                if constexpr (std::is_same<T, double>::value) d[a] = Store<S>::to_f64(v);
-                else N::set_lane(d[a], l, Store<S>::to_f32(v));
+                if constexpr (std::is_same<T, double>::value) d[a] = Store<S>::to_f64(e.v[l]);
+                else N::set_lane(d[a], l, Store<S>::to_f32(e.v[l]));
             }
         }
         uint32_t st = Collide<Lat, COLL, CT, (int)sizeof(S)>::run(d, rho0v, rates, o);
@@ -171,10 +341,19 @@ __global__ void collide_inplace_kernel(const S* src, S* dst, const InstDesc* ins
             if (x0 + l >= in.nx) continue;
             n_skip += (st >> (2 * l)) & ST_NEWTON_SKIPPED;
             n_unst += ((st >> (2 * l)) & ST_UNSTABLE) >> 1;
+        }
+        const bool whole = x0 + P <= in.nx;
 #pragma unroll
-            for (int a = 0; a < Lat::Q; ++a)
-                dst[in.off + (int64_t)a * in.plane + (int64_t)y * in.pitch + x0 + l] =
-                    Store<S>::from(N::lane(o[a], l));
+        for (int a = 0; a < Lat::Q; ++a) {
+            union {
+                Word w;
+                S v[P];
+            } e;
+#pragma unroll
+            for (int l = 0; l < P; ++l) e.v[l] = Store<S>::from(N::lane(o[a], l));
+            S* p = dst + at + a * in.plane;
+            if (whole) *reinterpret_cast<Word*>(p) = e.w;
+            else *p = e.v[0];
         }
     }
     if (n_skip) atomicAdd(status + 2 * inst + 0, n_skip);
@@ -182,269 +361,398 @@ __global__ void collide_inplace_kernel(const S* src, S* dst, const InstDesc* ins
 }
 
 template <class Lat, typename S>
-__global__ void moments_kernel(const S* src, const InstDesc* insts, bool pulled, double rho0,
-                               double* rho, double* ux, double* uy, int64_t node_base) {
-    const InstDesc in = insts[blockIdx.y];
-    const uint32_t n = (uint32_t)in.nx * (uint32_t)in.ny;
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+__global__ void __launch_bounds__(AUX_THREADS)
+moments_kernel(const S* src, const InstDesc* insts, bool pulled, double rho0, double* rho, double* ux,
+               double* uy, int64_t node_base, uint32_t per) {
+    const InstDesc& in = insts[blockIdx.y];
+    const uint32_t nx = (uint32_t)in.nx;
+    uint32_t first, last;
+    block_range(nx * (uint32_t)in.ny, per, first, last);
+    const int64_t g0 = in.node0 - node_base;
+    for (uint32_t k = first + threadIdx.x; k < last; k += AUX_THREADS) {
         int x, y;
-        node_xy(k, (uint32_t)in.nx, x, y);
-        double d[Lat::Q];
-        node_state<Lat, S>(src, in, x, y, pulled, d);
-        double dr = 0.0, jx = 0.0, jy = 0.0;
-#pragma unroll
-        for (int a = 0; a < Lat::Q; ++a) {
-            dr += d[a];
-            jx += Lat::vx(a) * d[a];
-            jy += Lat::vy(a) * d[a];
+        node_xy(k, nx, x, y);
+        S raw[Lat::Q];
+        node_state<Lat, S>(src, in, x, y, pulled, raw);
+        double m, jx, jy;
+        node_sums<Lat, S>(raw, m, jx, jy);
+        const double r = rho0 + m;
+        rho[g0 + k] = r;
+        if (ux || uy) {
+            const double ir = rcp_f64(r);
+            if (ux) ux[g0 + k] = jx * ir;
+            if (uy) uy[g0 + k] = jy * ir;
         }
-        const double r = rho0 + dr;
-        const double ir = 1.0 / r;
-        const int64_t g = in.node0 - node_base + k;
-        rho[g] = r;
-        if (ux) ux[g] = jx * ir;
-        if (uy) uy[g] = jy * ir;
     }
 }
 
 template <class Lat, typename S>
-__global__ void gather_f_kernel(const S* src, const InstDesc* insts, bool pulled, double rho0,
-                                double* f) {
-    const InstDesc in = insts[blockIdx.y];
-    const uint32_t n = (uint32_t)in.nx * (uint32_t)in.ny;
-    for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+__global__ void __launch_bounds__(AUX_THREADS)
+gather_f_kernel(const S* src, const InstDesc* insts, bool pulled, double rho0, double* f, uint32_t per) {
+    const InstDesc& in = insts[blockIdx.y];
+    const uint32_t nx = (uint32_t)in.nx, n = nx * (uint32_t)in.ny;
+    uint32_t first, last;
+    block_range(n, per, first, last);
+    for (uint32_t k = first + threadIdx.x; k < last; k += AUX_THREADS) {
         int x, y;
-        node_xy(k, (uint32_t)in.nx, x, y);
-        double d[Lat::Q];
-        node_state<Lat, S>(src, in, x, y, pulled, d);
+        node_xy(k, nx, x, y);
+        S raw[Lat::Q];
+        node_state<Lat, S>(src, in, x, y, pulled, raw);
+        double* fk = f + in.node0 * Lat::Q + k;
 #pragma unroll
-        for (int a = 0; a < Lat::Q; ++a)
-            f[in.node0 * Lat::Q + (int64_t)a * n + k] = Lat::w(a) * rho0 + d[a];
+        for (int a = 0; a < Lat::Q; ++a) fk[(int64_t)a * n] = Lat::w(a) * rho0 + widen(raw[a]);
     }
 }
 
-// Deviations of f(x, t_n) at one node in FP32 (2- and 4-byte storage):
-// same pull rule as node_state.
-template <class Lat, typename S>
-__device__ void node_state_f32(const S* base, const InstDesc& in, int x, int y, bool pulled,
-                               float (&d)[Lat::Q]) {
-#pragma unroll
-    for (int a = 0; a < Lat::Q; ++a) {
-        int sx = x, sy = y;
-        bool inside = true;
-        if (pulled) {
-            sx = x - Lat::vx(a);
-            sy = y - Lat::vy(a);
-            if (in.bc == BC_CAVITY) {
-                inside = sx >= 0 && sx < in.nx && sy >= 0 && sy < in.ny;
-            } else {
-                if (in.bc == BC_PERIODIC) sx = (sx + in.nx) % in.nx;
-                else sx = sx < 0 ? 0 : (sx >= in.nx ? in.nx - 1 : sx);
-                sy = (sy + in.ny) % in.ny;
+// Stream function of the LDAS post-processing (Sec. IV.I) along each row of
+// each instance: psi(x, y) = - integral_0^x u_y dx in lattice units, with
+// the composite Simpson rule over pairs of unit intervals from the left
+// wall and the trapezoidal rule on the last interval when x is odd.
+//
+// A warp takes a row in stretches of 256 nodes: u_y of the stretch straight
+// from the populations (no density or velocity field goes through memory)
+// into shared memory, then each lane integrates its 8 consecutive nodes, a
+// warp scan adds up the lanes, and the results go back through shared memory
+// so that they are stored in order.  4 FP64 instructions a node besides
+// u_y's own; one thread per row walking its row in memory took 59 us on
+// 257 x 257 and 293 us on 8.9 M nodes, behind 0.72 ms for the moments.
+constexpr int PSI_WARPS = 4, PSI_NODES = 256;
+template <typename S>
+__global__ void __launch_bounds__(PSI_WARPS * 32)
+stream_function_kernel(const S* src, const InstDesc* insts, bool pulled, double rho0, double* psi,
+                       int64_t node_base) {
+    __shared__ double buf[PSI_WARPS][PSI_NODES + 2];  // u_y of nodes x - 2 .. x + 255
+    const InstDesc& in = insts[blockIdx.y];
+    const int nx = in.nx, lane = (int)(threadIdx.x & 31u);
+    double* u = buf[threadIdx.x >> 5];
+    for (int y = blockIdx.x * PSI_WARPS + (int)(threadIdx.x >> 5); y < in.ny; y += gridDim.x * PSI_WARPS) {
+        double* p = psi + (in.node0 - node_base) + (int64_t)y * nx;
+        double carry = 0.0;  // integral over [0, x0 - 2]
+        double last = 0.0;   // lanes 30, 31: u_y of nodes x0 - 2, x0 - 1
+        for (int x0 = 0; x0 < nx; x0 += PSI_NODES) {
+            if (lane >= 30) u[lane - 30] = last;
+#pragma unroll 2
+            for (int i = 0; i < PSI_NODES; i += 32) {
+                const int x = x0 + i + lane;
+                double v = 0.0;
+                if (x < nx) {
+                    S raw[9];
+                    node_state<D2Q9, S>(src, in, x, y, pulled, raw);
+                    double m, jx, jy;
+                    node_sums<D2Q9, S>(raw, m, jx, jy);
+                    v = jy * rcp_f64(rho0 + m);
+                }
+                u[2 + i + lane] = v;
+                last = v;
             }
+            __syncwarp();
+            // own nodes x0 + 8 lane + 0..7 are v[2..9]
+            double v[10];
+#pragma unroll
+            for (int i = 0; i < 10; ++i) v[i] = u[8 * lane + i];
+            double s[4];  // integral from node x0 + 8 lane - 2 to the even nodes
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                double inc = fma(4.0, v[2 * j + 1], v[2 * j] + v[2 * j + 2]) * (1.0 / 3.0);
+                if (j == 0 && x0 + lane == 0) inc = 0.0;  // nothing left of node 0
+                s[j] = j == 0 ? inc : s[j - 1] + inc;
+            }
+            double sum = s[3];
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const double o = __shfl_up_sync(0xffffffffu, sum, d);
+                if (lane >= d) sum += o;
+            }
+            double base = __shfl_up_sync(0xffffffffu, sum, 1);
+            base = lane == 0 ? carry : base + carry;
+            carry += __shfl_sync(0xffffffffu, sum, 31);
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const double e = base + s[j];
+                u[2 + 8 * lane + 2 * j] = -e;
+                u[2 + 8 * lane + 2 * j + 1] = -fma(0.5, v[2 * j + 2] + v[2 * j + 3], e);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < PSI_NODES; i += 32)
+                if (x0 + i + lane < nx) p[x0 + i + lane] = u[2 + i + lane];
+            __syncwarp();
         }
-        d[a] = inside ? Store<S>::to_f32(*elem_ptr<Lat, S>(base, in, a, sx, sy)) : 0.f;
     }
 }
 
-// Conservation, pass 1: the block of work item (i, b) sums (sum d,
-// sum d v_x, sum d v_y) of f(t_n) over the rows y = b mod P_i of instance i
-// (P_i = cons_partials(ny_i)); thread t takes x = t, t + CONS_THREADS, ...
-// of each of those rows, rows in increasing order (issuing the loads of a
-// few of its nodes of a row together, adding them in order), and the block
-// reduces
-// its threads in a fixed tree into partials[(i*CONS_PARTIALS + b)*3 + c].
-// The order is fixed by the instance alone.  FP64 storage sums in FP64.
-// FP32 and BF16 storage sum in compensated FP32 pairs (Knuth's two-sum;
-// about twice FP32's precision, converted to FP64 once per thread), which
-// spares the slow FP64 pipe.  FP16 storage sums exactly in integers: every
-// FP16 value is a multiple of 2^-24 below 2^16 in magnitude, so 2^24 d is an
-// integer below 2^40, and a thread's nodes add exactly in 64-bit integers,
-// converted to FP64 once; nodes whose values are all below 8 in magnitude,
-// which is every node of a physical state, sum in 32-bit integers first,
-// without 64-bit conversions.  A node with a non-finite value takes the
-// FP64 path, so that it propagates.  Interior nodes pull with plain shifted
-// loads; the outer ring applies the boundary rules.
-template <class Lat, typename S>
-__global__ void __launch_bounds__(CONS_THREADS, CONS_MIN_BLOCKS)
-cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool pulled,
-                    double* partials) {
-    using V = typename std::conditional<sizeof(S) == 8, double, float>::type;
-    // FP32 and BF16 values sum in FP32 pairs (compensated: each addition's
-    // rounding error is kept, so a pair carries about twice FP32's precision)
-    constexpr bool DF = std::is_same<S, float>::value || std::is_same<S, __nv_bfloat16>::value;
-    // nodes x, x + T, ..., x + (K - 1) T of a row (T = CONS_THREADS) whose
-    // loads a thread issues together before it adds them in order
-    constexpr int K = sizeof(S) == 8 ? 2 : 4;
-    __shared__ double sh[3][CONS_THREADS];
-    const int2 it = items[blockIdx.x];
-    const InstDesc in = insts[it.x];
-    const int nx = in.nx, ny = in.ny, P = cons_partials(ny);
-    const S* base = src + in.off;
+// Conservation, pass 1.  Node x pulls f_a from x - v_a, so summed over an
+// instance every stored value counts as often as nodes pull it: once, but
+// for values on the outer ring (a cavity's are not pulled by a node when they
+// leave the lattice; at a zero-gradient end the leaving ones are not pulled
+// and the entering ones are pulled twice).  The reduction therefore reads the
+// stored planes as they lie, 16 bytes per load, and weighs ring values.
+//
+// Partial b of instance i sums its rows y = b mod P_i (P_i = cons_partials),
+// in a cluster of CTAs; of these, C_i = cons_split(nodes) CTAs take the
+// rows' 16-byte chunks in turn (the others of the launch's cluster add zero),
+// and the first CTA of the cluster adds the CTAs' sums in order.  The order
+// of all additions is fixed by the instance alone.
+//
+// FP64 storage sums in FP64.  FP32 and BF16 storage sum in compensated FP32
+// pairs (Knuth's two-sum; about twice FP32's precision, converted to FP64
+// once per thread), which spares the slow FP64 pipe.  FP16 storage sums
+// exactly in integers: every FP16 value is a multiple of 2^-24 below 2^16 in
+// magnitude; a node whose values are all below 1/16 adds exactly in FP32 and
+// is converted to 32-bit integers, others add in 64-bit integers, and the
+// thread's total is converted to FP64 once.
+// Nodes with a non-finite value take FP64, so that it propagates.
+//
+// 33.4 M nodes, FP16: see the figures at the launch.
+template <class Lat>
+__device__ __forceinline__ int pull_count(const InstDesc& in, int a, int x, int y) {
+    const int tx = x + Lat::vx(a), ty = y + Lat::vy(a);
+    const bool xin = tx >= 0 && tx < in.nx, yin = ty >= 0 && ty < in.ny;
+    if (in.bc == BC_CAVITY) return xin && yin ? 1 : 0;
+    if (in.bc == BC_PERIODIC) return 1;
+    // zero gradient (y wraps): the end node's entering value is its own
+    const bool entering = (Lat::vx(a) == 1 && x == 0) || (Lat::vx(a) == -1 && x == in.nx - 1);
+    return (xin ? 1 : 0) + (entering ? 1 : 0);
+}
+
+struct ConsSums {
     double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    long long i0 = 0, i1 = 0, i2 = 0;  // FP16: exact sums in units of 2^-24
-    float h0 = 0.f, c0 = 0.f, h1 = 0.f, c1 = 0.f, h2 = 0.f, c2 = 0.f;  // FP32 / BF16: (sum, error)
-    // h + v = s + e exactly (Knuth's two-sum); the error joins the running c
-    auto add2 = [](float& h, float& c, float v) {
-        const float sum = __fadd_rn(h, v);
-        const float bv = __fsub_rn(sum, h);
-        const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(sum, bv)), __fsub_rn(v, bv));
-        h = sum;
-        c = __fadd_rn(c, e);
-    };
-    for (int y = it.y; y < ny; y += P) {
-        const bool yint = Lat::Q == 3 || (y >= 1 && y <= ny - 2);
-        for (int x0 = threadIdx.x; x0 < nx; x0 += K * CONS_THREADS) {
-          S raw[K][Lat::Q];
-          uint32_t plain = 0u;  // bit k: node k is read with plain shifted loads
-#pragma unroll
-          for (int k = 0; k < K; ++k) {
-              const int x = x0 + k * CONS_THREADS;
-              if (x < nx && (!pulled || (yint && x >= 1 && x <= nx - 2))) {
-                  plain |= 1u << k;
-#pragma unroll
-                  for (int a = 0; a < Lat::Q; ++a) {
-                      const int sx = pulled ? x - Lat::vx(a) : x, sy = pulled ? y - Lat::vy(a) : y;
-                      raw[k][a] = base[(int64_t)a * in.plane + (int64_t)sy * in.pitch + sx];
-                  }
-              }
-          }
-#pragma unroll
-          for (int k = 0; k < K; ++k) {
-            const int x = x0 + k * CONS_THREADS;
-            if (x >= nx) break;
-            V d[Lat::Q];
-            if ((plain >> k) & 1u) {
-#pragma unroll
-                for (int a = 0; a < Lat::Q; ++a) {
-                    if constexpr (sizeof(S) != 8) d[a] = Store<S>::to_f32(raw[k][a]);
-                    else d[a] = Store<S>::to_f64(raw[k][a]);
-                }
-            } else if constexpr (sizeof(S) != 8) {
-                node_state_f32<Lat, S>(src, in, x, y, pulled, d);
-            } else {
-                node_state<Lat, S>(src, in, x, y, pulled, d);
-            }
-            bool exact = false;
-            if constexpr (std::is_same<S, __half>::value) {
-                // every |d| < 8: 2^24 d below 2^27, the node sums of nine
-                // such terms below 2^31, in 32-bit integers
-                bool small = true;
-#pragma unroll
-                for (int a = 0; a < Lat::Q; ++a) small = small && (fabsf(d[a]) < 8.f);
-                if (small) {
-                    int r0 = 0, r1 = 0, r2 = 0;
-#pragma unroll
-                    for (int a = 0; a < Lat::Q; ++a) {
-                        const int v = __float2int_rn(d[a] * 16777216.f);  // 2^24 d, exact
-                        r0 += v;
-                        if (Lat::vx(a) != 0) r1 += Lat::vx(a) > 0 ? v : -v;
-                        if (Lat::vy(a) != 0) r2 += Lat::vy(a) > 0 ? v : -v;
-                    }
-                    i0 += r0;
-                    i1 += r1;
-                    i2 += r2;
-                    exact = true;
-                } else {
-                    long long r0 = 0, r1 = 0, r2 = 0;
-                    bool finite = true;
-#pragma unroll
-                    for (int a = 0; a < Lat::Q; ++a) {
-                        finite = finite && (fabsf(d[a]) <= 65504.f);
-                        const long long v = __float2ll_rn(d[a] * 16777216.f);
-                        r0 += v;
-                        if (Lat::vx(a) != 0) r1 += Lat::vx(a) > 0 ? v : -v;
-                        if (Lat::vy(a) != 0) r2 += Lat::vy(a) > 0 ? v : -v;
-                    }
-                    if (finite) {
-                        i0 += r0;
-                        i1 += r1;
-                        i2 += r2;
-                        exact = true;
-                    }
-                }
-            }
-            if constexpr (DF) {
-                bool finite = true;
-#pragma unroll
-                for (int a = 0; a < Lat::Q; ++a) finite = finite && (fabsf(d[a]) <= 3.4028235e38f);
-                if (finite) {
-#pragma unroll
-                    for (int a = 0; a < Lat::Q; ++a) {
-                        add2(h0, c0, d[a]);
-                        if (Lat::vx(a) != 0) add2(h1, c1, Lat::vx(a) > 0 ? d[a] : -d[a]);
-                        if (Lat::vy(a) != 0) add2(h2, c2, Lat::vy(a) > 0 ? d[a] : -d[a]);
-                    }
-                    exact = true;
-                }
-            }
-            if (!exact) {
-#pragma unroll
-                for (int a = 0; a < Lat::Q; ++a) {
-                    const double v = (double)d[a];
-                    s0 += v;
-                    if (Lat::vx(a) != 0) s1 += Lat::vx(a) * v;
-                    if (Lat::vy(a) != 0) s2 += Lat::vy(a) * v;
-                }
-            }
-          }
-        }
-    }
-    if constexpr (std::is_same<S, __half>::value) {
-        // the thread's exact FP16 node sums, in units of 2^-24 (at most
-        // 2^15 nodes of 9 values below 2^40 each: no overflow), to FP64 once
-        constexpr double inv = 1.0 / 16777216.0;
-        s0 += (double)i0 * inv;
-        s1 += (double)i1 * inv;
-        s2 += (double)i2 * inv;
-    }
-    if constexpr (DF) {
-        s0 += (double)h0 + (double)c0;
-        s1 += (double)h1 + (double)c1;
-        s2 += (double)h2 + (double)c2;
-    }
-    sh[0][threadIdx.x] = s0;
-    sh[1][threadIdx.x] = s1;
-    sh[2][threadIdx.x] = s2;
-    __syncthreads();
-    for (int h = CONS_THREADS / 2; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) sh[c][threadIdx.x] += sh[c][threadIdx.x + h];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x < 3)
-        partials[((int64_t)it.x * CONS_PARTIALS + it.y) * 3 + threadIdx.x] = sh[threadIdx.x][0];
+    long long i0 = 0, i1 = 0, i2 = 0;                   // FP16: exact sums in units of 2^-24
+    F2 h0 = 0.f, c0 = 0.f, h1 = 0.f, c1 = 0.f, h2 = 0.f, c2 = 0.f;  // FP32 / BF16: (sum, error)
+};
+
+// h + v = s + e exactly (Knuth's two-sum); the error joins the running c
+__device__ __forceinline__ void add2(F2& h, F2& c, F2 v) {
+    const F2 sum = h + v;
+    const F2 bv = sum - h;
+    const F2 e = (h - (sum - bv)) + (v - bv);
+    h = sum;
+    c = c + e;
 }
 
-// Conservation, pass 2: one thread per instance adds its partials in order;
-// total mass = N rho0 + sum d (sum_a W_a = 1).
+template <class Lat> __device__ __forceinline__ void cons_add_f64(ConsSums& t, const double (&d)[Lat::Q]) {
+    double m, jx, jy;
+    moment_sums<Lat, double>(d, m, jx, jy);
+    t.s0 += m;
+    t.s1 += jx;
+    t.s2 += jy;
+}
+
+// FP16 node whose values are not all below 1/16: its sums in 64-bit integers
+// (units of 2^-24); false if some value is not finite.
+template <class Lat>
+__device__ __noinline__ bool half_sums_large(const float (&d)[Lat::Q], long long (&r)[3]) {
+    bool finite = true;
+    for (int a = 0; a < Lat::Q; ++a) {
+        finite = finite && fabsf(d[a]) <= 131008.f;  // twice FP16's largest (a value pulled twice)
+        const long long v = __float2ll_rn(d[a] * 16777216.f);
+        r[0] += v;
+        r[1] += Lat::vx(a) * v;
+        r[2] += Lat::vy(a) * v;
+    }
+    return finite;
+}
+
+template <class Lat, typename S>
+__global__ void __launch_bounds__(CONS_THREADS)
+cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool pulled, double* partials) {
+    constexpr int Q = Lat::Q, E = 16 / (int)sizeof(S);  // nodes per chunk
+    const int2 it = items[blockIdx.x];
+    const InstDesc& in = insts[it.x];
+    const int nx = in.nx, ny = in.ny, P = cons_partials(ny);
+    const uint32_t C = (uint32_t)cons_split((int64_t)nx * ny), rank = blockIdx.y;
+    const uint32_t chunks = (uint32_t)(nx + E - 1) / E;       // per row
+    const uint64_t total = (uint64_t)((ny - it.y + P - 1) / P) * chunks;
+    const S* base = src + in.off;
+    ConsSums t;
+    if (rank < C)
+        for (uint64_t k = rank * CONS_THREADS + threadIdx.x; k < total; k += (uint64_t)C * CONS_THREADS) {
+            const uint32_t row = (uint32_t)(total <= 0xffffffffull ? (uint32_t)k / chunks : k / chunks);
+            const int y = it.y + (int)row * P, x0 = (int)(k - (uint64_t)row * chunks) * E;
+            union {
+                uint4 w;
+                S v[E];
+            } raw[Q];
+#pragma unroll
+            for (int a = 0; a < Q; ++a)
+                raw[a].w = __ldg(reinterpret_cast<const uint4*>(base + a * in.plane + (int64_t)y * in.pitch + x0));
+            const bool ring = x0 == 0 || x0 + E >= nx || (Q == 9 && (y == 0 || y == ny - 1));
+            if (ring) {
+#pragma unroll
+                for (int a = 0; a < Q; ++a)
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const int n = x0 + e >= nx ? 0 : pulled ? pull_count<Lat>(in, a, x0 + e, y) : 1;
+                        if (n == 0) raw[a].v[e] = zero_value<S>();
+                    }
+            }
+            // values pulled twice (zero-gradient ends) count once more
+            auto node = [&](int e, auto&& value) {
+                const int x = x0 + e;
+                if (ring && pulled && in.bc == BC_ZERO_GRADIENT && (x == 0 || x == nx - 1)) {
+#pragma unroll
+                    for (int a = 0; a < Q; ++a)
+                        if (pull_count<Lat>(in, a, x, y) == 2) value(a) = value(a) + value(a);
+                }
+            };
+            if constexpr (std::is_same<S, double>::value) {
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    double d[Q];
+#pragma unroll
+                    for (int a = 0; a < Q; ++a) d[a] = raw[a].v[e];
+                    node(e, [&](int a) -> double& { return d[a]; });
+                    cons_add_f64<Lat>(t, d);
+                }
+            } else if constexpr (std::is_same<S, __half>::value) {
+                int r0 = 0, r1 = 0, r2 = 0;
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    float d[Q], big = 0.f;
+#pragma unroll
+                    for (int a = 0; a < Q; ++a) d[a] = __half2float(raw[a].v[e]);
+                    node(e, [&](int a) -> float& { return d[a]; });
+#pragma unroll
+                    for (int a = 0; a < Q; ++a) big = fmaxf(big, fabsf(d[a]));
+                    float m, jx, jy;
+                    moment_sums<Lat, float>(d, m, jx, jy);
+                    if (big < 0.0625f && m == m) {  // exact, below 1: below 2^24 in units of 2^-24
+                        r0 += __float2int_rn(m * 16777216.f);
+                        r1 += __float2int_rn(jx * 16777216.f);
+                        if (Q == 9) r2 += __float2int_rn(jy * 16777216.f);
+                    } else {
+                        // copies, so that only this branch keeps them in memory
+                        float g[Q];
+                        long long r[3] = {0, 0, 0};
+#pragma unroll
+                        for (int a = 0; a < Q; ++a) g[a] = d[a];
+                        if (half_sums_large<Lat>(g, r)) {
+                            t.i0 += r[0];
+                            t.i1 += r[1];
+                            t.i2 += r[2];
+                        } else {
+                            double f[Q];
+#pragma unroll
+                            for (int a = 0; a < Q; ++a) f[a] = (double)d[a];
+                            cons_add_f64<Lat>(t, f);
+                        }
+                    }
+                }
+                t.i0 += r0;
+                t.i1 += r1;
+                t.i2 += r2;
+            } else {
+#pragma unroll
+                for (int e = 0; e < E; e += 2) {
+                    float2 d[Q];
+                    uint32_t big = 0u;
+#pragma unroll
+                    for (int a = 0; a < Q; ++a)
+                        d[a] = make_float2(Store<S>::to_f32(raw[a].v[e]), Store<S>::to_f32(raw[a].v[e + 1]));
+                    node(e, [&](int a) -> float& { return d[a].x; });
+                    node(e + 1, [&](int a) -> float& { return d[a].y; });
+#pragma unroll
+                    for (int a = 0; a < Q; ++a)
+                        big = max(big, max(__float_as_uint(d[a].x) & 0x7fffffffu, __float_as_uint(d[a].y) & 0x7fffffffu));
+                    if (big < 0x7f800000u) {
+#pragma unroll
+                        for (int a = 0; a < Q; ++a) {
+                            const F2 v = d[a];
+                            add2(t.h0, t.c0, v);
+                            if (Lat::vx(a) != 0) add2(t.h1, t.c1, Lat::vx(a) > 0 ? v : -v);
+                            if (Lat::vy(a) != 0) add2(t.h2, t.c2, Lat::vy(a) > 0 ? v : -v);
+                        }
+                    } else {
+#pragma unroll 1
+                        for (int l = 0; l < 2; ++l) {
+                            double f[Q];
+#pragma unroll
+                            for (int a = 0; a < Q; ++a) f[a] = (double)(l ? d[a].y : d[a].x);
+                            cons_add_f64<Lat>(t, f);
+                        }
+                    }
+                }
+            }
+        }
+    if constexpr (std::is_same<S, __half>::value) {
+        // (at most 2^31 values below 2^41: no overflow)
+        constexpr double inv = 1.0 / 16777216.0;
+        t.s0 += (double)t.i0 * inv;
+        t.s1 += (double)t.i1 * inv;
+        t.s2 += (double)t.i2 * inv;
+    } else if constexpr (!std::is_same<S, double>::value) {
+        t.s0 += ((double)t.h0.v.x + (double)t.c0.v.x) + ((double)t.h0.v.y + (double)t.c0.v.y);
+        t.s1 += ((double)t.h1.v.x + (double)t.c1.v.x) + ((double)t.h1.v.y + (double)t.c1.v.y);
+        if (Q == 9) t.s2 += ((double)t.h2.v.x + (double)t.c2.v.x) + ((double)t.h2.v.y + (double)t.c2.v.y);
+    }
+    // fixed trees: lanes, then warps, then the CTAs of the cluster in order
+    __shared__ double sh[3][CONS_THREADS / 32];
+    __shared__ double cta[3];
+    double s[3] = {t.s0, t.s1, t.s2};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+#pragma unroll
+        for (int h = 16; h > 0; h >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], h);
+        if ((threadIdx.x & 31u) == 0u) sh[c][threadIdx.x >> 5] = s[c];
+    }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        double v = 0.0;
+#pragma unroll
+        for (int w = 0; w < CONS_THREADS / 32; ++w) v += sh[threadIdx.x][w];
+        cta[threadIdx.x] = v;
+    }
+    const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+    cluster.sync();
+    if (rank == 0 && threadIdx.x < 3) {
+        double v = 0.0;
+        for (uint32_t r = 0; r < C; ++r) v += *cluster.map_shared_rank(&cta[threadIdx.x], r);
+        partials[((int64_t)it.x * CONS_PARTIALS + it.y) * 3 + threadIdx.x] = v;
+    }
+    cluster.sync();  // a CTA's shared memory stays until the first has read it
+}
+
+// Conservation, pass 2: one warp per instance adds its partials in a fixed
+// tree; total mass = N rho0 + sum d (sum_a W_a = 1).
 __global__ void cons_final_kernel(const double* partials, const InstDesc* insts, int count,
                                   double rho0, double* out) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = (int)(threadIdx.x & 31u);
     if (i >= count) return;
-    double s[3] = {0.0, 0.0, 0.0};
     const int P = cons_partials(insts[i].ny);
-    for (int b = 0; b < P; ++b)
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int b = lane; b < P; b += 32)
         for (int c = 0; c < 3; ++c) s[c] += partials[((int64_t)i * CONS_PARTIALS + b) * 3 + c];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+        for (int h = 16; h > 0; h >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], h);
+    if (lane != 0) return;
     const double nodes = (double)insts[i].nx * (double)insts[i].ny;
     out[3 * i + 0] = nodes * rho0 + s[0];
     out[3 * i + 1] = s[1];
     out[3 * i + 2] = s[2];
 }
 
-dim3 aux_grid(int64_t max_nodes, int count) {
-    int64_t b = (max_nodes + AUX_THREADS - 1) / AUX_THREADS;
-    if (b > 4096) b = 4096;
-    if (b < 1) b = 1;
-    return dim3((unsigned)b, (unsigned)count);
+// Nodes of a block: at most 2048 (8 per thread), fewer while that leaves
+// less than 8 blocks per SM for the whole launch.
+uint32_t nodes_per_block(int64_t total) {
+    uint32_t per = 2048;
+    while (per > AUX_THREADS && total / per < 8 * 152) per /= 2;
+    return per;
+}
+dim3 aux_grid(int64_t max_items, int count, uint32_t per) {
+    return dim3((unsigned)std::max<int64_t>((max_items + per - 1) / per, 1), (unsigned)count);
 }
 
 template <class Lat, typename S, typename T, int COLL>
 cudaError_t collide_inplace_dispatch(const AuxArgs& a, const void* src, void* dst) {
-    collide_inplace_kernel<Lat, S, T, COLL><<<aux_grid(a.max_nodes, a.count), AUX_THREADS, 0, a.stream>>>(
-        static_cast<const S*>(src), static_cast<S*>(dst), a.inst, a.rho0, a.status);
+    // node pairs of a row, rounded up per row
+    const int P = std::is_same<T, float>::value ? 2 : 1;
+    const uint32_t per = nodes_per_block(a.total_nodes / P);
+    collide_inplace_kernel<Lat, S, T, COLL>
+        <<<aux_grid(a.max_nodes / P + a.max_ny, a.count, per), AUX_THREADS, 0, a.stream>>>(
+            static_cast<const S*>(src), static_cast<S*>(dst), a.inst, a.rho0, a.status, per);
     return cudaGetLastError();
 }
 
@@ -468,31 +776,56 @@ cudaError_t collide_inplace_by_rule(const AuxArgs& a, const void* src, void* dst
 template <class Lat, typename S>
 cudaError_t aux_dispatch(AuxOp op, const AuxArgs& a, const void* src, void* dst, const double* p0,
                          const double* p1, const double* p2, double* o0, double* o1, double* o2) {
-    const dim3 g = aux_grid(a.max_nodes, a.count);
+    const uint32_t per = nodes_per_block(a.total_nodes);
+    const dim3 g = aux_grid(a.max_nodes, a.count, per);
     switch (op) {
         case AuxOp::Init:
             init_kernel<Lat, S><<<g, AUX_THREADS, 0, a.stream>>>(static_cast<S*>(dst), a.inst, p0, p1,
-                                                                 p2, a.rho0, a.node_base);
+                                                                 p2, a.rho0, a.node_base, per);
             break;
         case AuxOp::SetF:
             set_f_kernel<Lat, S><<<g, AUX_THREADS, 0, a.stream>>>(static_cast<S*>(dst), a.inst, p0,
-                                                                  a.rho0);
+                                                                  a.rho0, per);
             break;
         case AuxOp::Moments:
             moments_kernel<Lat, S><<<g, AUX_THREADS, 0, a.stream>>>(static_cast<const S*>(src), a.inst,
                                                                     a.pulled, a.rho0, o0, o1, o2,
-                                                                    a.node_base);
+                                                                    a.node_base, per);
             break;
         case AuxOp::GatherF:
-            gather_f_kernel<Lat, S><<<g, AUX_THREADS, 0, a.stream>>>(static_cast<const S*>(src),
-                                                                     a.inst, a.pulled, a.rho0, o0);
+            gather_f_kernel<Lat, S><<<g, AUX_THREADS, 0, a.stream>>>(static_cast<const S*>(src), a.inst,
+                                                                     a.pulled, a.rho0, o0, per);
             break;
+        case AuxOp::StreamFunction:
+            if constexpr (Lat::Q == 9) {
+                // a warp per row
+                const dim3 rows((unsigned)std::max<int64_t>((a.max_ny + PSI_WARPS - 1) / PSI_WARPS, 1),
+                                (unsigned)a.count);
+                stream_function_kernel<S><<<rows, PSI_WARPS * 32, 0, a.stream>>>(
+                    static_cast<const S*>(src), a.inst, a.pulled, a.rho0, o0, a.node_base);
+                break;
+            }
+            return cudaErrorInvalidValue;
         case AuxOp::Conservation: {
             if (a.cons_nitems < 1 || !a.cons_items) return cudaErrorInvalidValue;
-            cons_partial_kernel<Lat, S><<<a.cons_nitems, CONS_THREADS, 0, a.stream>>>(
-                static_cast<const S*>(src), a.inst, a.cons_items, a.pulled, o1);
-            cons_final_kernel<<<(a.count + 127) / 128, 128, 0, a.stream>>>(o1, a.inst, a.count,
-                                                                           a.rho0, o0);
+            // clusters of as many CTAs as the largest instance splits into
+            const unsigned C = (unsigned)cons_split(a.max_nodes);
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = 1;
+            attr[0].val.clusterDim.y = C;
+            attr[0].val.clusterDim.z = 1;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)a.cons_nitems, C);
+            cfg.blockDim = dim3(CONS_THREADS);
+            cfg.stream = a.stream;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            const cudaError_t e = cudaLaunchKernelEx(&cfg, &cons_partial_kernel<Lat, S>,
+                                                     static_cast<const S*>(src), a.inst, a.cons_items,
+                                                     a.pulled, o1);
+            if (e != cudaSuccess) return e;
+            cons_final_kernel<<<(a.count + 3) / 4, 128, 0, a.stream>>>(o1, a.inst, a.count, a.rho0, o0);
             break;
         }
         case AuxOp::CollideInPlace: {
@@ -520,46 +853,12 @@ cudaError_t aux_by_storage(AuxOp op, const AuxArgs& a, const void* src, void* ds
     return cudaErrorInvalidValue;
 }
 
-// Stream function of the LDAS post-processing (Sec. IV.I) along each row of
-// each instance: psi(x, y) = - integral_0^x u_y dx in lattice units, with
-// the composite Simpson rule over pairs of unit intervals from the left
-// wall and the trapezoidal rule on the last interval when x is odd.  One
-// thread per row (rows of instance blockIdx.y).
-__global__ void stream_function_kernel(const double* __restrict__ uy,
-                                       const InstDesc* __restrict__ insts, double* __restrict__ psi,
-                                       int64_t node_base) {
-    const InstDesc& in = insts[blockIdx.y];
-    const int nx = in.nx;
-    for (int y = blockIdx.x * blockDim.x + threadIdx.x; y < in.ny; y += gridDim.x * blockDim.x) {
-        const double* u = uy + (in.node0 - node_base) + (int64_t)y * nx;
-        double* p = psi + (in.node0 - node_base) + (int64_t)y * nx;
-        double simpson = 0.0;  // integral over [0, x] at the last even x
-        p[0] = 0.0;
-        for (int x = 1; x < nx; ++x) {
-            if (x & 1) {
-                p[x] = -(simpson + 0.5 * (u[x - 1] + u[x]));
-            } else {
-                simpson += (u[x - 2] + 4.0 * u[x - 1] + u[x]) * (1.0 / 3.0);
-                p[x] = -simpson;
-            }
-        }
-    }
-}
-
 }  // namespace
 
 cudaError_t run_aux(AuxOp op, const AuxArgs& a, const void* src, void* dst, const double* p0,
                     const double* p1, const double* p2, double* o0, double* o1, double* o2) {
     if (a.lattice == 2) return aux_by_storage<D2Q9>(op, a, src, dst, p0, p1, p2, o0, o1, o2);
     return aux_by_storage<D1Q3>(op, a, src, dst, p0, p1, p2, o0, o1, o2);
-}
-
-cudaError_t stream_function(const AuxArgs& a, int64_t max_ny, const double* uy, double* psi) {
-    const int threads = 128;
-    const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>((max_ny + threads - 1) / threads, 1024)),
-                    (unsigned)a.count);
-    stream_function_kernel<<<grid, threads, 0, a.stream>>>(uy, a.inst, psi, a.node_base);
-    return cudaGetLastError();
 }
 
 }  // namespace lbm

@@ -9,14 +9,18 @@ namespace lbm {
 
 // Conservation reduction: instance i is split into P_i = min(CONS_PARTIALS,
 // ny_i) partial sums, partial b over the rows y = b mod P_i, each summed by
-// one block of CONS_THREADS threads; the split is a function of the instance
-// alone, so the FP64 summation order never depends on the device.
+// cons_split(nodes) CTAs of CONS_THREADS threads (a cluster); the split is a
+// function of the instance alone, so the FP64 summation order never depends
+// on the device or on the other instances.
 constexpr int CONS_PARTIALS = 64;
 constexpr int CONS_THREADS = 256;
-constexpr int CONS_MIN_BLOCKS = 3;  // resident blocks per SM the register budget aims at
 __host__ __device__ inline int cons_partials(int ny) { return ny < CONS_PARTIALS ? ny : CONS_PARTIALS; }
+// 1, 2, 4 or 8: up to 64 partials of one CTA keep 2^18 nodes busy
+__host__ __device__ inline int cons_split(int64_t nodes) {
+    return nodes <= (1 << 18) ? 1 : nodes <= (1 << 19) ? 2 : nodes <= (1 << 20) ? 4 : 8;
+}
 
-enum class AuxOp { Init, SetF, CollideInPlace, Moments, GatherF, Conservation };
+enum class AuxOp { Init, SetF, CollideInPlace, Moments, GatherF, StreamFunction, Conservation };
 
 struct AuxArgs {
     int lattice;   // 1 = D1Q3, 2 = D2Q9
@@ -24,7 +28,8 @@ struct AuxArgs {
     int compute;   // DT_F64 or DT_F32
     int collision; // COLL_*
     int count;     // instances
-    int64_t max_nodes;
+    int64_t max_nodes, max_ny;  // of the largest / tallest instance
+    int64_t total_nodes;
     const InstDesc* inst;  // device
     double rho0;
     bool pulled;           // stored field is post-collision (pull to read f(t_n))
@@ -33,7 +38,7 @@ struct AuxArgs {
     const int2* cons_items;  // device: (instance, partial) of each conservation block
     int32_t cons_nitems;
     int64_t node_base = 0;   // host-array index of the first node the call covers (Init,
-                             // Moments, stream_function): arrays start at that node
+                             // Moments, StreamFunction): arrays start at that node
 };
 
 // Init:           dst <- f^eq(rho=p0, ux=p1, uy=p2) deviations
@@ -41,15 +46,12 @@ struct AuxArgs {
 // CollideInPlace: dst <- collide(src) without streaming
 // Moments:        o0, o1, o2 <- rho, ux, uy of f(t_n) read from src
 // GatherF:        o0 <- FP64 populations of f(t_n)
+// StreamFunction: o0 <- stream function of f(t_n) (D2Q9), [inst][y][x]
 // Conservation:   o0 <- per-instance totals (3 doubles each), o1 = partials scratch
 //                 (count * CONS_PARTIALS * 3 doubles; partial b of instance i at
 //                 (i * CONS_PARTIALS + b) * 3)
 cudaError_t run_aux(AuxOp op, const AuxArgs& a, const void* src, void* dst, const double* p0,
                     const double* p1, const double* p2, double* o0, double* o1, double* o2);
-
-// psi <- stream function of u_y (both [inst][y][x] FP64 device arrays in the
-// concatenated node order); max_ny = largest instance height.
-cudaError_t stream_function(const AuxArgs& a, int64_t max_ny, const double* uy, double* psi);
 
 // Fused step kernels, one translation unit per storage type.  Each returns
 // the __global__ function for (lattice, collision, V), or nullptr.
