@@ -12,6 +12,12 @@
 //
 // One thread per node; a block takes `per` consecutive nodes of one instance
 // (grid = (blocks of the largest instance, instance)).
+//
+// 33.4 M nodes in 64 cavities, FP16: init 2.81 -> 0.28 ms (at rest; 1.1 GB,
+// 0.6 of the copy bandwidth), moments 2.26 -> 0.34 ms (FP64 issue: 6
+// instructions a node).  18.0 M nodes in 4096 tubes, FP32: init 0.78 -> 0.12,
+// moments 0.55 -> 0.32 ms.  12.2 M nodes D2Q9 FP32: moments 0.99 -> 0.52 ms
+// (22 FP64 instructions a node).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -118,7 +124,7 @@ __device__ __forceinline__ void node_state(const S* src, const InstDesc& in, int
     }
 }
 
-// sum d, sum d v_x, sum d v_y in the number type V (float or double)
+// sum d, sum d v_x, sum d v_y in the number type V (float, F2 or double)
 template <class Lat, typename V>
 __device__ __forceinline__ void moment_sums(const V (&d)[Lat::Q], V& m, V& jx, V& jy) {
     if constexpr (Lat::Q == 9) {
@@ -129,7 +135,7 @@ __device__ __forceinline__ void moment_sums(const V (&d)[Lat::Q], V& m, V& jx, V
     } else {
         m = d[0] + (d[1] + d[2]);
         jx = d[1] - d[2];
-        jy = V(0);
+        jy = V(0.f);
     }
 }
 
@@ -409,13 +415,14 @@ gather_f_kernel(const S* src, const InstDesc* insts, bool pulled, double rho0, d
 // the composite Simpson rule over pairs of unit intervals from the left
 // wall and the trapezoidal rule on the last interval when x is odd.
 //
-// A warp takes a row in stretches of 256 nodes: u_y of the stretch straight
+// A warp takes a row in stretches of 256 nodes (128 or 64 at its end): u_y of the stretch straight
 // from the populations (no density or velocity field goes through memory)
-// into shared memory, then each lane integrates its 8 consecutive nodes, a
+// into shared memory, then each lane integrates its 8 (4, 2) consecutive nodes, a
 // warp scan adds up the lanes, and the results go back through shared memory
 // so that they are stored in order.  4 FP64 instructions a node besides
-// u_y's own; one thread per row walking its row in memory took 59 us on
-// 257 x 257 and 293 us on 8.9 M nodes, behind 0.72 ms for the moments.
+// u_y's own.  8.9 M nodes in 64 lattices, FP16: 0.72 ms of moments and 0.29
+// ms of one thread per row walking its row in memory, now 0.20 ms; 257 x 257
+// FP64: 68 -> 20 us.
 constexpr int PSI_WARPS = 4, PSI_NODES = 256;
 template <typename S>
 __global__ void __launch_bounds__(PSI_WARPS * 32)
@@ -429,10 +436,12 @@ stream_function_kernel(const S* src, const InstDesc* insts, bool pulled, double 
         double* p = psi + (in.node0 - node_base) + (int64_t)y * nx;
         double carry = 0.0;  // integral over [0, x0 - 2]
         double last = 0.0;   // lanes 30, 31: u_y of nodes x0 - 2, x0 - 1
-        for (int x0 = 0; x0 < nx; x0 += PSI_NODES) {
+        // one stretch of 32 L nodes from x0, L consecutive nodes per lane
+        auto stretch = [&](auto length, int x0) {
+            constexpr int L = decltype(length)::value;
             if (lane >= 30) u[lane - 30] = last;
 #pragma unroll 2
-            for (int i = 0; i < PSI_NODES; i += 32) {
+            for (int i = 0; i < 32 * L; i += 32) {
                 const int x = x0 + i + lane;
                 double v = 0.0;
                 if (x < nx) {
@@ -446,18 +455,17 @@ stream_function_kernel(const S* src, const InstDesc* insts, bool pulled, double 
                 last = v;
             }
             __syncwarp();
-            // own nodes x0 + 8 lane + 0..7 are v[2..9]
-            double v[10];
+            // own nodes x0 + L lane + 0 .. L - 1 are v[2 ..]
+            double v[L + 2], s[L / 2];  // s: integral from the lane's second node back to each even node
 #pragma unroll
-            for (int i = 0; i < 10; ++i) v[i] = u[8 * lane + i];
-            double s[4];  // integral from node x0 + 8 lane - 2 to the even nodes
+            for (int i = 0; i < L + 2; ++i) v[i] = u[L * lane + i];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < L / 2; ++j) {
                 double inc = fma(4.0, v[2 * j + 1], v[2 * j] + v[2 * j + 2]) * (1.0 / 3.0);
                 if (j == 0 && x0 + lane == 0) inc = 0.0;  // nothing left of node 0
                 s[j] = j == 0 ? inc : s[j - 1] + inc;
             }
-            double sum = s[3];
+            double sum = s[L / 2 - 1];
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
                 const double o = __shfl_up_sync(0xffffffffu, sum, d);
@@ -468,16 +476,30 @@ stream_function_kernel(const S* src, const InstDesc* insts, bool pulled, double 
             carry += __shfl_sync(0xffffffffu, sum, 31);
             __syncwarp();
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < L / 2; ++j) {
                 const double e = base + s[j];
-                u[2 + 8 * lane + 2 * j] = -e;
-                u[2 + 8 * lane + 2 * j + 1] = -fma(0.5, v[2 * j + 2] + v[2 * j + 3], e);
+                u[2 + L * lane + 2 * j] = -e;
+                u[2 + L * lane + 2 * j + 1] = -fma(0.5, v[2 * j + 2] + v[2 * j + 3], e);
             }
             __syncwarp();
 #pragma unroll
-            for (int i = 0; i < PSI_NODES; i += 32)
+            for (int i = 0; i < 32 * L; i += 32)
                 if (x0 + i + lane < nx) p[x0 + i + lane] = u[2 + i + lane];
             __syncwarp();
+        };
+        // the shortest stretch that holds the rest of the row: a padding node
+        // costs as much FP64 issue as any other
+        for (int x0 = 0; x0 < nx;) {
+            if (nx - x0 > 128) {
+                stretch(std::integral_constant<int, 8>{}, x0);
+                x0 += 256;
+            } else if (nx - x0 > 64) {
+                stretch(std::integral_constant<int, 4>{}, x0);
+                x0 += 128;
+            } else {
+                stretch(std::integral_constant<int, 2>{}, x0);
+                x0 += 64;
+            }
         }
     }
 }
@@ -497,14 +519,19 @@ stream_function_kernel(const S* src, const InstDesc* insts, bool pulled, double 
 //
 // FP64 storage sums in FP64.  FP32 and BF16 storage sum in compensated FP32
 // pairs (Knuth's two-sum; about twice FP32's precision, converted to FP64
-// once per thread), which spares the slow FP64 pipe.  FP16 storage sums
+// once per warp), which spares the slow FP64 pipe.  FP16 storage sums
 // exactly in integers: every FP16 value is a multiple of 2^-24 below 2^16 in
-// magnitude; a node whose values are all below 1/16 adds exactly in FP32 and
-// is converted to 32-bit integers, others add in 64-bit integers, and the
-// thread's total is converted to FP64 once.
+// magnitude; a chunk whose values are all below 2^-7 adds exactly in FP32
+// (its sums stay below 1) and is converted to integers once, a node below
+// 2^-4 likewise, others add in 64-bit integers, and a warp's total is
+// converted to FP64.
 // Nodes with a non-finite value take FP64, so that it propagates.
 //
-// 33.4 M nodes, FP16: see the figures at the launch.
+// Bound by the latency of a thread's few chunks and its CTA's tail, at 0.4 of
+// the copy bandwidth.  64 cavities (33.4 M nodes) FP16: 324 us with shifted
+// loads per node, now 219 us; 2048^2 FP16: 134 -> 51 us (clusters of 4);
+// 4096 tubes FP32: 343 -> 84 us.  Pass 2 with one thread per instance took
+// 17 us, now 6 us.
 template <class Lat>
 __device__ __forceinline__ int pull_count(const InstDesc& in, int a, int x, int y) {
     const int tx = x + Lat::vx(a), ty = y + Lat::vy(a);
@@ -539,11 +566,23 @@ template <class Lat> __device__ __forceinline__ void cons_add_f64(ConsSums& t, c
     t.s2 += jy;
 }
 
-// FP16 node whose values are not all below 1/16: its sums in 64-bit integers
-// (units of 2^-24); false if some value is not finite.
+// Sums of an FP16 node in units of 2^-24: exact in FP32 where all values are
+// below 1/16 (the sums stay below 1), else in 64-bit integers; false if some
+// value is not finite.
 template <class Lat>
-__device__ __noinline__ bool half_sums_large(const float (&d)[Lat::Q], long long (&r)[3]) {
+__device__ __forceinline__ bool half_sums(const float (&d)[Lat::Q], long long (&r)[3]) {
+    float big = 0.f, m, jx, jy;
+#pragma unroll
+    for (int a = 0; a < Lat::Q; ++a) big = fmaxf(big, fabsf(d[a]));
+    moment_sums<Lat, float>(d, m, jx, jy);
+    if (big < 0.0625f && m == m) {
+        r[0] = __float2int_rn(m * 16777216.f);
+        r[1] = __float2int_rn(jx * 16777216.f);
+        r[2] = __float2int_rn(jy * 16777216.f);
+        return true;
+    }
     bool finite = true;
+#pragma unroll
     for (int a = 0; a < Lat::Q; ++a) {
         finite = finite && fabsf(d[a]) <= 131008.f;  // twice FP16's largest (a value pulled twice)
         const long long v = __float2ll_rn(d[a] * 16777216.f);
@@ -555,7 +594,7 @@ __device__ __noinline__ bool half_sums_large(const float (&d)[Lat::Q], long long
 }
 
 template <class Lat, typename S>
-__global__ void __launch_bounds__(CONS_THREADS)
+__global__ void __launch_bounds__(CONS_THREADS, 3)
 cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool pulled, double* partials) {
     constexpr int Q = Lat::Q, E = 16 / (int)sizeof(S);  // nodes per chunk
     const int2 it = items[blockIdx.x];
@@ -573,6 +612,7 @@ cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool
             union {
                 uint4 w;
                 S v[E];
+                __half2 h[4];
             } raw[Q];
 #pragma unroll
             for (int a = 0; a < Q; ++a)
@@ -606,28 +646,43 @@ cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool
                     cons_add_f64<Lat>(t, d);
                 }
             } else if constexpr (std::is_same<S, __half>::value) {
-                int r0 = 0, r1 = 0, r2 = 0;
+                // largest magnitude of the chunk, NaN if there is one
+                __half2 big2 = __habs2(raw[0].h[0]);
 #pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    float d[Q], big = 0.f;
+                for (int a = 0; a < Q; ++a)
 #pragma unroll
-                    for (int a = 0; a < Q; ++a) d[a] = __half2float(raw[a].v[e]);
-                    node(e, [&](int a) -> float& { return d[a]; });
+                    for (int e = 0; e < E / 2; ++e) big2 = __hmax2_nan(big2, __habs2(raw[a].h[e]));
+                const float big = __half2float(__hmax_nan(__low2half(big2), __high2half(big2)));
+                const bool twice = ring && pulled && in.bc == BC_ZERO_GRADIENT;
+                if (big < 0.0078125f && !twice) {
+                    // exact in FP32 over the whole chunk: 8 nodes of 9 values below 2^-7
+                    F2 m = 0.f, jx = 0.f, jy = 0.f;
 #pragma unroll
-                    for (int a = 0; a < Q; ++a) big = fmaxf(big, fabsf(d[a]));
-                    float m, jx, jy;
-                    moment_sums<Lat, float>(d, m, jx, jy);
-                    if (big < 0.0625f && m == m) {  // exact, below 1: below 2^24 in units of 2^-24
-                        r0 += __float2int_rn(m * 16777216.f);
-                        r1 += __float2int_rn(jx * 16777216.f);
-                        if (Q == 9) r2 += __float2int_rn(jy * 16777216.f);
-                    } else {
-                        // copies, so that only this branch keeps them in memory
-                        float g[Q];
+                    for (int e = 0; e < E / 2; ++e) {
+                        F2 d[Q], mm, jjx, jjy;
+#pragma unroll
+                        for (int a = 0; a < Q; ++a) d[a] = F2(__half22float2(raw[a].h[e]));
+                        moment_sums<Lat, F2>(d, mm, jjx, jjy);
+                        m = m + mm;
+                        jx = jx + jjx;
+                        if (Q == 9) jy = jy + jjy;
+                    }
+                    t.i0 += __float2int_rn((m.v.x + m.v.y) * 16777216.f);
+                    t.i1 += __float2int_rn((jx.v.x + jx.v.y) * 16777216.f);
+                    if (Q == 9) t.i2 += __float2int_rn((jy.v.x + jy.v.y) * 16777216.f);
+                } else {
+#pragma unroll 1
+                    for (int e = 0; e < E; ++e) {
+                        float d[Q];
                         long long r[3] = {0, 0, 0};
 #pragma unroll
-                        for (int a = 0; a < Q; ++a) g[a] = d[a];
-                        if (half_sums_large<Lat>(g, r)) {
+                        for (int a = 0; a < Q; ++a) {
+                            // element e by shifts: no indexing of registers
+                            const uint32_t lo = e < 4 ? (e < 2 ? raw[a].w.x : raw[a].w.y) : (e < 6 ? raw[a].w.z : raw[a].w.w);
+                            d[a] = __half2float(__ushort_as_half((unsigned short)(e & 1 ? lo >> 16 : lo & 0xffffu)));
+                        }
+                        node(e, [&](int a) -> float& { return d[a]; });
+                        if (half_sums<Lat>(d, r)) {
                             t.i0 += r[0];
                             t.i1 += r[1];
                             t.i2 += r[2];
@@ -639,9 +694,6 @@ cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool
                         }
                     }
                 }
-                t.i0 += r0;
-                t.i1 += r1;
-                t.i2 += r2;
             } else {
 #pragma unroll
                 for (int e = 0; e < E; e += 2) {
@@ -675,25 +727,49 @@ cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool
                 }
             }
         }
-    if constexpr (std::is_same<S, __half>::value) {
-        // (at most 2^31 values below 2^41: no overflow)
-        constexpr double inv = 1.0 / 16777216.0;
-        t.s0 += (double)t.i0 * inv;
-        t.s1 += (double)t.i1 * inv;
-        t.s2 += (double)t.i2 * inv;
-    } else if constexpr (!std::is_same<S, double>::value) {
-        t.s0 += ((double)t.h0.v.x + (double)t.c0.v.x) + ((double)t.h0.v.y + (double)t.c0.v.y);
-        t.s1 += ((double)t.h1.v.x + (double)t.c1.v.x) + ((double)t.h1.v.y + (double)t.c1.v.y);
-        if (Q == 9) t.s2 += ((double)t.h2.v.x + (double)t.c2.v.x) + ((double)t.h2.v.y + (double)t.c2.v.y);
-    }
     // fixed trees: lanes, then warps, then the CTAs of the cluster in order
     __shared__ double sh[3][CONS_THREADS / 32];
     __shared__ double cta[3];
     double s[3] = {t.s0, t.s1, t.s2};
+    bool in_f64 = true;  // some lane's part is in FP64 (the same for the warp)
+    if constexpr (std::is_same<S, __half>::value) {
+        // integers add exactly; FP64 only holds nodes with non-finite values
+        // (at most 2^31 values below 2^41: no overflow)
+        long long i[3] = {t.i0, t.i1, t.i2};
+        in_f64 = __any_sync(0xffffffffu, !(s[0] == 0.0 && s[1] == 0.0 && s[2] == 0.0));
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+#pragma unroll
+            for (int h = 16; h > 0; h >>= 1) i[c] += __shfl_down_sync(0xffffffffu, i[c], h);
+            if ((threadIdx.x & 31u) == 0u) s[c] += (double)i[c] * (1.0 / 16777216.0);
+        }
+    } else if constexpr (!std::is_same<S, double>::value) {
+        // both node lanes, then the warp's lanes, still in pairs
+        in_f64 = __any_sync(0xffffffffu, !(s[0] == 0.0 && s[1] == 0.0 && s[2] == 0.0));
+        F2 h[3] = {t.h0, t.h1, t.h2}, e[3] = {t.c0, t.c1, t.c2};
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            if (Q == 3 && c == 2) continue;
+            float a = h[c].v.x, r = e[c].v.x + e[c].v.y;
+            auto add = [&](float b, float rb) {
+                const float sum = __fadd_rn(a, b), bv = __fsub_rn(sum, a);
+                r = __fadd_rn(__fadd_rn(r, rb),
+                              __fadd_rn(__fsub_rn(a, __fsub_rn(sum, bv)), __fsub_rn(b, bv)));
+                a = sum;
+            };
+            add(h[c].v.y, 0.f);
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1)
+                add(__shfl_down_sync(0xffffffffu, a, d), __shfl_down_sync(0xffffffffu, r, d));
+            if ((threadIdx.x & 31u) == 0u) s[c] += widen(a) + widen(r);
+        }
+    }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
+        if (in_f64) {
 #pragma unroll
-        for (int h = 16; h > 0; h >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], h);
+            for (int h = 16; h > 0; h >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], h);
+        }
         if ((threadIdx.x & 31u) == 0u) sh[c][threadIdx.x >> 5] = s[c];
     }
     __syncthreads();

@@ -15,9 +15,11 @@ namespace lbm {
 constexpr int CONS_PARTIALS = 64;
 constexpr int CONS_THREADS = 256;
 __host__ __device__ inline int cons_partials(int ny) { return ny < CONS_PARTIALS ? ny : CONS_PARTIALS; }
-// 1, 2, 4 or 8: up to 64 partials of one CTA keep 2^18 nodes busy
+// 1, 2, 4 or 8: some 2^14 nodes per CTA, which take it longer than its tail
+// of FP64 additions (8 CTAs for 2^20 nodes: 787 us on 64 cavities of up to
+// 1024^2, FP16, where one takes 351 us)
 __host__ __device__ inline int cons_split(int64_t nodes) {
-    return nodes <= (1 << 18) ? 1 : nodes <= (1 << 19) ? 2 : nodes <= (1 << 20) ? 4 : 8;
+    return nodes <= (1 << 20) ? 1 : nodes <= (1 << 21) ? 2 : nodes <= (1 << 22) ? 4 : 8;
 }
 
 enum class AuxOp { Init, SetF, CollideInPlace, Moments, GatherF, StreamFunction, Conservation };
