@@ -241,9 +241,9 @@ AuxArgs aux_args(const lbm_ctx* ctx) {
     return a;
 }
 
-// One-node-per-thread kernel: colliding nodes of an instance, nodes per
+// One-node-per-thread kernel: colliding nodes of an instance, and nodes per
 // tile-table entry (the fewest, from one warp up, whose entries fit the
-// table) and CTA size.
+// table).
 int64_t flat_fluid(int64_t nx, int64_t ny, int bc) {
     return bc == LBM_BC_CAVITY ? (nx - 2) * (ny - 2) : nx * ny;
 }
@@ -251,8 +251,7 @@ int flat_nodes(const lbm_ctx* ctx) {
     for (int e = 32;; e *= 2) {
         int64_t n = 0;
         for (const InstDesc& in : ctx->layout.inst) {
-            const int64_t fluid = flat_fluid(in.nx, in.ny, ctx->bc);
-            n += (fluid + e - 1) / e + ((int64_t)in.nx * in.ny - fluid + e - 1) / e;
+            n += (flat_fluid(in.nx, in.ny, ctx->bc) + e - 1) / e;
         }
         if (n <= ctx->layout.max_tiles) return e;
     }
@@ -263,7 +262,7 @@ bool is_flat(const lbm_ctx* ctx, const Shape& s) {
 int block_threads(const lbm_ctx* ctx, const Shape& s) {
     if (s.kind >= 1) return smem_block_threads(s.kind - 1);
     if (ctx->lattice == 1) return std::max(32, std::min(s.tw * s.th, 256) / 32 * 32);
-    return is_flat(ctx, s) ? std::min(ctx->flat_nodes, FLAT_MAX_THREADS) : s.tw * s.th;
+    return is_flat(ctx, s) ? 32 : s.tw * s.th;
 }
 
 // Tube kernel: nodes per lane V and halo (= steps per launch) of a context,
@@ -334,17 +333,13 @@ std::vector<TileDesc> build_tiles(const lbm_ctx* ctx, const Shape& s) {
         return t;
     }
     if (is_flat(ctx, s)) {
-        // flat_nodes consecutive nodes per entry: the fluid nodes of every
-        // instance, then the rings of the cavities
-        for (int part = 0; part < 2; ++part)
-            for (int i = 0; i < ctx->count; ++i) {
-                const InstDesc& in = ctx->layout.inst[i];
-                const int64_t n = (int64_t)in.nx * in.ny, fluid = flat_fluid(in.nx, in.ny, ctx->bc);
-                const int64_t end = part == 0 ? fluid : n;
-                for (int64_t k = part == 0 ? 0 : fluid; k < end; k += ctx->flat_nodes)
-                    t.push_back({(int32_t)i, (int32_t)k,
-                                 (int32_t)std::min<int64_t>(k + ctx->flat_nodes, end), 0});
-            }
+        // flat_nodes consecutive (fluid) nodes per entry
+        for (int i = 0; i < ctx->count; ++i) {
+            const InstDesc& in = ctx->layout.inst[i];
+            const int64_t n = flat_fluid(in.nx, in.ny, ctx->bc);
+            for (int64_t k = 0; k < n; k += ctx->flat_nodes)
+                t.push_back({(int32_t)i, (int32_t)k, (int32_t)std::min<int64_t>(k + ctx->flat_nodes, n), 0});
+        }
         return t;
     }
     for (int i = 0; i < ctx->count; ++i) {
@@ -393,6 +388,15 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
                            cudaMemcpyHostToDevice, ctx->stream));
     LBM_CK(cudaStreamSynchronize(ctx->stream));
     const int block = block_threads(ctx, s);
+    if (is_flat(ctx, s)) {
+        // An SM takes as many CTAs as it has room for, so a grid of a few
+        // CTAs per SM is dealt unevenly: claim the shared memory that leaves
+        // room for an equal share and no more.
+        const int64_t ctas = (int64_t)t.size() * (ctx->flat_nodes / block);
+        const int64_t share = (ctas + ctx->num_sms - 1) / ctx->num_sms;
+        if (share > 1 && share <= 32) smem = (size_t)(227 * 1024 / share - 1024) / 1024 * 1024;
+        LBM_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024));
+    }
     int per_sm = 0;
     LBM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
     per_sm = std::max(per_sm, 1);

@@ -143,11 +143,6 @@ struct StepArgs {
     int32_t halo;                // tube kernel: nodes carried along at either end of a segment
 };
 
-// Most threads of a CTA of the one-node-per-thread kernel.
-#ifndef FLAT_MAX_THREADS
-#define FLAT_MAX_THREADS 32
-#endif
-
 __host__ __device__ inline int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }
 
 // Programmatic dependent launch between consecutive step kernels: a step

@@ -15,7 +15,7 @@ namespace lbm {
 // ---------------------------------------------------------------------------
 // Natural logarithm, table driven (P. T. P. Tang, "Table-driven
 // implementation of the logarithm function in IEEE floating-point
-// arithmetic", ACM TOMS 16, 1990): for y = 1 + delta in [1/2, 2) the leading
+// arithmetic", ACM TOMS 16, 1990): for y = 1 + delta in [1/4, 4) the leading
 // 10 mantissa bits select a rational rc close to 1/y, then
 //     ln y = ln(1/rc) + ln(1 + r),  r = y rc - 1 = delta rc + (rc - 1),
 // |r| <= 2^-10, by the Taylor series to r^6 (remainder below 2^-62 of r).
@@ -24,7 +24,7 @@ namespace lbm {
 // have their bracket in FP32: its rounding is below 2^-56 of r.  rc and
 // rc - 1 have at most 12 significant bits, so that their high words alone
 // are stored.  6 FP64 instructions and one 16-byte table read, where the
-// library's log1p takes about 25.  Outside [1/2, 2): log1p.
+// library's log1p takes about 25.
 // ---------------------------------------------------------------------------
 constexpr int LOG_BITS = 10, LOG_HALF = 1 << LOG_BITS;  // intervals of an octave
 struct alignas(16) LogEntry {
@@ -32,7 +32,7 @@ struct alignas(16) LogEntry {
     uint32_t rc, rm;     // high words of rc and rc - 1 (low words are 0)
 };
 struct LogTable {
-    LogEntry e[2 * LOG_HALF];  // first half: y in [1/2, 1), second: y in [1, 2)
+    LogEntry e[4 * LOG_HALF];  // octaves [1/4, 1/2), [1/2, 1), [1, 2), [2, 4) of y
 };
 
 // High word of j / 2^sh as a double (|j| < 2^20).
@@ -73,26 +73,21 @@ constexpr LogTable make_log_table() {
         const double c = 1.0 + (i + 0.5) / H;  // centre of the interval of m, y = m or m / 2
         int j = (int)(2.0 * H / c + 0.5);
         if (i == 0) j = 2 * H;  // rc = 1 right of y = 1 (and, with j = H for i = H - 1, left of it)
-        LogEntry& u = t.e[H + i];
-        u.lc = hi[j - H] + lo[j - H];
-        u.rc = ratio_high_word(j, LOG_BITS + 1);
-        u.rm = ratio_high_word(j - 2 * H, LOG_BITS + 1);
-        LogEntry& v = t.e[i];
-        v.lc = (hi[j - H] - hi[0]) + (lo[j - H] - lo[0]);
-        v.rc = ratio_high_word(j, LOG_BITS);
-        v.rm = ratio_high_word(j - H, LOG_BITS);
+        for (int o = 0; o < 4; ++o) {  // y = 2^k m, k = o - 2
+            const int k = o - 2;
+            LogEntry& u = t.e[o * H + i];
+            u.lc = (hi[j - H] + k * hi[0]) + (lo[j - H] + k * lo[0]);
+            u.rc = ratio_high_word(j, LOG_BITS + 1 + k);
+            u.rm = ratio_high_word(j - (k >= 0 ? (2 * H) << k : (2 * H) >> -k), LOG_BITS + 1 + k);
+        }
     }
     return t;
 }
 
 static __device__ const LogTable LOG_TABLE = make_log_table();
 
-__device__ __noinline__ static double log1p_slow(double delta) { return log1p(delta); }
-
-// ln(1 + delta), given delta and y = 1 + delta rounded
-__device__ __forceinline__ double log1p_f64(double delta, double y) {
-    const uint32_t i = ((uint32_t)__double2hiint(y) - 0x3fe00000u) >> (20 - LOG_BITS);
-    if (i >= 2u * LOG_HALF) return log1p_slow(delta);
+// ln(1/rc) + ln(1 + r) of table entry i, for the deviation of a y in its interval
+__device__ __forceinline__ double log_entry(uint32_t i, double delta) {
     const int4 e = __ldg(reinterpret_cast<const int4*>(&LOG_TABLE.e[i]));
     const double r = fma(delta, __hiloint2double(e.z, 0), __hiloint2double(e.w, 0));
     // r in FP32 from its high word (2^-20 relative): the upper exponent bits
@@ -105,6 +100,23 @@ __device__ __forceinline__ double log1p_f64(double delta, double y) {
     const double t = __hiloint2double((int)((tb >> 3) + 0x38000000u), (int)(tb << 29));
     const double q = fma(r, fma(-r, t, 1.0 / 3.0), -0.5);
     return __hiloint2double(e.y, e.x) + fma(r * r, q, r);
+}
+
+// Outside [1/4, 4): y = 2^k m, ln m by the table from m - 1, plus k ln 2.  Not
+// inlined: FP64 instructions hold the pipe even where their predicate is off.
+__device__ __noinline__ static double log1p_outside(double delta, double y) {
+    const uint32_t yh = (uint32_t)__double2hiint(y);
+    if (yh - 0x00100000u >= 0x7fe00000u) return log1p(delta);  // not positive and normal
+    const double m = __hiloint2double((int)((yh & 0xfffffu) | 0x3ff00000u), __double2loint(y));
+    const uint32_t i = 2u * LOG_HALF + ((yh >> (20 - LOG_BITS)) & (LOG_HALF - 1u));
+    return fma((double)((int)(yh >> 20) - 1023), 0.6931471805599453, log_entry(i, m - 1.0));
+}
+
+// ln(1 + delta), given delta and y = 1 + delta rounded
+__device__ __forceinline__ double log1p_f64(double delta, double y) {
+    const uint32_t i = ((uint32_t)__double2hiint(y) - 0x3fd00000u) >> (20 - LOG_BITS);
+    if (i >= 4u * LOG_HALF) return log1p_outside(delta, y);
+    return log_entry(i, delta);
 }
 
 // ---------------------------------------------------------------------------

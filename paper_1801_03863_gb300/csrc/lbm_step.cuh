@@ -320,101 +320,132 @@ __global__ void __launch_bounds__(256) step_kernel(const StepArgs args) {
 // instruction holds its scheduler's FP64 unit for 64 cycles, whatever the
 // number of active lanes, so what counts is that every scheduler gets the
 // same number of full warps, down to the smallest lattices.  Nodes are
-// numbered linearly, without tile padding; in a cavity the fluid nodes come
-// first and the outer ring (walls and lid, which do not collide) after them,
-// and the tile table lists the ring entries of all instances behind the
-// fluid ones, so that the colliding CTAs go to the SMs in turn.  An entry
-// covers up to args.tw nodes, [cx0, y0) of one instance in that numbering,
-// and args.tw / blockDim.x CTAs.  CTAs are single warps: with 64 or 128
-// threads whole CTAs are dealt to the SMs and the last round fills worse
-// (257 x 257: 42.6 us a step with one warp, 52.8 with two or four; 17 x 17
-// lattices alike within 1 %).
+// numbered linearly, without tile padding; in a cavity only the fluid nodes
+// are, and every CTA takes an equal share of the outer ring (walls and lid,
+// which do not collide) along.  A CTA is one warp; an entry of the tile table
+// covers up to args.tw nodes, [cx0, y0) of one instance, and args.tw / 32 CTAs.
+// (42.6 us a step on 257 x 257 with one warp per CTA against 52.8 with two or
+// four, ring nodes in colliding warps.)
+//
+// The hardware deals CTAs to SMs unevenly while some still have room, so the
+// launch claims shared memory that leaves each SM room for its equal share
+// and no more (257 x 257: 37.2 -> 34.2 us a step; at most 128 registers, so
+// that 16 warps fit an SM: with more, 38.9).
 //
 // Measured, MinxEnt4, per step, against the register-chunk kernel with log1p
-// and IEEE divisions: 120 lattices of 17 x 17: 122.5 -> 18.9 us; 257 x 257:
-// 110 -> 37.1 us; 800 x 4: 50 -> 12-16 us; 2048 x 2048: 3680 -> 1903 us (250
-// FP64 instructions per node against 485; 0.88 of the FP64 issue rate).
+// and IEEE divisions: 120 lattices of 17 x 17: 122.5 -> 18.7 us; 257 x 257:
+// 110 -> 34.2 us; 800 x 4: 50 -> 10.7 us; 2048 x 2048: 3680 -> 1900 us (250
+// FP64 instructions per node against 485; 0.88 of the FP64 issue rate).  The
+// smallest lattices are bound by one warp's instructions (250 x 64 cycles =
+// 7.7 us) and the launch.
 //
 // inplace: the first step after a state was loaded collides f(x, t_n) itself,
 // without streaming.
 // ---------------------------------------------------------------------------
+// Populations a cavity's or another lattice's node (x, y) pulls (or holds, inplace).
+__device__ __forceinline__ void flat_pull(const double* base, const InstDesc& in, uint32_t x, uint32_t y,
+                                          bool inplace, double (&d)[9]) {
+    const int64_t pitch = in.pitch, plane = in.plane;
+    if (inplace) {
+        const double* p = base + (int64_t)y * pitch + x;
+#pragma unroll
+        for (int a = 0; a < 9; ++a) d[a] = p[a * plane];
+        return;
+    }
+    // columns x - 1, x + 1 and rows y - 1, y + 1 under the boundary rule;
+    // a cavity node pulls deviation 0 from outside the lattice
+    const uint32_t nx = (uint32_t)in.nx, ny = (uint32_t)in.ny;
+    const bool cav = in.bc == BC_CAVITY, per = in.bc == BC_PERIODIC;
+    const bool l = x > 0u, r = x + 1u < nx, b = y > 0u, t = y + 1u < ny;
+    const uint32_t xs[3] = {l ? x - 1u : (per ? nx - 1u : 0u), x, r ? x + 1u : (per ? 0u : nx - 1u)};
+    const uint32_t ys[3] = {b ? y - 1u : ny - 1u, y, t ? y + 1u : 0u};
+    const bool xok[3] = {l || !cav, true, r || !cav}, yok[3] = {b || !cav, true, t || !cav};
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+        const int i = 1 - D2Q9::vx(a), j = 1 - D2Q9::vy(a);
+        d[a] = (xok[i] && yok[j]) ? __ldg(base + a * plane + (int64_t)ys[j] * pitch + xs[i]) : 0.0;
+    }
+}
+
+// Node j of a cavity's ring: bottom row, top row, then the two sides, row by row.
+__device__ __forceinline__ void ring_node(uint32_t j, uint32_t nx, uint32_t ny, uint32_t& x, uint32_t& y) {
+    if (j < 2u * nx) {
+        y = j < nx ? 0u : ny - 1u;
+        x = j < nx ? j : j - nx;
+    } else {
+        const uint32_t s = j - 2u * nx;
+        y = 1u + (s >> 1);
+        x = (s & 1u) ? nx - 1u : 0u;
+    }
+}
+
 template <int COLL>
-__global__ void __launch_bounds__(FLAT_MAX_THREADS) step_flat_kernel(const StepArgs args) {
+__global__ void __launch_bounds__(32, 16) step_flat_kernel(const StepArgs args) {
     constexpr int Q = 9;
-    const double* __restrict__ src = static_cast<const double*>(args.src);
+    const double* src = static_cast<const double*>(args.src);
     double* __restrict__ dst = static_cast<double*>(args.dst);
-    const uint32_t per = (uint32_t)args.tw / blockDim.x;  // CTAs per entry, a power of two
+    const uint32_t per = (uint32_t)args.tw / 32u, sub = blockIdx.x & (per - 1u);  // CTAs per entry: 2^n
+    const uint32_t lane = threadIdx.x;
     const TileDesc tile = args.tiles[blockIdx.x / per];
     const InstDesc& in = args.inst[tile.inst];
     const uint32_t nx = (uint32_t)in.nx, ny = (uint32_t)in.ny;
-    const int bc = in.bc;
-    const uint32_t k = (uint32_t)tile.cx0 + (blockIdx.x & (per - 1u)) * blockDim.x + threadIdx.x;
+    const bool cav = in.bc == BC_CAVITY;
+    const uint32_t k = (uint32_t)tile.cx0 + sub * 32u + lane;
     const bool active = k < (uint32_t)tile.y0;
-    uint32_t x, y;
-    bool ring = false;
-    if (bc == BC_CAVITY) {
-        const uint32_t mx = nx - 2u, fluid = mx * (ny - 2u);
-        if (k < fluid) {
-            const uint32_t r = k / mx;
-            y = 1u + r;
-            x = 1u + k - r * mx;
-        } else {
-            // ring: bottom row, top row, then the two sides, row by row
-            const uint32_t j = k - fluid;
-            ring = true;
-            if (j < 2u * nx) {
-                y = j < nx ? 0u : ny - 1u;
-                x = j < nx ? j : j - nx;
-            } else {
-                const uint32_t s = j - 2u * nx;
-                y = 1u + (s >> 1);
-                x = (s & 1u) ? nx - 1u : 0u;
-            }
-        }
-    } else {
-        y = k / nx;
-        x = k - y * nx;
+    const uint32_t mx = cav ? nx - 2u : nx;
+    const uint32_t row = k / mx;
+    const uint32_t x = k - row * mx + (cav ? 1u : 0u), y = row + (cav ? 1u : 0u);
+    // this CTA's share of the cavity's ring
+    uint32_t ring = 0u, ring_end = 0u;
+    if (cav) {
+        const uint32_t fluid = mx * (ny - 2u), all = 2u * (nx + ny) - 4u;
+        const uint64_t ctas = (uint64_t)((fluid + (uint32_t)args.tw - 1u) / (uint32_t)args.tw) * per;
+        const uint64_t me = (uint64_t)((uint32_t)tile.cx0 / (uint32_t)args.tw) * per + sub;
+        ring = (uint32_t)(me * all / ctas) + lane;
+        ring_end = (uint32_t)((me + 1u) * all / ctas);
     }
     wait_previous_grid();
     allow_next_grid();
-    if (!active) return;
 
-    const int64_t pitch = in.pitch, plane = in.plane;
     const double* base = src + in.off;
-    double d[Q];
-    if (args.inplace) {
-        const double* p = base + (int64_t)y * pitch + x;
+    double* obase = dst + in.off;
+    const bool inplace = args.inplace != 0;
+    double d[Q], rd[Q];
+    if (active) flat_pull(base, in, x, y, inplace, d);
+    // ring node: bounce-back of the pulled populations, or the lid's equilibrium;
+    // its loads are issued before the collision and stored after it
+    uint32_t rx = 0u, ry = 0u;
+    auto ring_load = [&]() {
+        ring_node(ring, nx, ny, rx, ry);
+        if (ry == ny - 1u && rx > 0u && rx < nx - 1u) {
 #pragma unroll
-        for (int a = 0; a < Q; ++a) d[a] = p[a * plane];
-    } else {
-        // columns x - 1, x + 1 and rows y - 1, y + 1 under the boundary rule;
-        // a cavity node pulls deviation 0 from outside the lattice
-        const bool cav = bc == BC_CAVITY;
-        const bool l = x > 0u, r = x + 1u < nx, b = y > 0u, t = y + 1u < ny;
-        const uint32_t wrap_l = bc == BC_PERIODIC ? nx - 1u : 0u, wrap_r = bc == BC_PERIODIC ? 0u : nx - 1u;
-        const uint32_t xs[3] = {l ? x - 1u : wrap_l, x, r ? x + 1u : wrap_r};
-        const uint32_t ys[3] = {b ? y - 1u : ny - 1u, y, t ? y + 1u : 0u};
-        const bool xok[3] = {l || !cav, true, r || !cav}, yok[3] = {b || !cav, true, t || !cav};
-#pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            const int i = 1 - D2Q9::vx(a), j = 1 - D2Q9::vy(a);
-            d[a] = (xok[i] && yok[j]) ? __ldg(base + a * plane + (int64_t)ys[j] * pitch + xs[i]) : 0.0;
+            for (int a = 0; a < Q; ++a) rd[D2Q9::opp(a)] = in.lid_dev[a];
+        } else {
+            flat_pull(base, in, rx, ry, inplace, rd);
         }
-    }
-    double o[Q];
-    double* op = dst + in.off + (int64_t)y * pitch + x;
-    if (ring) {
-        const bool lid = y == ny - 1u && x > 0u && x < nx - 1u;
+    };
+    auto ring_store = [&]() {
+        double* p = obase + (int64_t)ry * in.pitch + rx;
 #pragma unroll
-        for (int a = 0; a < Q; ++a) op[a * plane] = lid ? in.lid_dev[a] : d[D2Q9::opp(a)];
-        return;
-    }
-    const Rates<double> rates{in.omega, in.omega2, in.s_e, in.s_eps};
-    const uint32_t st = Collide<D2Q9, COLL, double, 8>::run(d, args.rho0, rates, o);
+        for (int a = 0; a < Q; ++a) p[a * in.plane] = rd[D2Q9::opp(a)];
+    };
+    const bool first = ring < ring_end;
+    if (first) ring_load();
+    if (active) {
+        double o[Q];
+        const Rates<double> rates{in.omega, in.omega2, in.s_e, in.s_eps};
+        const uint32_t st = Collide<D2Q9, COLL, double, 8>::run(d, args.rho0, rates, o);
+        double* op = obase + (int64_t)y * in.pitch + x;
 #pragma unroll
-    for (int a = 0; a < Q; ++a) op[a * plane] = o[a];
-    if (st & ST_NEWTON_SKIPPED) atomicAdd(args.status + 2 * tile.inst + 0, 1ull);
-    if (st & ST_UNSTABLE) atomicAdd(args.status + 2 * tile.inst + 1, 1ull);
+        for (int a = 0; a < Q; ++a) op[a * in.plane] = o[a];
+        if (st & ST_NEWTON_SKIPPED) atomicAdd(args.status + 2 * tile.inst + 0, 1ull);
+        if (st & ST_UNSTABLE) atomicAdd(args.status + 2 * tile.inst + 1, 1ull);
+    }
+    if (first) ring_store();
+    for (ring += 32u; ring < ring_end; ring += 32u) {  // thin cavities: more ring than fluid
+        ring_load();
+        ring_store();
+    }
 }
 
 inline const void* pick_step_flat_kernel(int collision) {

@@ -60,3 +60,21 @@ def test_one_step_far_from_equilibrium(bc, rule):
     assert np.abs(f1 - sim.get_f()).max() <= 1e5 * 2.0 ** -53 * np.abs(f1).max()
     assert 0 < st["newton_skipped"] == co["newton_skipped"]
     assert st["unstable"] == co["unstable"]
+
+
+def test_thin_cavities_share_out_their_ring():
+    """More ring nodes than lanes of the colliding warps, and the smallest fluid regions."""
+    dims = [(3, 90), (90, 3), (4, 4), (3, 3), (200, 4)]
+    nus, uls = [0.02, 0.03, 0.04, 0.05, 0.02], [0.05, 0.06, 0.07, 0.08, 0.09]
+    with lbm.Lattice("d2q9", dims, nus, "cavity", u_lid=uls) as lat:
+        lat.init(np.ones(sum(a * b for a, b in dims)))
+        lat.step(25)
+        f = lat.populations()
+    k = 0
+    for (nx, ny), nu, ul in zip(dims, nus, uls):
+        sim = oracle.Sim(oracle.D2Q9, nx, ny, oracle.tau_from_nu(nu), oracle.BC_CAVITY, u_lid=ul)
+        sim.init(np.ones((ny, nx)), np.zeros((ny, nx)), np.zeros((ny, nx)))
+        sim.step(25)
+        g = f[k:k + 9 * nx * ny].reshape(9, ny, nx)
+        assert np.abs(g - sim.get_f()).max() <= 1e-12 * np.abs(g).max()
+        k += 9 * nx * ny
