@@ -168,7 +168,8 @@ int lbm_init_batch(lbm_ctx* ctx, int32_t instance, const double* rho, const doub
                    const double* uy);
 
 /* Advance every instance by n >= 0 time steps (Eq. 2).  Asynchronous on the
- * context's stream; runs of 16 or more steps replay CUDA graphs of 16
+ * context's stream.  D1Q3 and small D2Q9 lattices take several steps per
+ * launch; elsewhere runs of 16 or more steps replay CUDA graphs of 16
  * launches, captured and uploaded when the context is created. */
 int lbm_step(lbm_ctx* ctx, int64_t n);
 
@@ -275,32 +276,36 @@ int lbm_conservation_noalloc(lbm_ctx* ctx, double* out);
 int lbm_status(lbm_ctx* ctx, int64_t* counters);
 int lbm_status_instance(lbm_ctx* ctx, int32_t instance, int64_t* counters);
 
-/* Launch shape in use: out[0] = nodes per thread (1 on D2Q9: the FP64 kernel
- * with one node per thread, warps of 32 consecutive nodes, tw = 32, th = 1;
- * on D1Q3 nodes per lane of the tube kernel, tw x th = threads of a CTA, both
- * following from the sizes), out[1] = tile width in thread chunks, out[2] = tile height in rows, out[3] = grid size (CTAs),
- * out[4] = kernel kind (0: register-chunk kernel; 1 to 4: the TMA-staged
- * D2Q9 kernel, whose CTAs have one warp that only moves tiles in and out
- * besides the colliding warps.  1: large tiles, 8-warp CTAs, 1792 nodes for
- * 2-byte storage or 896 for FP32, two-stage ring; 2: small tiles, 8-warp
- * CTAs, 896 / 448 nodes, three-stage ring; 3: 10-warp CTAs, 2304 / 1152
- * nodes, two-stage ring; 4: deep ring, one 16-warp CTA per SM, 1920 / 960
- * nodes, five stages (four for FP32 storage).  For kinds 1
- * to 4 the tile width is 64/128/256 nodes chosen per instance (at most
- * 32 tile nodes / colliding threads; of those, for the MinxEnt rules the
- * one whose tiles cover the instance with the fewest padding nodes, for the
- * others the widest) and out[1], out[2] are 0;
- * tiles go in and out of
- * shared memory by TMA).  Selection: the create-time
- * autotuner (each candidate shape timed over back-to-back launches, the
- * candidates within 5 % of the fastest timed again as a captured graph,
- * which decides; the choice
- * is cached per device, lattice, types, rule, boundary and instance sizes
- * for the life of the process, and in the text file named by the
- * environment variable LBM_AUTOTUNE_CACHE when set, which later processes
- * reuse without timing), or the environment variable LBM_SHAPE = "V,tw,th"
- * (register chunks), "smem" (kind 1), "smems" (kind 2), "smemw" (kind 3) or
- * "smemd" (kind 4). */
+/* Launch shape in use: out[0] = nodes per thread, out[1] = tile width in
+ * thread chunks, out[2] = tile height in rows, out[3] = grid size (CTAs),
+ * out[4] = kernel kind:
+ *  0  D2Q9: register-chunk kernel; with out[0] = 1 the FP64 kernel with one
+ *     node per thread (warps of 32 consecutive nodes, tw = 32, th = 1).
+ *     D1Q3: the tube kernel, out[0] nodes per lane, tw x th threads a CTA,
+ *     several steps per launch; both follow from the sizes.
+ *  1 to 4  the TMA-staged D2Q9 kernel, whose CTAs have one warp that only
+ *     moves tiles in and out of shared memory besides the colliding warps.
+ *     1: large tiles, 8-warp CTAs, 1792 nodes for 2-byte storage or 896 for
+ *     FP32, two-stage ring; 2: small tiles, 8-warp CTAs, 896 / 448 nodes,
+ *     three-stage ring; 3: 10-warp CTAs, 2304 / 1152 nodes, two-stage ring;
+ *     4: deep ring, one 16-warp CTA per SM, 1920 / 960 nodes, five stages
+ *     (four for FP32 storage).  The tile width is 64/128/256 nodes chosen
+ *     per instance (at most 32 tile nodes / colliding threads; of those, for
+ *     the MinxEnt rules the one whose tiles cover the instance with the
+ *     fewest padding nodes, for the others the widest) and out[1], out[2]
+ *     are 0.
+ *  5  overlapping regions of 64 columns by th rows that take tw steps per
+ *     launch in shared memory (D2Q9 with FP32 arithmetic; lattices that do
+ *     not fill the GPU).
+ * Selection: the create-time autotuner (D2Q9 with FP32 arithmetic: each
+ * candidate shape timed over back-to-back launches, the close ones timed
+ * again as a captured graph, which decides; the choice is cached per device,
+ * lattice, types, rule, boundary and instance sizes for the life of the
+ * process, and in the text file named by the environment variable
+ * LBM_AUTOTUNE_CACHE when set, which later processes reuse without timing),
+ * or the environment variable LBM_SHAPE = "V,tw,th" (kind 0), "smem" (kind
+ * 1), "smems" (kind 2), "smemw" (kind 3), "smemd" (kind 4) or "block,tw,th"
+ * (kind 5). */
 int lbm_launch_shape(lbm_ctx* ctx, int32_t* out);
 
 /* Destroy a context (NULL-safe).  Frees library-owned memory only. */

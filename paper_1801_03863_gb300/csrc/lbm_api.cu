@@ -17,6 +17,7 @@
 
 #include "../../include/lbm.h"
 #include "lbm_aux.h"
+#include "lbm_step_block.cuh"
 
 using namespace lbm;
 
@@ -25,6 +26,7 @@ namespace {
 constexpr int64_t ROW_ALIGN = 8;       // row pitch multiple (nodes)
 constexpr int64_t PLANE_ALIGN = 128;   // plane / instance alignment (elements)
 constexpr int GRAPH_STEPS = 16;        // steps per captured graph (even)
+constexpr int BLOCK_WHOLE_STEPS = 32;  // steps per launch on uncut regions
 
 size_t dtype_bytes(int dt) { return dt == DT_F64 ? 8 : (dt == DT_F32 ? 4 : 2); }
 
@@ -32,12 +34,16 @@ size_t dtype_bytes(int dt) { return dt == DT_F64 ? 8 : (dt == DT_F32 ? 4 : 2); }
 // tw x th chunks); kind 1 / 2 / 3 / 4: TMA-staged D2Q9 kernel with node
 // pairs (V = 2) in the large-tile / small-tile / wide-CTA / deep-ring
 // geometry (smem_tile_nodes variant kind - 1), tile width per instance.
+// Kind 5: overlapping regions (lbm_step_block.cuh), tw steps per launch on
+// regions of th rows.
 // Kind 0 with V = 1 on D2Q9 is the FP64 kernel with one node per thread
 // (warps of 32 consecutive nodes: tw = 32, th = 1).  On D1Q3 kind 0 is the
 // tube kernel: V nodes per lane, tw x th threads per CTA.
 struct Shape {
     int V, tw, th;
     int kind = 0;
+    bool tma() const { return kind >= 1 && kind <= 4; }
+    bool block() const { return kind == 5; }
 };
 
 Shape default_shape_d2q9(int storage) {
@@ -187,7 +193,8 @@ struct lbm_ctx {
     int64_t steps = 0;
     Shape shape{};
     int flat_nodes = 0;  // one-node-per-thread kernel: nodes per tile-table entry
-    int halo = 0;        // tube kernel: halo nodes of a segment, steps per launch
+    int halo = 0;         // tube and region kernels: halo nodes, steps per launch
+    int block_warps = 0;  // region kernel: warps of a CTA
     const void* kern = nullptr;
     int grid = 0;
     size_t smem = 0;  // dynamic shared memory of the step kernel
@@ -260,7 +267,8 @@ bool is_flat(const lbm_ctx* ctx, const Shape& s) {
     return ctx->lattice == 2 && s.kind == 0 && s.V == 1;
 }
 int block_threads(const lbm_ctx* ctx, const Shape& s) {
-    if (s.kind >= 1) return smem_block_threads(s.kind - 1);
+    if (s.tma()) return smem_block_threads(s.kind - 1);
+    if (s.block()) return 32 * ctx->block_warps;
     if (ctx->lattice == 1) return std::max(32, std::min(s.tw * s.th, 256) / 32 * 32);
     return is_flat(ctx, s) ? 32 : s.tw * s.th;
 }
@@ -311,8 +319,72 @@ void tube_plan(const lbm_ctx* ctx, int V_pinned, int* V, int* halo) {
     }
 }
 
+// Regions of the kernel of lbm_step_block.cuh with K steps per launch and
+// regions of `rows` rows: their number, and the table (t may be null).  An
+// instance that fits a region along an axis with boundary rules of its own at
+// both ends is not cut there; *whole = no instance is cut at all, so that the
+// steps of a launch are not limited by the overlap.
+int64_t block_tiles(const lbm_ctx* ctx, int K, int rows, bool* whole, std::vector<TileDesc>* t) {
+    int64_t n = 0;
+    *whole = true;
+    for (int i = 0; i < ctx->count; ++i) {
+        const InstDesc& in = ctx->layout.inst[i];
+        const bool wide = ctx->bc == LBM_BC_PERIODIC || in.nx > BLOCK_COLS;
+        const bool high = ctx->bc != LBM_BC_CAVITY || in.ny > rows;
+        *whole = *whole && !wide && !high;
+        const int U = wide ? BLOCK_COLS - 2 * K : BLOCK_COLS, V = high ? rows - 2 * K : rows;
+        n += (int64_t)((in.nx + U - 1) / U) * ((in.ny + V - 1) / V);
+        if (!t) continue;
+        const int hx = wide ? K : 0, hy = high ? K : 0;
+        for (int y = 0; y < in.ny; y += V)
+            for (int x = 0; x < in.nx; x += U)
+                t->push_back({(int32_t)i, x - hx, y - hy,
+                              pack_part(hx, hx + std::min(U, in.nx - x), hy, hy + std::min(V, in.ny - y), !high)});
+    }
+    return n;
+}
+
+// Steps per launch and region height of a context, or false where the
+// regions are too many for this kernel to be ahead of the TMA kernel (more
+// than four per SM).  The modelled time per step, in us: a row of a region
+// holds its scheduler for `unit` (16 warps take 16 rows at a time), a launch
+// adds a region's loads and stores and the launch itself.  The constants fit
+// 512 x 512, 64 x 64, 200 x 200 and 17 x 17 lattices with K = 2 .. 8 and 12 ..
+// 64 rows within 15 %; whether the TMA kernel is ahead is timed.
+bool block_plan(const lbm_ctx* ctx, int* K, int* rows) {
+    const int cap = block_max_rows(ctx->storage);
+    const double unit = ctx->collision == LBM_MINXENT4 ? 0.41 : 0.28;
+    double best = 1e30;
+    auto consider = [&](int r, int steps, double live, int64_t n) {
+        const double turns = std::ceil(live / BLOCK_WARPS);
+        const double units = std::max(std::ceil(live / 4), turns > 1 ? 4 * (turns - 1) + 2.4 : 0.0);
+        const double rounds = std::ceil((double)n / ctx->num_sms);
+        const double t = rounds * (units * unit + 0.15 + 2.5 / steps) + 2.0 / steps;
+        if (n <= 4 * ctx->num_sms && n <= ctx->layout.max_tiles && t < best) {
+            best = t;
+            *K = steps;
+            *rows = r;
+        }
+    };
+    bool whole;
+    const int tall = (int)std::min<int64_t>(ctx->layout.max_ny, cap);
+    const int64_t n = block_tiles(ctx, 0, tall, &whole, nullptr);
+    if (whole) consider(tall, BLOCK_WHOLE_STEPS, tall, n);
+    for (int k = 2; k <= 8; k += 2)
+        for (int r = 2 * k + 1; r <= cap; ++r) {
+            const int64_t cut = block_tiles(ctx, k, r, &whole, nullptr);
+            if (!whole) consider(r, k, r - k - 1, cut);  // (rows computed, on average)
+        }
+    return best < 1e30;
+}
+
 std::vector<TileDesc> build_tiles(const lbm_ctx* ctx, const Shape& s) {
     std::vector<TileDesc> t;
+    if (s.block()) {
+        bool whole;
+        block_tiles(ctx, s.tw, s.th, &whole, &t);
+        return t;
+    }
     if (s.kind >= 1) {
         for (int i = 0; i < ctx->count; ++i) {
             const InstDesc& in = ctx->layout.inst[i];
@@ -364,7 +436,21 @@ int build_tensor_maps(lbm_ctx* ctx, int variant);
 int apply_shape(lbm_ctx* ctx, const Shape& s) {
     const void* k = nullptr;
     size_t smem = 0;
-    if (s.kind >= 1) {
+    if (s.block()) {
+        if (ctx->lattice != 2 || ctx->compute != DT_F32) return LBM_ERR_ARG;
+        bool whole;
+        if (s.th < 1 || s.th > block_max_rows(ctx->storage) || s.tw < 1 || s.tw > 64) return LBM_ERR_ARG;
+        const bool cut = s.tw % 2 == 0 && 2 * s.tw < std::min(s.th, BLOCK_COLS);  // halos fit, words stay aligned
+        block_tiles(ctx, cut ? s.tw : 0, s.th, &whole, nullptr);
+        if (!whole && !cut) return LBM_ERR_ARG;
+        if (ctx->storage == DT_F32) k = step_kernel_block_f32(ctx->collision, s.th);
+        else if (ctx->storage == DT_F16) k = step_kernel_block_f16(ctx->collision, s.th);
+        else if (ctx->storage == DT_BF16) k = step_kernel_block_bf16(ctx->collision, s.th);
+        if (!k) return LBM_ERR_ARG;
+        smem = block_smem_bytes(ctx->storage, s.th);
+        ctx->halo = s.tw;
+        LBM_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    } else if (s.kind >= 1) {
         if (ctx->lattice != 2 || ctx->compute != DT_F32 || s.kind > 4) return LBM_ERR_ARG;
         const int var = s.kind - 1;
         if (ctx->storage == DT_F32) k = step_kernel_smem_f32(ctx->collision, var, &smem);
@@ -387,6 +473,9 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
     LBM_CK(cudaMemcpyAsync(ctx->d_inst, ctx->layout.inst.data(), sizeof(InstDesc) * ctx->count,
                            cudaMemcpyHostToDevice, ctx->stream));
     LBM_CK(cudaStreamSynchronize(ctx->stream));
+    // two CTAs of 8 warps on an SM where there are more regions than SMs
+    if (s.block())
+        ctx->block_warps = (int64_t)t.size() > ctx->num_sms && 2 * smem <= 220 * 1024 ? BLOCK_WARPS / 2 : BLOCK_WARPS;
     const int block = block_threads(ctx, s);
     if (is_flat(ctx, s)) {
         // An SM takes as many CTAs as it has room for, so a grid of a few
@@ -400,7 +489,8 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
     int per_sm = 0;
     LBM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
     per_sm = std::max(per_sm, 1);
-    const int64_t g = ctx->lattice == 1 ? ((int64_t)t.size() * 32 + block - 1) / block
+    const int64_t g = s.block() ? (int64_t)t.size()
+                      : ctx->lattice == 1 ? ((int64_t)t.size() * 32 + block - 1) / block
                       : is_flat(ctx, s) ? (int64_t)t.size() * (ctx->flat_nodes / block)
                                         : std::min<int64_t>((int64_t)per_sm * ctx->num_sms, (int64_t)t.size());
     ctx->tiles.swap(t);
@@ -522,19 +612,20 @@ float time_current_shape(lbm_ctx* ctx, cudaEvent_t* ev) {
     // one warm-up launch, then twice three back-to-back launches (as the
     // step loop runs them: a launch's tail overlaps the next one's start);
     // the faster of the two, per launch
-    if (launch_step(ctx, 0, ctx->stream) != cudaSuccess) return -1.f;
+    const int steps = ctx->shape.block() ? ctx->halo : 1;  // of a launch
+    if (launch_step(ctx, 0, ctx->stream, false, steps) != cudaSuccess) return -1.f;
     int src = 1;
     float t[2];
     for (int r = 0; r < 2; ++r) {
         if (cudaEventRecord(ev[2 * r], ctx->stream) != cudaSuccess) return -1.f;
         for (int k = 0; k < 3; ++k, src ^= 1)
-            if (launch_step(ctx, src, ctx->stream) != cudaSuccess) return -1.f;
+            if (launch_step(ctx, src, ctx->stream, false, steps) != cudaSuccess) return -1.f;
         if (cudaEventRecord(ev[2 * r + 1], ctx->stream) != cudaSuccess) return -1.f;
     }
     if (cudaEventSynchronize(ev[3]) != cudaSuccess) return -1.f;
     for (int r = 0; r < 2; ++r)
         if (cudaEventElapsedTime(&t[r], ev[2 * r], ev[2 * r + 1]) != cudaSuccess) return -1.f;
-    return std::min(t[0], t[1]) / 3.f;
+    return std::min(t[0], t[1]) / (3.f * steps);
 }
 
 // The same timing through a captured graph of four launches, as the step
@@ -546,7 +637,9 @@ float time_current_shape_graph(lbm_ctx* ctx, cudaEvent_t* ev) {
     if (cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
         return -1.f;
     bool ok = true;
-    for (int k = 0; k < 4; ++k) ok = ok && launch_step(ctx, k & 1, ctx->capture_stream) == cudaSuccess;
+    const int steps = ctx->shape.block() ? ctx->halo : 1;
+    for (int k = 0; k < 4; ++k)
+        ok = ok && launch_step(ctx, k & 1, ctx->capture_stream, false, steps) == cudaSuccess;
     if (cudaStreamEndCapture(ctx->capture_stream, &graph) != cudaSuccess || !ok) return -1.f;
     cudaGraphExec_t g = nullptr;
     const cudaError_t e = cudaGraphInstantiate(&g, graph, 0);
@@ -562,7 +655,7 @@ float time_current_shape_graph(lbm_ctx* ctx, cudaEvent_t* ev) {
     for (int r = 0; r < 2 && ok; ++r)
         ok = cudaEventElapsedTime(&t[r], ev[2 * r], ev[2 * r + 1]) == cudaSuccess;
     cudaGraphExecDestroy(g);
-    return ok ? std::min(t[0], t[1]) / 4.f : -1.f;
+    return ok ? std::min(t[0], t[1]) / (4.f * steps) : -1.f;
 }
 
 // Autotuner cache: the chosen shape per (device, lattice, types, rule,
@@ -595,7 +688,8 @@ std::string tune_key(const lbm_ctx* ctx) {
             h *= 1099511628211ull;
         }
     char buf[256];
-    snprintf(buf, sizeof buf, "%s/sm%d/lat%d/st%d/cp%d/co%d/bc%d/n%d/%016llx", name.c_str(),
+    // "k2": the set of kernels that were timed
+    snprintf(buf, sizeof buf, "%s/k2/sm%d/lat%d/st%d/cp%d/co%d/bc%d/n%d/%016llx", name.c_str(),
              ctx->num_sms, ctx->lattice, ctx->storage, ctx->compute, ctx->collision, ctx->bc,
              ctx->count, (unsigned long long)h);
     return buf;
@@ -648,6 +742,8 @@ int autotune(lbm_ctx* ctx) {
     Shape cached;
     if (tune_lookup(key, &cached) && apply_shape(ctx, cached) == LBM_OK) return LBM_OK;
     std::vector<Shape> cands = candidate_shapes(ctx->storage);
+    int K, rows;
+    if (ctx->storage != DT_F64 && block_plan(ctx, &K, &rows)) cands.push_back({2, K, rows, 5});
     if (cands.size() == 1) return apply_shape(ctx, cands[0]);
     cudaEvent_t ev[6];
     for (int i = 0; i < 6; ++i) LBM_CK(cudaEventCreate(&ev[i]));
@@ -667,10 +763,12 @@ int autotune(lbm_ctx* ctx) {
     }
     // The candidates within 5 % of the fastest are timed once more, after
     // the others, through a captured graph as the step loop runs them, and
-    // that time decides between them.
+    // that time decides between them.  Below 20 us a single launch is mostly
+    // launch (7.1 us where the graph takes 5.8), so there the margin is wider.
+    const float margin = best < 0.02f ? 1.6f : 1.05f;
     std::vector<float> tg(cands.size(), -1.f);
     for (size_t c = 0; c < cands.size() && rc == LBM_OK; ++c) {
-        if (t[c] < 0.f || t[c] > 1.05f * best) continue;
+        if (t[c] < 0.f || t[c] > margin * best) continue;
         if (apply_shape(ctx, cands[c]) != LBM_OK) continue;
         const float ms = time_current_shape_graph(ctx, ev);
         if (ms < 0.f) {
@@ -707,6 +805,7 @@ int autotune(lbm_ctx* ctx) {
 // upload the executable graphs, so that no capture or first-launch upload
 // happens inside a later lbm_step.
 int capture_graphs(lbm_ctx* ctx) {
+    if (ctx->shape.block()) return LBM_OK;  // several steps per launch: no graph
     for (int p = 0; p < 2; ++p) {
         cudaGraphExec_t& g = ctx->graph[p];
         if (g) continue;
@@ -749,8 +848,11 @@ bool parse_shape_env(Shape* s) {
         *s = {2, 0, 0, 4};
         return true;
     }
-
     int v, tw, th;
+    if (sscanf(e, "block,%d,%d", &tw, &th) == 2) {
+        *s = {2, tw, th, 5};
+        return true;
+    }
     if (sscanf(e, "%d,%d,%d", &v, &tw, &th) != 3) return false;
     *s = {v, tw, th};
     return true;
@@ -1140,6 +1242,13 @@ int lbm_step(lbm_ctx* ctx, int64_t n) {
         ctx->post = true;
         ctx->steps += 1;
         --n;
+    }
+    while (ctx->shape.block() && n > 0) {
+        const int k = (int)std::min<int64_t>(n, ctx->halo);
+        LBM_CK(launch_step(ctx, ctx->cur, ctx->stream, false, k));
+        ctx->cur = 1 - ctx->cur;
+        ctx->steps += k;
+        n -= k;
     }
     while (n >= GRAPH_STEPS) {
         cudaGraphExec_t& g = ctx->graph[ctx->cur];

@@ -62,6 +62,22 @@ const void* step_kernel_f32(int lattice, int collision, int V);
 const void* step_kernel_f16(int lattice, int collision, int V);
 const void* step_kernel_bf16(int lattice, int collision, int V);
 
+// D2Q9 step kernels that take several steps per launch on overlapping regions
+// (lbm_step_block.cuh; FP32 arithmetic): regions of 64 columns and at most
+// block_max_rows rows, CTAs of at most BLOCK_WARPS warps.
+const void* step_kernel_block_f32(int collision, int rows);
+const void* step_kernel_block_f16(int collision, int rows);
+const void* step_kernel_block_bf16(int collision, int rows);
+constexpr int BLOCK_WARPS = 16;
+constexpr int BLOCK_COLS = 64;
+// two buffers of nine planes of 64-node rows within 221 KB (storage 1: FP32)
+constexpr int block_max_rows(int storage) { return storage == 1 ? 48 : 96; }
+constexpr int BLOCK_SMALL_ROWS = 24;  // regions up to this height take buffers of it (two CTAs per SM)
+constexpr size_t block_smem_bytes(int storage, int rows) {
+    return (size_t)2 * 9 * BLOCK_COLS * (storage == 1 ? 4 : 2) *
+           (rows <= BLOCK_SMALL_ROWS ? BLOCK_SMALL_ROWS : block_max_rows(storage));
+}
+
 // D2Q9 step kernels with shared-memory tile staging (FP32 arithmetic); also
 // return the dynamic shared memory they need.
 const void* step_kernel_smem_f32(int collision, int variant, size_t* smem_bytes);

@@ -1,6 +1,7 @@
 // lbm_step_bf16.cu -- fused step kernels with __nv_bfloat16 storage and float arithmetic.
 #include "lbm_aux.h"
 #include "lbm_step.cuh"
+#include "lbm_step_block.cuh"
 #include "lbm_step_smem.cuh"
 
 namespace lbm {
@@ -14,6 +15,10 @@ const void* step_kernel_bf16(int lattice, int collision, int V) {
     if (V == 4) return pick_step_kernel<__nv_bfloat16, float, 4>(collision);
     if (V == 8) return pick_step_kernel<__nv_bfloat16, float, 8>(collision);
     return nullptr;
+}
+
+const void* step_kernel_block_bf16(int collision, int rows) {
+    return pick_step_block_kernel<__nv_bfloat16>(collision, rows);
 }
 
 const void* step_kernel_smem_bf16(int collision, int variant, size_t* smem_bytes) {

@@ -1,6 +1,7 @@
 // lbm_step_f32.cu -- fused step kernels with float storage and float arithmetic.
 #include "lbm_aux.h"
 #include "lbm_step.cuh"
+#include "lbm_step_block.cuh"
 #include "lbm_step_smem.cuh"
 
 namespace lbm {
@@ -15,6 +16,10 @@ const void* step_kernel_f32(int lattice, int collision, int V) {
     if (V == 2) return pick_step_kernel<float, float, 2>(collision);
     if (V == 4) return pick_step_kernel<float, float, 4>(collision);
     return nullptr;
+}
+
+const void* step_kernel_block_f32(int collision, int rows) {
+    return pick_step_block_kernel<float>(collision, rows);
 }
 
 const void* step_kernel_smem_f32(int collision, int variant, size_t* smem_bytes) {

@@ -257,7 +257,7 @@ def lbm_launch_shape(h) -> dict:
     _check(load().lbm_launch_shape(h, _p(c)), "lbm_launch_shape")
     return {"V": int(c[0]), "tw": int(c[1]), "th": int(c[2]), "grid": int(c[3]),
             "kind": {0: "chunks", 1: "smem", 2: "smem_small", 3: "smem_wide",
-                     4: "smem_deep"}[int(c[4])]}
+                     4: "smem_deep", 5: "block"}[int(c[4])]}
 
 
 def lbm_init_batch(h, instance: int, rho, ux=None, uy=None) -> None:
