@@ -16,8 +16,8 @@
 // 33.4 M nodes in 64 cavities, FP16: init 2.81 -> 0.28 ms (at rest; 1.1 GB,
 // 0.6 of the copy bandwidth), moments 2.26 -> 0.34 ms (FP64 issue: 6
 // instructions a node).  18.0 M nodes in 4096 tubes, FP32: init 0.78 -> 0.12,
-// moments 0.55 -> 0.32 ms.  12.2 M nodes D2Q9 FP32: moments 0.99 -> 0.52 ms
-// (22 FP64 instructions a node).
+// moments 0.55 -> 0.22 ms.  12.2 M nodes D2Q9 FP32: moments 0.99 -> 0.25 ms
+// (sums in fixed point: 6 FP64 instructions a node instead of 22).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -124,7 +124,7 @@ __device__ __forceinline__ void node_state(const S* src, const InstDesc& in, int
     }
 }
 
-// sum d, sum d v_x, sum d v_y in the number type V (float, F2 or double)
+// sum d, sum d v_x, sum d v_y in the number type V
 template <class Lat, typename V>
 __device__ __forceinline__ void moment_sums(const V (&d)[Lat::Q], V& m, V& jx, V& jy) {
     if constexpr (Lat::Q == 9) {
@@ -135,13 +135,59 @@ __device__ __forceinline__ void moment_sums(const V (&d)[Lat::Q], V& m, V& jx, V
     } else {
         m = d[0] + (d[1] + d[2]);
         jx = d[1] - d[2];
-        jy = V(0.f);
+        jy = V(0);
     }
+}
+
+// v 2^(e - 1023) rounded to FP64 (to nearest, ties to even), 64 < e < 1983
+__device__ __forceinline__ double fixed_to_f64(long long v, int e) {
+    const uint64_t sign = (uint64_t)v & 0x8000000000000000ull;
+    const uint64_t a = (uint64_t)(v < 0 ? -v : v);
+    if (a == 0u) return 0.0;
+    const int lz = __clzll((long long)a);
+    const uint64_t n = a << lz;  // leading bit at 63: it adds one to the exponent field below
+    const uint64_t up = ((n & 0x7ffu) + 0x3ffu + ((n >> 11) & 1u)) >> 11;
+    const uint64_t bits = sign | (((uint64_t)(e + 62 - lz) << 52) + (n >> 11) + up);
+    return __longlong_as_double((long long)bits);
+}
+
+// moment_sums of FP32 values in 64-bit fixed point, the largest value at bit
+// 58: what a smaller value loses below 2^-58 of it is less than the rounding
+// of FP64 additions, and the integer pipe does the work.  False where some
+// value is not finite or all are below 2^-80 (but zeros are fine).
+template <class Lat>
+__device__ __forceinline__ bool fixed_sums(const float (&d)[Lat::Q], double& m, double& jx, double& jy) {
+    uint32_t top = 0u;
+#pragma unroll
+    for (int a = 0; a < Lat::Q; ++a) top = max(top, __float_as_uint(d[a]) & 0x7fffffffu);
+    const int emax = (int)(top >> 23);
+    if (top == 0u) {
+        m = jx = jy = 0.0;
+        return true;
+    }
+    if (emax == 255 || emax < 47) return false;
+    long long v[Lat::Q];
+#pragma unroll
+    for (int a = 0; a < Lat::Q; ++a) {
+        const uint32_t b = __float_as_uint(d[a]);
+        const int e = max((int)((b >> 23) & 0xffu), 1), down = emax - e;
+        const uint32_t mant = (b & 0x7fffffu) | ((b & 0x7f800000u) ? 0x800000u : 0u);
+        const long long u = (long long)(((uint64_t)mant << 35) >> min(down, 63));
+        v[a] = (int)b < 0 ? -u : u;
+    }
+    long long im, ix, iy;
+    moment_sums<Lat, long long>(v, im, ix, iy);
+    // units of 2^(emax - 150 - 35)
+    const int e = 1023 + emax - 185;
+    m = fixed_to_f64(im, e);
+    jx = fixed_to_f64(ix, e);
+    jy = Lat::Q == 9 ? fixed_to_f64(iy, e) : 0.0;
+    return true;
 }
 
 // The same in FP64 from stored values.  FP16 values are multiples of 2^-24:
 // where all are below 1/16 in magnitude, their sums (below 1) are exact in
-// FP32.
+// FP32.  FP32 and BF16 values add in fixed point.
 template <class Lat, typename S>
 __device__ __forceinline__ void node_sums(const S (&raw)[Lat::Q], double& m, double& jx, double& jy) {
     if constexpr (std::is_same<S, __half>::value) {
@@ -159,6 +205,12 @@ __device__ __forceinline__ void node_sums(const S (&raw)[Lat::Q], double& m, dou
             jy = widen(fy);
             return;
         }
+    }
+    if constexpr (std::is_same<S, float>::value || std::is_same<S, __nv_bfloat16>::value) {
+        float d[Lat::Q];
+#pragma unroll
+        for (int a = 0; a < Lat::Q; ++a) d[a] = Store<S>::to_f32(raw[a]);
+        if (fixed_sums<Lat>(d, m, jx, jy)) return;
     }
     double d[Lat::Q];
 #pragma unroll

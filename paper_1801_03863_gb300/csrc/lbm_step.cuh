@@ -577,10 +577,11 @@ __global__ void __launch_bounds__(256) step_tube_kernel(const StepArgs args) {
         for (int p = 0; p < NP; ++p) {
             const CT d[3] = {f[0][p], from_l[p], from_r[p]};
             CT o[3];
-            const uint32_t st = Collide<D1Q3, COLL_MINXENT4, CT, (int)sizeof(S)>::run(d, rho0, rates, o);
+            const uint32_t bits = Collide<D1Q3, COLL_MINXENT4, CT, (int)sizeof(S)>::run(d, rho0, rates, o);
 #pragma unroll
             for (int a = 0; a < 3; ++a) f[a][p] = round_to_storage<CT, S>(o[a]);
-            if (st && mine) {  // rare: a population is negative or not finite
+            if (bgk_suspect(bits) && mine) {  // rare: a population is negative or not finite
+                const uint32_t st = bgk_status(o[0], o[1], o[2], rho0);
 #pragma unroll
                 for (int l = 0; l < P; ++l)
                     if (x + p + l * NP < nx) n_unst += ((st >> (2 * l)) & ST_UNSTABLE) >> 1;

@@ -122,3 +122,28 @@ def test_large_instance_splits_alike_alone_and_in_a_batch():
         two = lat.conservation()
     assert np.array_equal(one, two[0])
     assert abs(two[1, 0] - math.fsum(rho[1])) <= 1e-6 * 2100 * 2100 * 2.0 ** -10
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+def test_moments_over_the_whole_exponent_range(storage):
+    """Fixed-point sums of values of very different size, of vanishing ones and of none: rho, u against
+    exact sums of the stored deviations.  Each sum is within 2^-53 of the largest value (fixed point
+    keeps 2^-58 of it), and so is rho's rounding."""
+    rng = np.random.default_rng(8)
+    nx, ny = 64, 40
+    d = np.ldexp(rng.uniform(-1, 1, (9, ny, nx)), rng.integers(-60, -4, (9, ny, nx)))
+    d[:, :4] = 0.0
+    d[:, 4:8] = np.ldexp(rng.uniform(-1, 1, (9, 4, nx)), -100)
+    w = W9[:, None, None]
+    with lbm.Lattice("d2q9", [(nx, ny)], 0.1, "periodic", compute="f32", storage=storage) as lat:
+        # deviations survive the FP64 populations only down to 2^-53 W: read back what is stored
+        lat.set_populations(w + d)
+        g = lat.populations().reshape(9, ny, nx) - w
+        rho, ux, uy = (v.reshape(ny, nx) for v in lat.moments(allow_unstable=True))
+    vx = np.array([0, 1, 0, -1, 0, 1, -1, -1, 1])
+    vy = np.array([0, 0, 1, 0, -1, 1, 1, -1, -1])
+    m, jx, jy = (np.vectorize(lambda i, j: math.fsum(c * g[:, i, j]))(*np.mgrid[:ny, :nx])
+                 for c in (np.ones(9), vx, vy))
+    tol = 2.0 ** -52 * (1.0 + 9 * np.abs(g).max(0))
+    assert np.all(np.abs(rho - (1.0 + m)) <= tol)
+    assert np.all(np.abs(ux - jx / (1.0 + m)) <= 2 * tol) and np.all(np.abs(uy - jy / (1.0 + m)) <= 2 * tol)
