@@ -155,7 +155,7 @@ Carve carve(const Layout& L, int lattice, int storage, int count) {
     p += al(sizeof(double) * std::max<int64_t>(3 * L.total_nodes, Q * L.total_nodes));
     c.tmap_off = p;  // four TMA tensor maps per instance: [buffer][tile | halo]
     p += al(4 * sizeof(CUtensorMapOpaque) * count);
-    c.err_off = p;
+    c.err_off = p;  // error word and, from word 8 on, the TMA kernel's tile counters
     p += 256;
     c.total = p;
     return c;
@@ -574,6 +574,7 @@ StepArgs step_args(const lbm_ctx* ctx, int src) {
     a.tmaps_halo = ctx->d_tmaps + (size_t)(src * 2 + 1) * ctx->count;
     a.tmaps_dst = ctx->d_tmaps + (size_t)(1 - src) * 2 * ctx->count;
     a.error = ctx->d_error;
+    a.tile_counters = ctx->d_error + 8;
     a.spin_limit = ctx->spin_limit;
     a.lost_tile = ctx->lost_tile;
     a.inplace = 0;

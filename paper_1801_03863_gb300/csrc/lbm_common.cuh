@@ -135,6 +135,7 @@ struct StepArgs {
     const void* tmaps;           // TMA kernel only, per instance: tensor maps of src with
     const void* tmaps_halo;      // the tile box and with the halo box,
     const void* tmaps_dst;       // and of dst with the tile box (the stores)
+    unsigned int* tile_counters; // TMA kernel: tiles drawn and CTAs done (both 0 between launches)
     unsigned int* error;         // device error word (bounded waits that ran out)
     int32_t spin_limit;          // polls of one bounded mbarrier wait (TMA kernel)
     int32_t lost_tile;           // test hook: tile whose copies are never issued (-1: none)

@@ -4,7 +4,7 @@
 // Same time step as step_kernel (pull-stream + collide + boundary rules of
 // Sec. IV.F, Eq. 2), organised around the Tensor Memory Accelerator:
 //
-//  * A CTA walks the tile table of the context; a tile is X nodes (64, 128
+//  * The CTAs share out the tile table of the context; a tile is X nodes (64, 128
 //    or 256, chosen per instance) by R = TILE_NODES / X rows.  Four
 //    geometries are compiled (smem_tile_nodes): 8-warp CTAs with large or
 //    small tiles on two- or three-stage rings, 10-warp CTAs, and one
@@ -103,7 +103,7 @@ struct SmemTile {
 struct StageParams {
     InstDesc in;
     TileDesc next;  // descriptor of the tile this stage takes next (NS tiles later)
-    int32_t inst, X, x0, y0;
+    int32_t inst, X, x0, y0;  // X = 0: no further tile (drawn tiles)
 };
 static_assert(offsetof(StageParams, next) % 16 == 0 && sizeof(TileDesc) == 16,
               "the next-tile descriptor is a 16-byte bulk copy");
@@ -342,7 +342,16 @@ __global__ void __launch_bounds__(NTHREADS + 32, NTHREADS + 32 >= 512 ? 1 : LBM_
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const CT rho0v = CT((float)args.rho0);
     const int G = gridDim.x;
-    // local tile j of this CTA is global tile blockIdx.x + j * G
+    // This CTA's first NS tiles are blockIdx.x + j * G.  On a two-stage ring the
+    // further ones are drawn from a counter as stages become free; on deeper
+    // rings tile j is blockIdx.x + j * G throughout.  Dealt out beforehand, the
+    // SMs that take longer for their tiles hold up the end of every launch:
+    // FP32 MRT on 64 cavities 310 -> 272 us a step with drawn tiles, 48 ragged
+    // ones 149 -> 130, MinxEnt4 FP16 326 -> 311.  A deep ring evens that out by
+    // itself and its one copy warp per SM has no time for the draws (SRT FP16
+    // 144 -> 208 us).
+    constexpr bool DRAWS = NS == 2;
+    const bool draws = DRAWS && NS * G < args.ntiles;
     const int ntl = (args.ntiles > (int)blockIdx.x) ? (args.ntiles - 1 - (int)blockIdx.x) / G + 1 : 0;
 
     if (tid == 0) {
@@ -369,20 +378,21 @@ __global__ void __launch_bounds__(NTHREADS + 32, NTHREADS + 32 >= 512 ? 1 : LBM_
         bulk_commit();
     };
 
-    // Fill stage j % NS with local tile j (descriptor `tile`): store the
-    // tile's place, then issue the instance-descriptor, plane and halo
-    // copies, and the copy of the descriptor of tile j + NS (which this
-    // stage takes next), all on the stage's full barrier.
-    auto fill = [&](int j, const TileDesc tile) {
+    // Fill stage j % NS with local tile j (descriptor `tile`, number `index`):
+    // store the tile's place, then issue the instance-descriptor, plane and
+    // halo copies, and unless tiles are drawn the copy of the descriptor of
+    // tile j + NS (which this stage takes next), all on the stage's full
+    // barrier.
+    auto fill = [&](int j, const TileDesc tile, int index) {
         const int st = j % NS;
         *filled = j + 1;
         // test hook of the timeout path: the copies of one chosen tile are
         // never issued, so its full barrier never completes
-        if ((int)blockIdx.x + j * G == args.lost_tile) return;
+        if (index == args.lost_tile) return;
         StageParams& p = params[st];
         const int X = tile.pad, R = TS::TILE_NODES / X;
         p.inst = tile.inst; p.X = X; p.x0 = tile.cx0; p.y0 = tile.y0;
-        const bool more = j + NS < ntl;
+        const bool more = !draws && j + NS < ntl;
         const uint32_t bytes = (uint32_t)((Q * R * X + 6 * R * E) * sizeof(S) + sizeof(InstDesc) +
                                           (more ? sizeof(TileDesc) : 0));
         S* sbase = stage_base + (size_t)st * TS::STAGE_ELEMS;
@@ -419,22 +429,60 @@ __global__ void __launch_bounds__(NTHREADS + 32, NTHREADS + 32 >= 512 ? 1 : LBM_
         // tiles; then, once every colliding warp is done with tile j, write
         // it out and refill its stage with tile j + NS.
         if (lane == 0) {
-            for (int t = 0; t < min(NS, ntl); ++t) fill(t, args.tiles[blockIdx.x + t * G]);
+            for (int t = 0; t < min(NS, ntl); ++t)
+                fill(t, args.tiles[blockIdx.x + t * G], blockIdx.x + t * G);
+            // Drawn tiles: the next one, its descriptor, and the draw after it
+            // (used a tile later, so that its latency is not waited for).
+            const int dealt = NS * G;
+            int i1 = args.ntiles, nf = min(NS, ntl);
+            TileDesc d1{};
+            uint32_t ahead = 0u;
+            bool ended = !draws;
+            auto draw = [&]() { return atomicAdd(args.tile_counters, 1u); };
+            // No draws by this CTA any more: the last CTA to say so (the count
+            // wraps to 0 by itself) leaves the draws at 0 for the next launch.
+            auto end_draws = [&]() {
+                ended = true;
+                if (atomicInc(args.tile_counters + 1, (unsigned)G - 1u) == (unsigned)G - 1u)
+                    args.tile_counters[0] = 0u;
+            };
+            if (draws) {
+                i1 = dealt + (int)draw();
+                if (i1 < args.ntiles) {
+                    d1 = args.tiles[i1];
+                    ahead = draw();
+                }
+            }
             int jp = 0;
             bool pfail = false;
-            for (; jp < ntl; ++jp) {
+            for (; jp < (draws ? nf : ntl); ++jp) {
                 const int st = jp % NS;
                 if (!mbar_wait_bounded(&empty[st], (uint32_t)((jp / NS) & 1), args.spin_limit)) {
                     pfail = true;
                     break;
                 }
                 store_tile(jp);
-                if (jp + NS < ntl) {
+                if (draws) {
+                    if (i1 < args.ntiles) {
+                        bulk_wait_read();  // the stores have read the stage
+                        fill(nf++, d1, i1);
+                        i1 = dealt + (int)ahead;
+                        if (i1 < args.ntiles) {
+                            d1 = args.tiles[i1];
+                            ahead = draw();
+                        }
+                    } else if (!ended) {
+                        params[st].X = 0;  // tells the colliding warps
+                        mbar_arrive(&full[st]);
+                        end_draws();
+                    }
+                } else if (jp + NS < ntl) {
                     const TileDesc nt = params[st].next;
-                    bulk_wait_read();  // the stores have read the stage
-                    fill(jp + NS, nt);
+                    bulk_wait_read();
+                    fill(jp + NS, nt, (int)blockIdx.x + (jp + NS) * G);
                 }
             }
+            if (!ended) end_draws();  // (after a failure)
             if (pfail) {
                 // the colliding warps gave up on a tile: report it, and give
                 // the copies still in flight a bounded chance to land
@@ -453,7 +501,7 @@ __global__ void __launch_bounds__(NTHREADS + 32, NTHREADS + 32 >= 512 ? 1 : LBM_
     // from there.
     bool fail = false;
     int j = 0;
-    for (; j < ntl && !fail; ++j) {
+    for (; draws || j < ntl; ++j) {
         const int st = j % NS;
         // the warp leaves together if the copies did not land in time
         const bool landed = mbar_wait_bounded(&full[st], (uint32_t)((j / NS) & 1), args.spin_limit);
@@ -465,6 +513,7 @@ __global__ void __launch_bounds__(NTHREADS + 32, NTHREADS + 32 >= 512 ? 1 : LBM_
         // what every unit needs; the boundary data (bc, strides, lid) is read
         // by the edge units only
         const StageParams& p = params[st];
+        if (DRAWS && p.X == 0) break;  // no further tile
         const int x0 = p.x0, y0 = p.y0, nx = p.in.nx, ny = p.in.ny;
         unsigned char* sb = reinterpret_cast<unsigned char*>(stage_base + (size_t)st * TS::STAGE_ELEMS);
         const int lgX = 31 - __clz(p.X);   // log2 of the tile width X
