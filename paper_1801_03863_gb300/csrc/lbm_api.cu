@@ -480,10 +480,12 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
     if (is_flat(ctx, s)) {
         // An SM takes as many CTAs as it has room for, so a grid of a few
         // CTAs per SM is dealt unevenly: claim the shared memory that leaves
-        // room for an equal share and no more.
+        // room for an equal share and no more.  Up to four warps per SM, one
+        // per scheduler, gain nothing (40 lattices of 17 x 17: 12.6 us either
+        // way), and leave their SMs free for other streams' work.
         const int64_t ctas = (int64_t)t.size() * (ctx->flat_nodes / block);
         const int64_t share = (ctas + ctx->num_sms - 1) / ctx->num_sms;
-        if (share > 1 && share <= 32) smem = (size_t)(227 * 1024 / share - 1024) / 1024 * 1024;
+        if (share > 4 && share <= 32) smem = (size_t)(227 * 1024 / share - 1024) / 1024 * 1024;
         LBM_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024));
     }
     int per_sm = 0;
