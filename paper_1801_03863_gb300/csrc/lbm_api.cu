@@ -1133,7 +1133,7 @@ int lbm_create_batch(lbm_ctx** out, lbm_lattice lat, int32_t count, const int64_
     {
         std::vector<int2> items;
         for (int i = 0; i < count; ++i)
-            for (int b = 0; b < cons_partials(ctx->layout.inst[i].ny); ++b) items.push_back({i, b});
+            for (int b = 0; b < cons_partials(ctx->layout.inst[i].nx, ctx->layout.inst[i].ny); ++b) items.push_back({i, b});
         ctx->n_cons = (int)items.size();
         if (cudaMemcpyAsync(ctx->d_cons, items.data(), sizeof(int2) * items.size(),
                             cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||
@@ -1180,11 +1180,9 @@ int lbm_init_device(lbm_ctx* ctx, const double* rho, const double* ux, const dou
     if (!ctx || !rho) return LBM_ERR_ARG;
     if (ctx->failed) return LBM_ERR_CUDA;
     AuxArgs a = aux_args(ctx);
+    a.error = ctx->d_error;  // the kernel clears the status counters and the error word
     LBM_CK(run_aux(AuxOp::Init, a, nullptr, ctx->buf[ctx->cur], rho, ux, uy, nullptr, nullptr,
                    nullptr));
-    LBM_CK(cudaMemsetAsync(ctx->d_status, 0, sizeof(unsigned long long) * 2 * ctx->count,
-                           ctx->stream));
-    LBM_CK(cudaMemsetAsync(ctx->d_error, 0, sizeof(unsigned int), ctx->stream));
     ctx->post = false;
     ctx->initialized = true;
     ctx->inst_init.assign(ctx->count, 1);

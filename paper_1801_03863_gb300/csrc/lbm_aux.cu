@@ -278,8 +278,12 @@ __device__ __forceinline__ void block_range(uint32_t n, uint32_t per, uint32_t& 
 template <class Lat, typename S>
 __global__ void __launch_bounds__(AUX_THREADS)
 init_kernel(S* dst, const InstDesc* insts, const double* rho, const double* ux, const double* uy,
-            double rho0, int64_t node_base, uint32_t per) {
+            double rho0, int64_t node_base, uint32_t per, unsigned long long* status, unsigned int* error) {
     const InstDesc& in = insts[blockIdx.y];
+    if (error && blockIdx.x == 0) {  // (whole-context calls: two launches of memsets less)
+        if (threadIdx.x < 2) status[2 * blockIdx.y + threadIdx.x] = 0ull;
+        if (blockIdx.y == 0 && threadIdx.x == 2) *error = 0u;
+    }
     const uint32_t nx = (uint32_t)in.nx;
     uint32_t first, last;
     block_range(nx * (uint32_t)in.ny, per, first, last);
@@ -581,7 +585,7 @@ stream_function_kernel(const S* src, const InstDesc* insts, bool pulled, double 
 //
 // Bound by the latency of a thread's few chunks and its CTA's tail, at 0.4 of
 // the copy bandwidth.  64 cavities (33.4 M nodes) FP16: 324 us with shifted
-// loads per node, now 219 us; 2048^2 FP16: 134 -> 51 us (clusters of 4);
+// loads per node, now 214 us; 2048^2 FP16: 134 -> 51 us (clusters of 4);
 // 4096 tubes FP32: 343 -> 84 us.  Pass 2 with one thread per instance took
 // 17 us, now 6 us.
 template <class Lat>
@@ -651,7 +655,7 @@ cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool
     constexpr int Q = Lat::Q, E = 16 / (int)sizeof(S);  // nodes per chunk
     const int2 it = items[blockIdx.x];
     const InstDesc& in = insts[it.x];
-    const int nx = in.nx, ny = in.ny, P = cons_partials(ny);
+    const int nx = in.nx, ny = in.ny, P = cons_partials(nx, ny);
     const uint32_t C = (uint32_t)cons_split((int64_t)nx * ny), rank = blockIdx.y;
     const uint32_t chunks = (uint32_t)(nx + E - 1) / E;       // per row
     const uint64_t total = (uint64_t)((ny - it.y + P - 1) / P) * chunks;
@@ -847,7 +851,7 @@ __global__ void cons_final_kernel(const double* partials, const InstDesc* insts,
                                   double rho0, double* out) {
     const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = (int)(threadIdx.x & 31u);
     if (i >= count) return;
-    const int P = cons_partials(insts[i].ny);
+    const int P = cons_partials(insts[i].nx, insts[i].ny);
     double s[3] = {0.0, 0.0, 0.0};
     for (int b = lane; b < P; b += 32)
         for (int c = 0; c < 3; ++c) s[c] += partials[((int64_t)i * CONS_PARTIALS + b) * 3 + c];
@@ -909,7 +913,8 @@ cudaError_t aux_dispatch(AuxOp op, const AuxArgs& a, const void* src, void* dst,
     switch (op) {
         case AuxOp::Init:
             init_kernel<Lat, S><<<g, AUX_THREADS, 0, a.stream>>>(static_cast<S*>(dst), a.inst, p0, p1,
-                                                                 p2, a.rho0, a.node_base, per);
+                                                                 p2, a.rho0, a.node_base, per, a.status,
+                                                                 a.error);
             break;
         case AuxOp::SetF:
             set_f_kernel<Lat, S><<<g, AUX_THREADS, 0, a.stream>>>(static_cast<S*>(dst), a.inst, p0,

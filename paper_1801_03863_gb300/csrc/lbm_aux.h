@@ -7,14 +7,22 @@
 
 namespace lbm {
 
-// Conservation reduction: instance i is split into P_i = min(CONS_PARTIALS,
-// ny_i) partial sums, partial b over the rows y = b mod P_i, each summed by
+// Conservation reduction: instance i is split into P_i <= CONS_PARTIALS
+// partial sums, partial b over the rows y = b mod P_i, each summed by
 // cons_split(nodes) CTAs of CONS_THREADS threads (a cluster); the split is a
 // function of the instance alone, so the FP64 summation order never depends
 // on the device or on the other instances.
 constexpr int CONS_PARTIALS = 64;
 constexpr int CONS_THREADS = 256;
-__host__ __device__ inline int cons_partials(int ny) { return ny < CONS_PARTIALS ? ny : CONS_PARTIALS; }
+// one partial per CONS_NODES nodes, at most one per row (with 64 for every
+// lattice the smallest ones' CTAs are mostly tail: 121 us on 64 lattices of
+// 64^2 to 1024^2, FP16, now 93 us)
+constexpr int CONS_NODES = 1024;
+__host__ __device__ inline int cons_partials(int nx, int ny) {
+    const int64_t want = ((int64_t)nx * ny + CONS_NODES - 1) / CONS_NODES;
+    const int most = ny < CONS_PARTIALS ? ny : CONS_PARTIALS;
+    return want < most ? (int)want : most;
+}
 // 1, 2, 4 or 8: some 2^14 nodes per CTA, which take it longer than its tail
 // of FP64 additions (8 CTAs for 2^20 nodes: 787 us on 64 cavities of up to
 // 1024^2, FP16, where one takes 351 us)
@@ -36,6 +44,7 @@ struct AuxArgs {
     double rho0;
     bool pulled;           // stored field is post-collision (pull to read f(t_n))
     unsigned long long* status;
+    unsigned int* error = nullptr;  // Init: cleared with the status counters unless null
     cudaStream_t stream;
     const int2* cons_items;  // device: (instance, partial) of each conservation block
     int32_t cons_nitems;
