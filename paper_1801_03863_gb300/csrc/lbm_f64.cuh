@@ -15,18 +15,31 @@ namespace lbm {
 // ---------------------------------------------------------------------------
 // Natural logarithm, table driven (P. T. P. Tang, "Table-driven
 // implementation of the logarithm function in IEEE floating-point
-// arithmetic", ACM TOMS 16, 1990): for y = 1 + delta in [1/4, 4) the leading
+// arithmetic", ACM TOMS 16, 1990) with accurate tables (S. Gal, "Computing
+// elementary functions: a new approach for achieving high accuracy and good
+// performance", LNCS 235, 1986): for y = 1 + delta in [1/4, 4) the leading
 // 10 mantissa bits select a rational rc close to 1/y, then
 //     ln y = ln(1/rc) + ln(1 + r),  r = y rc - 1 = delta rc + (rc - 1),
 // |r| <= 2^-10, by the Taylor series to r^6 (remainder below 2^-62 of r).
-// rc is 1 in the two intervals that touch y = 1, so ln y keeps its relative
-// precision for small delta.  The terms from r^4 on, r^4 (-1/4 + r/5 - r^2/6),
-// have their bracket in FP32: its rounding is below 2^-56 of r.  rc and
-// rc - 1 have at most 12 significant bits, so that their high words alone
-// are stored.  6 FP64 instructions and one 16-byte table read, where the
+// Of the rc near 1/y the table holds the one whose ln(1/rc) lies closest to
+// an FP64 number (0.04 ulp off on average instead of 0.25), which costs nothing
+// here and leaves one rounding where |ln y| is large against r.  rc is 1 in
+// the two intervals that touch y = 1, so ln y keeps its relative precision
+// for small delta.  The terms from r^4 on, r^4 (-1/4 + r/5 - r^2/6), have
+// their bracket in FP32: its rounding is below 2^-56 of r.  rc and rc - 1
+// have at most 17 significant bits, so that their high words alone are
+// stored.  6 FP64 instructions and one 16-byte table read, where the
 // library's log1p takes about 25.
+//
+// Relative error in units of 2^-53, largest / rms over 2^20 values (the
+// library's log1p in brackets): delta in (-3/4, 3) 2.0 / 0.445 (2.6 / 0.608),
+// [1/4, 1/2] 1.4 / 0.442 (1.5 / 0.482), [2^-5, 2^-4] 1.06 / 0.414
+// (1.06 / 0.416); worst in the binade that meets the intervals of rc = 1,
+// [2^-10, 2^-9] 2.0 / 0.482 (1.0 / 0.408), where the rounding of r counts.  With rc at
+// the intervals' centres it was 2.8 / 0.6 to 0.7 nearly everywhere.
 // ---------------------------------------------------------------------------
 constexpr int LOG_BITS = 10, LOG_HALF = 1 << LOG_BITS;  // intervals of an octave
+constexpr int LOG_GRID = 1 << 14;                        // rc = j / (2^(k + 1) LOG_GRID), k: octave of y
 struct alignas(16) LogEntry {
     double lc;           // ln(1 / rc)
     uint32_t rc, rm;     // high words of rc and rc - 1 (low words are 0)
@@ -44,41 +57,71 @@ constexpr uint32_t ratio_high_word(int j, int sh) {
     return (j < 0 ? 0x80000000u : 0u) | ((uint32_t)(1023 + top - sh) << 20) | ((m << (20 - top)) & 0xfffffu);
 }
 
-// ln(2 H / j), j = H .. 2 H (H = LOG_HALF), as sums of ln((k + 1) / k) =
-// 2 atanh(1 / (2 k + 1)), each term a short series, summed in double-double
-// (Knuth's two-sum).
-constexpr LogTable make_log_table() {
-    constexpr int H = LOG_HALF;
-    LogTable t{};
-    double hi[H + 1] = {}, lo[H + 1] = {};  // index j - H
-    for (int k = 2 * H - 1; k >= H; --k) {
+// a + b as hi + lo exactly (Knuth's two-sum)
+struct DoubleDouble {
+    double hi, lo;
+};
+constexpr DoubleDouble two_sum(double a, double b) {
+    const double s = a + b, v = s - a;
+    return {s, (a - (s - v)) + (b - v)};
+}
+
+// ln(2 G / j), j = G .. 2 G (G = LOG_GRID), as sums of ln((k + 1) / k) =
+// 2 atanh(1 / (2 k + 1)), each term a short series, summed in double-double.
+struct LogGrid {
+    DoubleDouble v[LOG_GRID + 1];  // index j - G
+};
+constexpr LogGrid make_log_grid() {
+    constexpr int G = LOG_GRID;
+    LogGrid t{};
+    for (int k = 2 * G - 1; k >= G; --k) {
         const double n = 2.0 * k + 1.0, z = 1.0 / n, z2 = z * z;
         // z = fl(1 / n); its rounding error is (1 - n z) / n, with n z split
-        // exactly: n < 2^13, z cut to its upper 26 bits
+        // exactly: n < 2^17, z cut to its upper 26 bits
         const double big = z * 134217729.0;  // Veltkamp split, 2^27 + 1
         const double zh = big - (big - z), zl = z - zh;
         const double ze = ((1.0 - n * zh) - n * zl) * z;
-        double s = 0.0;  // z^3 / 3 + z^5 / 5 + ...
-        for (int m = 6; m >= 1; --m) s = (s + 1.0 / (2.0 * m + 1.0)) * z2;
-        s = s * z;
-        const int i = k - H;
-        const double a = hi[i + 1], b = 2.0 * z;
-        const double sum = a + b, bv = sum - a;
-        const double err = (a - (sum - bv)) + (b - bv);
-        const double tail = lo[i + 1] + err + 2.0 * (ze + s);
-        hi[i] = sum + tail;
-        lo[i] = tail - (hi[i] - sum);
+        // z^3 / 3 + z^5 / 5 + z^7 / 7 (z < 2^-15: the next term is below 2^-120 z)
+        const double s = ((1.0 / 7.0 * z2 + 1.0 / 5.0) * z2 + 1.0 / 3.0) * z2 * z;
+        const DoubleDouble p = t.v[k + 1 - G];
+        const DoubleDouble q = two_sum(p.hi, 2.0 * z);
+        t.v[k - G] = two_sum(q.hi, q.lo + (p.lo + 2.0 * (ze + s)));
     }
+    return t;
+}
+
+constexpr LogTable make_log_table() {
+    constexpr int H = LOG_HALF, G = LOG_GRID;
+    const LogGrid ln = make_log_grid();
+    LogTable t{};
     for (int i = 0; i < H; ++i) {
-        const double c = 1.0 + (i + 0.5) / H;  // centre of the interval of m, y = m or m / 2
-        int j = (int)(2.0 * H / c + 0.5);
-        if (i == 0) j = 2 * H;  // rc = 1 right of y = 1 (and, with j = H for i = H - 1, left of it)
-        for (int o = 0; o < 4; ++o) {  // y = 2^k m, k = o - 2
+        const double c = 1.0 + (i + 0.5) / H;  // centre of the interval of m, y = 2^k m
+        const int centre = (int)(2.0 * G / c + 0.5);
+        for (int o = 0; o < 4; ++o) {
             const int k = o - 2;
+            // rc = 1 right of y = 1 and left of it
+            const bool at_one = (k == 0 && i == 0) || (k == -1 && i == H - 1);
+            int best = at_one ? (k == 0 ? 2 * G : G) : centre;
+            // others within 2^-12 of the centre: |r| stays below 2^-10
+            const int reach = at_one ? 0 : centre >> 12;
+            double least = 1e300, lc = 0.0;
+            for (int j = centre - reach; j <= centre + reach; ++j) {
+                const int jj = at_one ? best : j;
+                if (jj < G || jj > 2 * G) continue;
+                const DoubleDouble a = two_sum(ln.v[jj - G].hi, k * ln.v[0].hi);
+                const DoubleDouble b = two_sum(a.hi, a.lo + (ln.v[jj - G].lo + k * ln.v[0].lo));
+                // in units of the logarithm itself
+                const double off = b.hi == 0.0 ? 0.0 : (b.lo < 0 ? -b.lo : b.lo) / (b.hi < 0 ? -b.hi : b.hi);
+                if (off < least) {
+                    least = off;
+                    best = jj;
+                    lc = b.hi;
+                }
+            }
             LogEntry& u = t.e[o * H + i];
-            u.lc = (hi[j - H] + k * hi[0]) + (lo[j - H] + k * lo[0]);
-            u.rc = ratio_high_word(j, LOG_BITS + 1 + k);
-            u.rm = ratio_high_word(j - (k >= 0 ? (2 * H) << k : (2 * H) >> -k), LOG_BITS + 1 + k);
+            u.lc = lc;
+            u.rc = ratio_high_word(best, 15 + k);
+            u.rm = ratio_high_word(best - (k >= 0 ? (2 * G) << k : (2 * G) >> -k), 15 + k);
         }
     }
     return t;
@@ -102,20 +145,14 @@ __device__ __forceinline__ double log_entry(uint32_t i, double delta) {
     return __hiloint2double(e.y, e.x) + fma(r * r, q, r);
 }
 
-// Outside [1/4, 4): y = 2^k m, ln m by the table from m - 1, plus k ln 2.  Not
-// inlined: FP64 instructions hold the pipe even where their predicate is off.
-__device__ __noinline__ static double log1p_outside(double delta, double y) {
-    const uint32_t yh = (uint32_t)__double2hiint(y);
-    if (yh - 0x00100000u >= 0x7fe00000u) return log1p(delta);  // not positive and normal
-    const double m = __hiloint2double((int)((yh & 0xfffffu) | 0x3ff00000u), __double2loint(y));
-    const uint32_t i = 2u * LOG_HALF + ((yh >> (20 - LOG_BITS)) & (LOG_HALF - 1u));
-    return fma((double)((int)(yh >> 20) - 1023), 0.6931471805599453, log_entry(i, m - 1.0));
-}
+// Outside [1/4, 4): the library's.  Not inlined: FP64 instructions hold the
+// pipe even where their predicate is off.
+__device__ __noinline__ static double log1p_outside(double delta) { return log1p(delta); }
 
 // ln(1 + delta), given delta and y = 1 + delta rounded
 __device__ __forceinline__ double log1p_f64(double delta, double y) {
     const uint32_t i = ((uint32_t)__double2hiint(y) - 0x3fd00000u) >> (20 - LOG_BITS);
-    if (i >= 4u * LOG_HALF) return log1p_outside(delta, y);
+    if (i >= 4u * LOG_HALF) return log1p_outside(delta);
     return log_entry(i, delta);
 }
 
