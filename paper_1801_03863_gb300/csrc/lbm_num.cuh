@@ -36,16 +36,23 @@ __device__ __forceinline__ float lg2_approx(float x) {
     return r;
 }
 
-// 1 / x in FP64: the 20-bit hardware seed and one third-order Newton step,
-// r (1 + e + e^2) with e = 1 - x r (error e^3 < 2^-60, then one rounding):
-// 3 FP64 instructions instead of an IEEE division's 8.  Operands near the
-// ends of the exponent range, zeros, infinities and NaN take the division.
+// 1 / x in FP64: the FP32 reciprocal of x cut to 24 bits (error below 2^-21.9)
+// as the seed and one third-order Newton step, r (1 + e + e^2) with e = 1 - x r:
+// 3 FP64 instructions instead of an IEEE division's 8.  The error before the
+// last rounding is e^3 < 2^-65, so that about one result in 10^5 differs
+// from the IEEE quotient, by one unit, and none is off by more than 0.501 ulp
+// (the 20-bit FP64 seed left 2^-60: one result in 100).  The seed's conversions
+// run on the integer pipe.  Operands or results outside FP32's normal range,
+// zeros, infinities and NaN take the division.
 __device__ __noinline__ static double rcp_f64_slow(double x) { return 1.0 / x; }
 __device__ __forceinline__ double rcp_f64(double x) {
-    const uint32_t ex = ((uint32_t)__double2hiint(x) >> 20) & 0x7ffu;
-    if (ex - 64u >= 1920u) return rcp_f64_slow(x);
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    if (((hi >> 20) & 0x7ffu) - 899u >= 249u) return rcp_f64_slow(x);  // |x| in [2^-124, 2^125)
+    const uint32_t m = __funnelshift_l(lo, hi, 3);  // exponent and leading 23 bits, FP64's bias
+    const uint32_t s = __float_as_uint(
+        rcp_approx(__uint_as_float(((m - 0xc0000000u) & 0x7fffffffu) | (hi & 0x80000000u))));
+    const double r = __hiloint2double(
+        (int)((s & 0x80000000u) | (((s & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(s << 29));
     const double e = fma(-x, r, 1.0);
     return fma(r, fma(e, e, e), r);
 }

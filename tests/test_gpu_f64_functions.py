@@ -77,3 +77,17 @@ def test_logarithm_outside_the_table(device_function):
     outside = (1.0 + x < 0.25) | (1.0 + x >= 4.0) | np.isnan(x)
     np.testing.assert_array_equal(a[outside], b[outside])
     assert (a[~outside] == b[~outside]).sum() >= 2  # the zeros
+
+
+def test_reciprocal(device_function):
+    """Error before the last rounding below 2^-65 of the result, so below half a unit in the last place
+    and 2^-12 after it; outside FP32's range the IEEE quotient."""
+    rng = np.random.default_rng(4)
+    x = rng.uniform(1.0, 2.0, 1 << 18) * 2.0 ** rng.integers(-120, 120, 1 << 18) * rng.choice([-1.0, 1.0], 1 << 18)
+    got = device_function(RCP, x)
+    off = np.abs(got - 1 / x.astype(np.longdouble)) / np.abs(np.spacing(got))
+    assert off.max() <= 0.5 + 2.0 ** -12
+    edge = np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 5e-324, 1e-310, -1e-310, 1.7e308, -1.7e308, 1e300,
+                     -1e-300, 2.0 ** 125, 2.0 ** -125, 2.0 ** 126, 2.0 ** -126, 2.0 ** 1022, 2.0 ** 1023])
+    with np.errstate(divide="ignore", over="ignore"):
+        np.testing.assert_array_equal(device_function(RCP, edge), 1.0 / edge)
