@@ -573,9 +573,9 @@ stream_function_kernel(const S* src, const InstDesc* insts, bool pulled, double 
 // and the first CTA of the cluster adds the CTAs' sums in order.  The order
 // of all additions is fixed by the instance alone.
 //
-// FP64 storage sums in FP64.  FP32 and BF16 storage sum in compensated FP32
-// pairs (Knuth's two-sum; about twice FP32's precision, converted to FP64
-// once per warp), which spares the slow FP64 pipe.  FP16 storage sums
+// FP64 storage sums in FP64.  FP32 and BF16 storage sum a thread's nodes in
+// compensated FP32 pairs (Knuth's two-sum; about twice FP32's precision,
+// converted to FP64 once per thread), which spares the slow FP64 pipe.  FP16 storage sums
 // exactly in integers: every FP16 value is a multiple of 2^-24 below 2^16 in
 // magnitude; a chunk whose values are all below 2^-7 adds exactly in FP32
 // (its sums stay below 1) and is converted to integers once, a node below
@@ -783,57 +783,63 @@ cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool
                 }
             }
         }
-    // fixed trees: lanes, then warps, then the CTAs of the cluster in order
-    __shared__ double sh[3][CONS_THREADS / 32];
+    // fixed trees: threads, then the CTAs of the cluster in order
     __shared__ double cta[3];
-    double s[3] = {t.s0, t.s1, t.s2};
-    bool in_f64 = true;  // some lane's part is in FP64 (the same for the warp)
     if constexpr (std::is_same<S, __half>::value) {
-        // integers add exactly; FP64 only holds nodes with non-finite values
+        // integers add exactly within a warp; FP64 only holds nodes with non-finite values
         // (at most 2^31 values below 2^41: no overflow)
+        __shared__ double sh[3][CONS_THREADS / 32];
+        double s[3] = {t.s0, t.s1, t.s2};
         long long i[3] = {t.i0, t.i1, t.i2};
-        in_f64 = __any_sync(0xffffffffu, !(s[0] == 0.0 && s[1] == 0.0 && s[2] == 0.0));
+        const bool in_f64 = __any_sync(0xffffffffu, !(s[0] == 0.0 && s[1] == 0.0 && s[2] == 0.0));
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
 #pragma unroll
             for (int h = 16; h > 0; h >>= 1) i[c] += __shfl_down_sync(0xffffffffu, i[c], h);
             if ((threadIdx.x & 31u) == 0u) s[c] += (double)i[c] * (1.0 / 16777216.0);
+            if (in_f64) {
+#pragma unroll
+                for (int h = 16; h > 0; h >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], h);
+            }
+            if ((threadIdx.x & 31u) == 0u) sh[c][threadIdx.x >> 5] = s[c];
         }
-    } else if constexpr (!std::is_same<S, double>::value) {
-        // both node lanes, then the warp's lanes, still in pairs
-        in_f64 = __any_sync(0xffffffffu, !(s[0] == 0.0 && s[1] == 0.0 && s[2] == 0.0));
-        F2 h[3] = {t.h0, t.h1, t.h2}, e[3] = {t.c0, t.c1, t.c2};
+        __syncthreads();
+        if (threadIdx.x < 3) {
+            double v = 0.0;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            if (Q == 3 && c == 2) continue;
-            float a = h[c].v.x, r = e[c].v.x + e[c].v.y;
-            auto add = [&](float b, float rb) {
-                const float sum = __fadd_rn(a, b), bv = __fsub_rn(sum, a);
-                r = __fadd_rn(__fadd_rn(r, rb),
-                              __fadd_rn(__fsub_rn(a, __fsub_rn(sum, bv)), __fsub_rn(b, bv)));
-                a = sum;
-            };
-            add(h[c].v.y, 0.f);
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1)
-                add(__shfl_down_sync(0xffffffffu, a, d), __shfl_down_sync(0xffffffffu, r, d));
-            if ((threadIdx.x & 31u) == 0u) s[c] += widen(a) + widen(r);
+            for (int w = 0; w < CONS_THREADS / 32; ++w) v += sh[threadIdx.x][w];
+            cta[threadIdx.x] = v;
         }
-    }
+    } else {
+        // A thread's sums in FP64, then one warp per sum adds them: 8 of every lane and a shuffle
+        // tree, 36 FP64 warp instructions a CTA where a tree in each warp takes 120
+        __shared__ double sh[3][CONS_THREADS];
+        double s[3] = {t.s0, t.s1, t.s2};
+        if constexpr (!std::is_same<S, double>::value) {
+            const F2 h[3] = {t.h0, t.h1, t.h2}, e[3] = {t.c0, t.c1, t.c2};
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        if (in_f64) {
-#pragma unroll
-            for (int h = 16; h > 0; h >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], h);
+            for (int c = 0; c < (Q == 3 ? 2 : 3); ++c) {
+                // the thread's two node lanes as one pair
+                const float x = h[c].v.x, y = h[c].v.y;
+                const float sum = __fadd_rn(x, y), bv = __fsub_rn(sum, x);
+                const float r = __fadd_rn(__fadd_rn(e[c].v.x, e[c].v.y),
+                                          __fadd_rn(__fsub_rn(x, __fsub_rn(sum, bv)), __fsub_rn(y, bv)));
+                const double v = widen(sum) + widen(r);
+                s[c] = __double_as_longlong(s[c]) == 0 ? v : s[c] + v;  // (FP64 part: nodes that are not finite)
+            }
         }
-        if ((threadIdx.x & 31u) == 0u) sh[c][threadIdx.x >> 5] = s[c];
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        double v = 0.0;
 #pragma unroll
-        for (int w = 0; w < CONS_THREADS / 32; ++w) v += sh[threadIdx.x][w];
-        cta[threadIdx.x] = v;
+        for (int c = 0; c < 3; ++c) sh[c][threadIdx.x] = s[c];
+        __syncthreads();
+        const int c = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31u);
+        if (c < 3) {
+            double v = sh[c][lane];
+#pragma unroll
+            for (int w = 1; w < CONS_THREADS / 32; ++w) v += sh[c][lane + 32 * w];
+#pragma unroll
+            for (int h = 16; h > 0; h >>= 1) v += __shfl_down_sync(0xffffffffu, v, h);
+            if (lane == 0) cta[c] = v;
+        }
     }
     const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     cluster.sync();
