@@ -649,6 +649,8 @@ __device__ __forceinline__ bool half_sums(const float (&d)[Lat::Q], long long (&
     return finite;
 }
 
+__device__ __noinline__ double add_slow(long long a, long long b) { return (double)a + (double)b; }
+
 template <class Lat, typename S>
 __global__ void __launch_bounds__(CONS_THREADS, 3)
 cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool pulled, double* partials) {
@@ -786,8 +788,11 @@ cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool
     // fixed trees: threads, then the CTAs of the cluster in order
     __shared__ double cta[3];
     if constexpr (std::is_same<S, __half>::value) {
-        // integers add exactly within a warp; FP64 only holds nodes with non-finite values
-        // (at most 2^31 values below 2^41: no overflow)
+        // integers add exactly within a warp; FP64 only holds nodes with non-finite values.
+        // A lane has some 2^15 nodes at most (2^31 nodes of an instance, of at least 1 in 8 CTAs
+        // of 256 threads; a row has at most 2^26), so its sums stay below
+        // 2^15 x 9 x 2^40 < 2^58.2 and those of 16 lanes below 2^62.2; those of
+        // two such halves may not fit.
         __shared__ double sh[3][CONS_THREADS / 32];
         double s[3] = {t.s0, t.s1, t.s2};
         long long i[3] = {t.i0, t.i1, t.i2};
@@ -795,8 +800,13 @@ cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
 #pragma unroll
-            for (int h = 16; h > 0; h >>= 1) i[c] += __shfl_down_sync(0xffffffffu, i[c], h);
-            if ((threadIdx.x & 31u) == 0u) s[c] += (double)i[c] * (1.0 / 16777216.0);
+            for (int h = 16; h > 1; h >>= 1) i[c] += __shfl_down_sync(0xffffffffu, i[c], h);
+            const long long o = __shfl_down_sync(0xffffffffu, i[c], 1);
+            const long long sum = (long long)((uint64_t)i[c] + (uint64_t)o);
+            if ((threadIdx.x & 31u) == 0u) {
+                const bool wraps = ((i[c] ^ sum) & (o ^ sum)) < 0;
+                s[c] += (wraps ? add_slow(i[c], o) : (double)sum) * (1.0 / 16777216.0);
+            }
             if (in_f64) {
 #pragma unroll
                 for (int h = 16; h > 0; h >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], h);
