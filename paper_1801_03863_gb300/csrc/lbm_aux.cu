@@ -152,27 +152,31 @@ __device__ __forceinline__ double fixed_to_f64(long long v, int e) {
 }
 
 // moment_sums of FP32 values in 64-bit fixed point, the largest value at bit
-// 58: what a smaller value loses below 2^-58 of it is less than the rounding
-// of FP64 additions, and the integer pipe does the work.  False where some
-// value is not finite or all are below 2^-80 (but zeros are fine).
+// 58: exact, so that each sum rounds once, and the work of the integer pipe.
+// False where a value is not finite, the largest is below 2^-80, or the
+// smallest (but for zeros) has bits more than 58 places below the largest's
+// first: FP64 additions then lose less where the largest is not in the sum.
 template <class Lat>
 __device__ __forceinline__ bool fixed_sums(const float (&d)[Lat::Q], double& m, double& jx, double& jy) {
-    uint32_t top = 0u;
+    uint32_t top = 0u, low = 0xffffffffu;  // low: smallest magnitude's bits less 1, zeros apart
 #pragma unroll
-    for (int a = 0; a < Lat::Q; ++a) top = max(top, __float_as_uint(d[a]) & 0x7fffffffu);
+    for (int a = 0; a < Lat::Q; ++a) {
+        const uint32_t b = __float_as_uint(d[a]) & 0x7fffffffu;
+        top = max(top, b);
+        low = min(low, b - 1u);
+    }
     const int emax = (int)(top >> 23);
     if (top == 0u) {
         m = jx = jy = 0.0;
         return true;
     }
-    if (emax == 255 || emax < 47) return false;
+    if (emax == 255 || emax < 47 || emax - (int)((low + 1u) >> 23) > 35) return false;
     long long v[Lat::Q];
 #pragma unroll
     for (int a = 0; a < Lat::Q; ++a) {
-        const uint32_t b = __float_as_uint(d[a]);
-        const int e = max((int)((b >> 23) & 0xffu), 1), down = emax - e;
-        const uint32_t mant = (b & 0x7fffffu) | ((b & 0x7f800000u) ? 0x800000u : 0u);
-        const long long u = (long long)(((uint64_t)mant << 35) >> min(down, 63));
+        const uint32_t b = __float_as_uint(d[a]);  // (no subnormals here)
+        const uint64_t mant = (b & 0x7fffffffu) ? (b & 0x7fffffu) | 0x800000u : 0u;
+        const long long u = (long long)(mant << (((b >> 23) & 0xffu) + 35u - (uint32_t)emax & 63u));
         v[a] = (int)b < 0 ? -u : u;
     }
     long long im, ix, iy;
