@@ -155,7 +155,7 @@ Carve carve(const Layout& L, int lattice, int storage, int count) {
     p += al(sizeof(double) * std::max<int64_t>(3 * L.total_nodes, Q * L.total_nodes));
     c.tmap_off = p;  // four TMA tensor maps per instance: [buffer][tile | halo]
     p += al(4 * sizeof(CUtensorMapOpaque) * count);
-    c.err_off = p;  // error word and, from word 8 on, the TMA kernel's tile counters
+    c.err_off = p;  // ERROR_WORDS words (256 bytes are kept for them)
     p += 256;
     c.total = p;
     return c;
@@ -576,7 +576,7 @@ StepArgs step_args(const lbm_ctx* ctx, int src) {
     a.tmaps_halo = ctx->d_tmaps + (size_t)(src * 2 + 1) * ctx->count;
     a.tmaps_dst = ctx->d_tmaps + (size_t)(1 - src) * 2 * ctx->count;
     a.error = ctx->d_error;
-    a.tile_counters = ctx->d_error + 8;
+    a.tile_counters = ctx->d_error + TILE_COUNTERS;
     a.spin_limit = ctx->spin_limit;
     a.lost_tile = ctx->lost_tile;
     a.inplace = 0;
@@ -963,6 +963,13 @@ uint64_t layout_hash(const lbm_ctx* ctx) {
     return h;
 }
 
+// The counters of the TMA kernel's drawn tiles are 0 between launches; a
+// launch that timed out may leave them otherwise, so every entry point that
+// sets a state clears them (the sticky error word is another matter).
+cudaError_t clear_tile_counters(lbm_ctx* ctx) {
+    return cudaMemsetAsync(ctx->d_error + TILE_COUNTERS, 0, 2 * sizeof(unsigned int), ctx->stream);
+}
+
 // LBM_ERR_UNSTABLE when instance i has flagged an unstable node (sticky
 // error word first); syncs.
 int instance_status(lbm_ctx* ctx, int32_t instance) {
@@ -1180,7 +1187,7 @@ int lbm_init_device(lbm_ctx* ctx, const double* rho, const double* ux, const dou
     if (!ctx || !rho) return LBM_ERR_ARG;
     if (ctx->failed) return LBM_ERR_CUDA;
     AuxArgs a = aux_args(ctx);
-    a.error = ctx->d_error;  // the kernel clears the status counters and the error word
+    a.error = ctx->d_error;  // the kernel clears the status counters and the error block
     LBM_CK(run_aux(AuxOp::Init, a, nullptr, ctx->buf[ctx->cur], rho, ux, uy, nullptr, nullptr,
                    nullptr));
     ctx->post = false;
@@ -1387,6 +1394,7 @@ int lbm_set_populations(lbm_ctx* ctx, const double* f) {
     AuxArgs a = aux_args(ctx);
     LBM_CK(run_aux(AuxOp::SetF, a, nullptr, ctx->buf[ctx->cur], ctx->d_stage, nullptr, nullptr,
                    nullptr, nullptr, nullptr));
+    LBM_CK(clear_tile_counters(ctx));
     LBM_CK(cudaStreamSynchronize(ctx->stream));
     ctx->post = false;
     ctx->initialized = true;
@@ -1435,12 +1443,13 @@ int lbm_init_batch(lbm_ctx* ctx, int32_t instance, const double* rho, const doub
                    nullptr));
     LBM_CK(cudaMemsetAsync(ctx->d_status + 2 * instance, 0, 2 * sizeof(unsigned long long),
                            ctx->stream));
+    LBM_CK(clear_tile_counters(ctx));
     LBM_CK(cudaStreamSynchronize(ctx->stream));
     if (ctx->inst_init.size() != (size_t)ctx->count) ctx->inst_init.assign(ctx->count, 0);
     ctx->inst_init[instance] = 1;
     if (!ctx->initialized &&
         std::all_of(ctx->inst_init.begin(), ctx->inst_init.end(), [](uint8_t v) { return v; })) {
-        LBM_CK(cudaMemsetAsync(ctx->d_error, 0, sizeof(unsigned int), ctx->stream));
+        LBM_CK(cudaMemsetAsync(ctx->d_error, 0, ERROR_WORDS * sizeof(unsigned int), ctx->stream));
         LBM_CK(cudaStreamSynchronize(ctx->stream));
         ctx->initialized = true;
         ctx->steps = 0;
@@ -1537,7 +1546,7 @@ int lbm_load_state(lbm_ctx* ctx, const void* host_buf) {
                            ctx->stream));
     LBM_CK(cudaMemcpyAsync(ctx->buf[0], in + sizeof h + h.status_bytes, h.buf_bytes,
                            cudaMemcpyHostToDevice, ctx->stream));
-    LBM_CK(cudaMemsetAsync(ctx->d_error, 0, sizeof(unsigned int), ctx->stream));
+    LBM_CK(cudaMemsetAsync(ctx->d_error, 0, ERROR_WORDS * sizeof(unsigned int), ctx->stream));
     LBM_CK(cudaStreamSynchronize(ctx->stream));
     ctx->cur = 0;
     ctx->post = h.post != 0;

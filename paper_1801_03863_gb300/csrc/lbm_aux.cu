@@ -286,7 +286,7 @@ init_kernel(S* dst, const InstDesc* insts, const double* rho, const double* ux, 
     const InstDesc& in = insts[blockIdx.y];
     if (error && blockIdx.x == 0) {  // (whole-context calls: two launches of memsets less)
         if (threadIdx.x < 2) status[2 * blockIdx.y + threadIdx.x] = 0ull;
-        if (blockIdx.y == 0 && threadIdx.x == 2) *error = 0u;
+        if (blockIdx.y == 0 && threadIdx.x >= 32 && threadIdx.x < 32 + ERROR_WORDS) error[threadIdx.x - 32] = 0u;
     }
     const uint32_t nx = (uint32_t)in.nx;
     uint32_t first, last;

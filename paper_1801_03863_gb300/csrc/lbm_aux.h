@@ -30,6 +30,10 @@ __host__ __device__ inline int cons_split(int64_t nodes) {
     return nodes <= (1 << 20) ? 1 : nodes <= (1 << 21) ? 2 : nodes <= (1 << 22) ? 4 : 8;
 }
 
+// Words of a context's error block: the error word, and from TILE_COUNTERS on
+// the two counters of the TMA kernel's drawn tiles.
+constexpr int TILE_COUNTERS = 8, ERROR_WORDS = 16;
+
 enum class AuxOp { Init, SetF, CollideInPlace, Moments, GatherF, StreamFunction, Conservation };
 
 struct AuxArgs {
@@ -44,7 +48,7 @@ struct AuxArgs {
     double rho0;
     bool pulled;           // stored field is post-collision (pull to read f(t_n))
     unsigned long long* status;
-    unsigned int* error = nullptr;  // Init: cleared with the status counters unless null
+    unsigned int* error = nullptr;  // Init: ERROR_WORDS words cleared with the status counters unless null
     cudaStream_t stream;
     const int2* cons_items;  // device: (instance, partial) of each conservation block
     int32_t cons_nitems;

@@ -482,7 +482,12 @@ __global__ void __launch_bounds__(NTHREADS + 32, NTHREADS + 32 >= 512 ? 1 : LBM_
                     fill(jp + NS, nt, (int)blockIdx.x + (jp + NS) * G);
                 }
             }
-            if (!ended) end_draws();  // (after a failure)
+            if (!ended) {
+                // after a failure: the draw ahead may still be under way and
+                // must not follow the reset
+                __threadfence();
+                end_draws();
+            }
             if (pfail) {
                 // the colliding warps gave up on a tile: report it, and give
                 // the copies still in flight a bounded chance to land
