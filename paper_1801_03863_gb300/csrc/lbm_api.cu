@@ -228,6 +228,15 @@ const void* find_step_kernel(int lattice, int storage, int collision, int V) {
     return nullptr;
 }
 
+const void* find_smem_kernel(const lbm_ctx* ctx, int variant, bool draws, size_t* smem) {
+    switch (ctx->storage) {
+        case DT_F32: return step_kernel_smem_f32(ctx->collision, variant, draws, smem);
+        case DT_F16: return step_kernel_smem_f16(ctx->collision, variant, draws, smem);
+        case DT_BF16: return step_kernel_smem_bf16(ctx->collision, variant, draws, smem);
+    }
+    return nullptr;
+}
+
 AuxArgs aux_args(const lbm_ctx* ctx) {
     AuxArgs a;
     a.lattice = ctx->lattice;
@@ -452,13 +461,10 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
         LBM_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     } else if (s.kind >= 1) {
         if (ctx->lattice != 2 || ctx->compute != DT_F32 || s.kind > 4) return LBM_ERR_ARG;
-        const int var = s.kind - 1;
-        if (ctx->storage == DT_F32) k = step_kernel_smem_f32(ctx->collision, var, &smem);
-        else if (ctx->storage == DT_F16) k = step_kernel_smem_f16(ctx->collision, var, &smem);
-        else if (ctx->storage == DT_BF16) k = step_kernel_smem_bf16(ctx->collision, var, &smem);
+        k = find_smem_kernel(ctx, s.kind - 1, false, &smem);
         if (!k) return LBM_ERR_ARG;
         LBM_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        const int rc = build_tensor_maps(ctx, var);
+        const int rc = build_tensor_maps(ctx, s.kind - 1);
         if (rc != LBM_OK) return rc;
     } else {
         if (is_flat(ctx, s) && (s.tw != 32 || s.th != 1)) return LBM_ERR_ARG;
@@ -491,10 +497,21 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
     int per_sm = 0;
     LBM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
     per_sm = std::max(per_sm, 1);
-    const int64_t g = s.block() ? (int64_t)t.size()
-                      : ctx->lattice == 1 ? ((int64_t)t.size() * 32 + block - 1) / block
-                      : is_flat(ctx, s) ? (int64_t)t.size() * (ctx->flat_nodes / block)
-                                        : std::min<int64_t>((int64_t)per_sm * ctx->num_sms, (int64_t)t.size());
+    int64_t g = s.block() ? (int64_t)t.size()
+                : ctx->lattice == 1 ? ((int64_t)t.size() * 32 + block - 1) / block
+                : is_flat(ctx, s) ? (int64_t)t.size() * (ctx->flat_nodes / block)
+                                  : std::min<int64_t>((int64_t)per_sm * ctx->num_sms, (int64_t)t.size());
+    if (s.tma() && smem_stages(ctx->storage, s.kind - 1) == 2 && 2 * g < (int64_t)t.size()) {
+        // more tiles than the CTAs' first two: the others are drawn
+        const void* kd = find_smem_kernel(ctx, s.kind - 1, true, &smem);
+        LBM_CK(cudaFuncSetAttribute(kd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        LBM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kd, block, smem));
+        const int64_t gd = (int64_t)std::max(per_sm, 1) * ctx->num_sms;
+        if (2 * gd < (int64_t)t.size()) {
+            k = kd;
+            g = gd;
+        }
+    }
     ctx->tiles.swap(t);
     ctx->shape = s;
     ctx->kern = k;

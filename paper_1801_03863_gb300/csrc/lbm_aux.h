@@ -91,11 +91,12 @@ constexpr size_t block_smem_bytes(int storage, int rows) {
            (rows <= BLOCK_SMALL_ROWS ? BLOCK_SMALL_ROWS : block_max_rows(storage));
 }
 
-// D2Q9 step kernels with shared-memory tile staging (FP32 arithmetic); also
-// return the dynamic shared memory they need.
-const void* step_kernel_smem_f32(int collision, int variant, size_t* smem_bytes);
-const void* step_kernel_smem_f16(int collision, int variant, size_t* smem_bytes);
-const void* step_kernel_smem_bf16(int collision, int variant, size_t* smem_bytes);
+// D2Q9 step kernels with shared-memory tile staging (FP32 arithmetic), tiles
+// dealt out or (two-stage rings) drawn; also return the dynamic shared memory
+// they need.
+const void* step_kernel_smem_f32(int collision, int variant, bool draws, size_t* smem_bytes);
+const void* step_kernel_smem_f16(int collision, int variant, bool draws, size_t* smem_bytes);
+const void* step_kernel_smem_bf16(int collision, int variant, bool draws, size_t* smem_bytes);
 // Geometries of the TMA-staged kernel (variant = launch-shape kind - 1).
 // Every CTA has one copy warp, which writes finished tiles out and issues
 // the copies of the next ones, besides its colliding warps; a tile holds
@@ -119,6 +120,18 @@ const void* step_kernel_smem_bf16(int collision, int variant, size_t* smem_bytes
 #ifndef LBM_DEEP_WARPS
 #define LBM_DEEP_WARPS 15  // colliding warps of the deep-ring CTA
 #endif
+#ifndef LBM_SMEM_STAGES
+#define LBM_SMEM_STAGES 2        // ring depth, large tiles
+#endif
+#ifndef LBM_SMEM_STAGES_SMALL
+#define LBM_SMEM_STAGES_SMALL 3  // ring depth, small tiles
+#endif
+// ring depth (storage 1: FP32)
+constexpr int smem_stages(int storage, int variant) {
+    return variant == 1   ? LBM_SMEM_STAGES_SMALL
+           : variant == 3 ? (storage == 1 ? LBM_SMEM_STAGES_DEEP : LBM_SMEM_STAGES_DEEP2)
+                          : LBM_SMEM_STAGES;
+}
 // colliding threads of a CTA (the copy warp comes on top)
 constexpr int smem_threads(int variant) {
     return variant == 2 ? 288 : (variant == 3 ? 32 * LBM_DEEP_WARPS : 224);

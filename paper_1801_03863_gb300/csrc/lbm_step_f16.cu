@@ -21,11 +21,11 @@ const void* step_kernel_block_f16(int collision, int rows) {
     return pick_step_block_kernel<__half>(collision, rows);
 }
 
-const void* step_kernel_smem_f16(int collision, int variant, size_t* smem_bytes) {
-    if (variant == 2) return pick_step_kernel_smem<__half, 2>(collision, smem_bytes);
-    if (variant == 3) return pick_step_kernel_smem<__half, 3>(collision, smem_bytes);
-    return variant == 1 ? pick_step_kernel_smem<__half, 1>(collision, smem_bytes)
-                        : pick_step_kernel_smem<__half, 0>(collision, smem_bytes);
+const void* step_kernel_smem_f16(int collision, int variant, bool draws, size_t* smem_bytes) {
+    if (variant == 2) return pick_step_kernel_smem<__half, 2>(collision, draws, smem_bytes);
+    if (variant == 3) return pick_step_kernel_smem<__half, 3>(collision, draws, smem_bytes);
+    return variant == 1 ? pick_step_kernel_smem<__half, 1>(collision, draws, smem_bytes)
+                        : pick_step_kernel_smem<__half, 0>(collision, draws, smem_bytes);
 }
 
 }  // namespace lbm

@@ -52,13 +52,6 @@
 
 namespace lbm {
 
-#ifndef LBM_SMEM_STAGES
-#define LBM_SMEM_STAGES 2        // ring depth, large tiles
-#endif
-#ifndef LBM_SMEM_STAGES_SMALL
-#define LBM_SMEM_STAGES_SMALL 3  // ring depth, small tiles
-#endif
-
 // TILE nodes per tile, NST stages, NTHREADS colliding threads (the copy
 // warp comes on top)
 template <typename S, int TILE, int NST, int NTHREADS>
@@ -314,7 +307,7 @@ __device__ __forceinline__ float2 global_pair(const S* base, int64_t pitch, int 
 // results agree bit for bit: the compiler may fuse a packed product into a
 // following packed add, and it does so alike wherever the collision is
 // inlined, which scalar code would not reproduce.
-template <typename S, int COLL, int TILE, int NST, int NTHREADS>
+template <typename S, int COLL, int TILE, int NST, int NTHREADS, bool DRAWS>
 __global__ void __launch_bounds__(NTHREADS + 32, NTHREADS + 32 >= 512 ? 1 : LBM_SMEM_MINBLOCKS)
     step_kernel_smem(const StepArgs args) {
     using TS = SmemTile<S, TILE, NST, NTHREADS>;
@@ -342,16 +335,17 @@ __global__ void __launch_bounds__(NTHREADS + 32, NTHREADS + 32 >= 512 ? 1 : LBM_
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const CT rho0v = CT((float)args.rho0);
     const int G = gridDim.x;
-    // This CTA's first NS tiles are blockIdx.x + j * G.  On a two-stage ring the
-    // further ones are drawn from a counter as stages become free; on deeper
-    // rings tile j is blockIdx.x + j * G throughout.  Dealt out beforehand, the
-    // SMs that take longer for their tiles hold up the end of every launch:
-    // FP32 MRT on 64 cavities 310 -> 272 us a step with drawn tiles, 48 ragged
-    // ones 149 -> 130, MinxEnt4 FP16 326 -> 311.  A deep ring evens that out by
-    // itself and its one copy warp per SM has no time for the draws (SRT FP16
-    // 144 -> 208 us).
-    constexpr bool DRAWS = NS == 2;
-    const bool draws = DRAWS && NS * G < args.ntiles;
+    // Local tile j of this CTA is tile blockIdx.x + j * G, or with DRAWS its first
+    // NS tiles are and the further ones are drawn from a counter as stages
+    // become free.  Dealt out beforehand, the SMs that take longer for their
+    // tiles hold up the end of every launch: FP32 MRT on 64 cavities 310 -> 272
+    // us a step with drawn tiles, 48 ragged ones 149 -> 130.  Drawn are the
+    // tiles of two-stage rings, where there are more than the CTAs' first two
+    // (asked for at run time the draws cost lattices without any 4 %: 512 x 512
+    // FP32 7.98 -> 8.39 us).  A deeper ring evens the SMs out by itself and its
+    // one copy warp per SM has no time for the draws (SRT FP16 144 -> 208 us).
+    static_assert(!DRAWS || NS == 2, "two-stage rings draw");
+    constexpr bool draws = DRAWS;  // (the host sees to NS * G < ntiles)
     const int ntl = (args.ntiles > (int)blockIdx.x) ? (args.ntiles - 1 - (int)blockIdx.x) / G + 1 : 0;
 
     if (tid == 0) {
@@ -518,7 +512,7 @@ __global__ void __launch_bounds__(NTHREADS + 32, NTHREADS + 32 >= 512 ? 1 : LBM_
         // what every unit needs; the boundary data (bc, strides, lid) is read
         // by the edge units only
         const StageParams& p = params[st];
-        if (DRAWS && p.X == 0) break;  // no further tile
+        if (draws && p.X == 0) break;  // no further tile
         const int x0 = p.x0, y0 = p.y0, nx = p.in.nx, ny = p.in.ny;
         unsigned char* sb = reinterpret_cast<unsigned char*>(stage_base + (size_t)st * TS::STAGE_ELEMS);
         const int lgX = 31 - __clz(p.X);   // log2 of the tile width X
@@ -674,25 +668,30 @@ __global__ void __launch_bounds__(NTHREADS + 32, NTHREADS + 32 >= 512 ? 1 : LBM_
 
 // The TMA-staged D2Q9 kernel for a collision rule and tile geometry VARIANT
 // (0: large tiles, 1: small tiles, 2: wide CTAs, 3: deep ring, see
-// smem_tile_nodes);
+// smem_tile_nodes), with drawn or dealt tiles;
 // *smem_bytes receives its dynamic shared memory size.
-template <typename S, int VARIANT>
-const void* pick_step_kernel_smem(int collision, size_t* smem_bytes) {
-    constexpr int TN = smem_tile_nodes(sizeof(S) == 4 ? 1 : 2, VARIANT);  // 1: FP32 storage
-    constexpr int NS = VARIANT == 1   ? LBM_SMEM_STAGES_SMALL
-                     : VARIANT == 3 ? (sizeof(S) == 2 ? LBM_SMEM_STAGES_DEEP2 : LBM_SMEM_STAGES_DEEP)
-                                    : LBM_SMEM_STAGES;
+template <typename S, int VARIANT, bool DRAWS>
+const void* pick_step_kernel_smem_tiles(int collision, size_t* smem_bytes) {
+    constexpr int ST = sizeof(S) == 4 ? 1 : 2;  // 1: FP32 storage
+    constexpr int TN = smem_tile_nodes(ST, VARIANT), NS = smem_stages(ST, VARIANT);
     constexpr int NT = smem_threads(VARIANT);
     using TS = SmemTile<S, TN, NS, NT>;
     *smem_bytes = TS::SMEM_BYTES;
     switch (collision) {
-        case COLL_MINXENT4: return (const void*)&step_kernel_smem<S, COLL_MINXENT4, TN, NS, NT>;
-        case COLL_SRT: return (const void*)&step_kernel_smem<S, COLL_SRT, TN, NS, NT>;
-        case COLL_MINXENT2: return (const void*)&step_kernel_smem<S, COLL_MINXENT2, TN, NS, NT>;
+        case COLL_MINXENT4: return (const void*)&step_kernel_smem<S, COLL_MINXENT4, TN, NS, NT, DRAWS>;
+        case COLL_SRT: return (const void*)&step_kernel_smem<S, COLL_SRT, TN, NS, NT, DRAWS>;
+        case COLL_MINXENT2: return (const void*)&step_kernel_smem<S, COLL_MINXENT2, TN, NS, NT, DRAWS>;
         case COLL_MRT:
-        case COLL_TRT: return (const void*)&step_kernel_smem<S, COLL_MRT, TN, NS, NT>;
+        case COLL_TRT: return (const void*)&step_kernel_smem<S, COLL_MRT, TN, NS, NT, DRAWS>;
     }
     return nullptr;
+}
+template <typename S, int VARIANT>
+const void* pick_step_kernel_smem(int collision, bool draws, size_t* smem_bytes) {
+    if constexpr (smem_stages(sizeof(S) == 4 ? 1 : 2, VARIANT) == 2) {
+        if (draws) return pick_step_kernel_smem_tiles<S, VARIANT, true>(collision, smem_bytes);
+    }
+    return pick_step_kernel_smem_tiles<S, VARIANT, false>(collision, smem_bytes);
 }
 
 }  // namespace lbm
