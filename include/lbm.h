@@ -296,7 +296,8 @@ int lbm_status_instance(lbm_ctx* ctx, int32_t instance, int64_t* counters);
  *     are 0.
  *  5  overlapping regions of 64 columns by th rows that take tw steps per
  *     launch in shared memory (D2Q9 with FP32 arithmetic; lattices that do
- *     not fill the GPU).
+ *     not fill the GPU).  Calls and remainders of fewer steps than pay for a
+ *     region's loads and stores run on the fastest of the other kinds.
  * Selection: the create-time autotuner (D2Q9 with FP32 arithmetic: each
  * candidate shape timed over back-to-back launches, the close ones timed
  * again as a captured graph, which decides; the choice is cached per device,
@@ -307,6 +308,12 @@ int lbm_status_instance(lbm_ctx* ctx, int32_t instance, int64_t* counters);
  * 1), "smems" (kind 2), "smemw" (kind 3), "smemd" (kind 4) or "block,tw,th"
  * (kind 5). */
 int lbm_launch_shape(lbm_ctx* ctx, int32_t* out);
+
+/* Step-kernel launches that lbm_step(ctx, n) makes from the present state:
+ * out[0] = all of them (a graph's launches each; the collision that opens a
+ * run included), out[1] = those of a kernel that takes several steps per
+ * launch (D1Q3 and kind 5 of lbm_launch_shape; the others take one). */
+int lbm_step_launches(lbm_ctx* ctx, int64_t n, int64_t* out);
 
 /* Destroy a context (NULL-safe).  Frees library-owned memory only. */
 int lbm_destroy(lbm_ctx* ctx);

@@ -46,6 +46,19 @@ struct Shape {
     bool block() const { return kind == 5; }
 };
 
+// A step kernel ready to launch: its shape, and its tiles' place in the
+// context's tile table.
+struct StepPlan {
+    Shape shape{};
+    const void* kern = nullptr;
+    int grid = 0;
+    size_t smem = 0;  // dynamic shared memory
+    int32_t tile0 = 0, ntiles = 0;
+    int flat_nodes = 0;   // one-node-per-thread kernel: nodes per tile-table entry
+    int halo = 0;         // tube and region kernels: halo nodes, steps per launch
+    int block_warps = 0;  // region kernel: warps of a CTA
+};
+
 Shape default_shape_d2q9(int storage) {
     if (storage == DT_F64) return {1, 32, 1};
     if (storage == DT_F32) return {4, 16, 8};
@@ -186,18 +199,15 @@ struct lbm_ctx {
     CUtensorMapOpaque* d_tmaps = nullptr;  // [buffer][tile | halo][instance]
     unsigned int* d_error = nullptr;
     int tmaps_variant = -1;  // tile variant the TMA tensor maps were built for
-    std::vector<TileDesc> tiles;
     bool initialized = false;
     std::vector<uint8_t> inst_init;  // per-instance initial fields set (lbm_init_batch)
     bool post = false;  // stored field is post-collision
     int64_t steps = 0;
-    Shape shape{};
-    int flat_nodes = 0;  // one-node-per-thread kernel: nodes per tile-table entry
-    int halo = 0;         // tube and region kernels: halo nodes, steps per launch
-    int block_warps = 0;  // region kernel: warps of a CTA
-    const void* kern = nullptr;
-    int grid = 0;
-    size_t smem = 0;  // dynamic shared memory of the step kernel
+    StepPlan plan;
+    // One step per launch, beside a plan that takes several (kern = null where
+    // there is none): launches of less than `plan_from` steps go to it.
+    StepPlan single;
+    int plan_from = 1;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     bool failed = false;
     int spin_limit = 1 << 20;  // polls of one bounded mbarrier wait in the TMA kernel
@@ -275,9 +285,10 @@ int flat_nodes(const lbm_ctx* ctx) {
 bool is_flat(const lbm_ctx* ctx, const Shape& s) {
     return ctx->lattice == 2 && s.kind == 0 && s.V == 1;
 }
-int block_threads(const lbm_ctx* ctx, const Shape& s) {
+int block_threads(const lbm_ctx* ctx, const StepPlan& p) {
+    const Shape& s = p.shape;
     if (s.tma()) return smem_block_threads(s.kind - 1);
-    if (s.block()) return 32 * ctx->block_warps;
+    if (s.block()) return 32 * p.block_warps;
     if (ctx->lattice == 1) return std::max(32, std::min(s.tw * s.th, 256) / 32 * 32);
     return is_flat(ctx, s) ? 32 : s.tw * s.th;
 }
@@ -353,24 +364,26 @@ int64_t block_tiles(const lbm_ctx* ctx, int K, int rows, bool* whole, std::vecto
     return n;
 }
 
-// Steps per launch and region height of a context, or false where the
-// regions are too many for this kernel to be ahead of the TMA kernel (more
+// Steps per launch and region height of a context with their modelled time per
+// step, or false where the regions are too many for this kernel to be ahead of the TMA kernel (more
 // than four per SM).  The modelled time per step, in us: a row of a region
 // holds its scheduler for `unit` (16 warps take 16 rows at a time), a launch
 // adds a region's loads and stores and the launch itself.  The constants fit
 // 512 x 512, 64 x 64, 200 x 200 and 17 x 17 lattices with K = 2 .. 8 and 12 ..
-// 64 rows within 15 %; whether the TMA kernel is ahead is timed.
-bool block_plan(const lbm_ctx* ctx, int* K, int* rows) {
+// 64 rows within 15 %; over 60 lattices of all rules and types the measured
+// time was 0.95 to 1.9 of the modelled one.  Whether the TMA kernel is ahead
+// is timed, unless the model is already behind it.
+bool block_plan(const lbm_ctx* ctx, int* K, int* rows, double* us) {
     const int cap = block_max_rows(ctx->storage);
     const double unit = ctx->collision == LBM_MINXENT4 ? 0.41 : 0.28;
-    double best = 1e30;
+    *us = 1e30;
     auto consider = [&](int r, int steps, double live, int64_t n) {
         const double turns = std::ceil(live / BLOCK_WARPS);
         const double units = std::max(std::ceil(live / 4), turns > 1 ? 4 * (turns - 1) + 2.4 : 0.0);
         const double rounds = std::ceil((double)n / ctx->num_sms);
         const double t = rounds * (units * unit + 0.15 + 2.5 / steps) + 2.0 / steps;
-        if (n <= 4 * ctx->num_sms && n <= ctx->layout.max_tiles && t < best) {
-            best = t;
+        if (n <= 4 * ctx->num_sms && n <= ctx->layout.max_tiles && t < *us) {
+            *us = t;
             *K = steps;
             *rows = r;
         }
@@ -384,10 +397,11 @@ bool block_plan(const lbm_ctx* ctx, int* K, int* rows) {
             const int64_t cut = block_tiles(ctx, k, r, &whole, nullptr);
             if (!whole) consider(r, k, r - k - 1, cut);  // (rows computed, on average)
         }
-    return best < 1e30;
+    return *us < 1e30;
 }
 
-std::vector<TileDesc> build_tiles(const lbm_ctx* ctx, const Shape& s) {
+std::vector<TileDesc> build_tiles(const lbm_ctx* ctx, const StepPlan& p) {
+    const Shape& s = p.shape;
     std::vector<TileDesc> t;
     if (s.block()) {
         bool whole;
@@ -408,7 +422,7 @@ std::vector<TileDesc> build_tiles(const lbm_ctx* ctx, const Shape& s) {
         return t;
     }
     if (ctx->lattice == 1) {
-        const int u = 32 * s.V - 2 * ctx->halo;
+        const int u = 32 * s.V - 2 * p.halo;
         for (int i = 0; i < ctx->count; ++i)
             for (int32_t x = 0; x < ctx->layout.inst[i].nx; x += u) t.push_back({(int32_t)i, x, 0, 0});
         return t;
@@ -418,8 +432,8 @@ std::vector<TileDesc> build_tiles(const lbm_ctx* ctx, const Shape& s) {
         for (int i = 0; i < ctx->count; ++i) {
             const InstDesc& in = ctx->layout.inst[i];
             const int64_t n = flat_fluid(in.nx, in.ny, ctx->bc);
-            for (int64_t k = 0; k < n; k += ctx->flat_nodes)
-                t.push_back({(int32_t)i, (int32_t)k, (int32_t)std::min<int64_t>(k + ctx->flat_nodes, n), 0});
+            for (int64_t k = 0; k < n; k += p.flat_nodes)
+                t.push_back({(int32_t)i, (int32_t)k, (int32_t)std::min<int64_t>(k + p.flat_nodes, n), 0});
         }
         return t;
     }
@@ -441,8 +455,13 @@ int ilog2(int v) {
 
 int build_tensor_maps(lbm_ctx* ctx, int variant);
 
-// Make shape s current: tile table to the device, kernel and grid size.
-int apply_shape(lbm_ctx* ctx, const Shape& s) {
+// The plan of shape s: kernel, grid size, and its tiles to the device's table
+// from entry tile0 on.  halo: tube kernel's.
+int make_plan(lbm_ctx* ctx, const Shape& s, int halo, int32_t tile0, StepPlan* out) {
+    StepPlan p;
+    p.shape = s;
+    p.halo = halo;
+    p.tile0 = tile0;
     const void* k = nullptr;
     size_t smem = 0;
     if (s.block()) {
@@ -457,7 +476,7 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
         else if (ctx->storage == DT_BF16) k = step_kernel_block_bf16(ctx->collision, s.th);
         if (!k) return LBM_ERR_ARG;
         smem = block_smem_bytes(ctx->storage, s.th);
-        ctx->halo = s.tw;
+        p.halo = s.tw;
         LBM_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     } else if (s.kind >= 1) {
         if (ctx->lattice != 2 || ctx->compute != DT_F32 || s.kind > 4) return LBM_ERR_ARG;
@@ -471,25 +490,25 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
         k = find_step_kernel(ctx->lattice, ctx->storage, ctx->collision, s.V);
     }
     if (!k) return LBM_ERR_ARG;
-    if (is_flat(ctx, s)) ctx->flat_nodes = flat_nodes(ctx);
-    std::vector<TileDesc> t = build_tiles(ctx, s);
-    if ((int64_t)t.size() > ctx->layout.max_tiles) return LBM_ERR_ARG;
-    LBM_CK(cudaMemcpyAsync(ctx->d_tiles, t.data(), sizeof(TileDesc) * t.size(),
+    if (is_flat(ctx, s)) p.flat_nodes = flat_nodes(ctx);
+    const std::vector<TileDesc> t = build_tiles(ctx, p);
+    if (tile0 + (int64_t)t.size() > ctx->layout.max_tiles) return LBM_ERR_ARG;
+    LBM_CK(cudaMemcpyAsync(ctx->d_tiles + tile0, t.data(), sizeof(TileDesc) * t.size(),
                            cudaMemcpyHostToDevice, ctx->stream));
     LBM_CK(cudaMemcpyAsync(ctx->d_inst, ctx->layout.inst.data(), sizeof(InstDesc) * ctx->count,
                            cudaMemcpyHostToDevice, ctx->stream));
     LBM_CK(cudaStreamSynchronize(ctx->stream));
     // two CTAs of 8 warps on an SM where there are more regions than SMs
     if (s.block())
-        ctx->block_warps = (int64_t)t.size() > ctx->num_sms && 2 * smem <= 220 * 1024 ? BLOCK_WARPS / 2 : BLOCK_WARPS;
-    const int block = block_threads(ctx, s);
+        p.block_warps = (int64_t)t.size() > ctx->num_sms && 2 * smem <= 220 * 1024 ? BLOCK_WARPS / 2 : BLOCK_WARPS;
+    const int block = block_threads(ctx, p);
     if (is_flat(ctx, s)) {
         // An SM takes as many CTAs as it has room for, so a grid of a few
         // CTAs per SM is dealt unevenly: claim the shared memory that leaves
         // room for an equal share and no more.  Up to four warps per SM, one
         // per scheduler, gain nothing (40 lattices of 17 x 17: 12.6 us either
         // way), and leave their SMs free for other streams' work.
-        const int64_t ctas = (int64_t)t.size() * (ctx->flat_nodes / block);
+        const int64_t ctas = (int64_t)t.size() * (p.flat_nodes / block);
         const int64_t share = (ctas + ctx->num_sms - 1) / ctx->num_sms;
         if (share > 4 && share <= 32) smem = (size_t)(227 * 1024 / share - 1024) / 1024 * 1024;
         LBM_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024));
@@ -499,7 +518,7 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
     per_sm = std::max(per_sm, 1);
     int64_t g = s.block() ? (int64_t)t.size()
                 : ctx->lattice == 1 ? ((int64_t)t.size() * 32 + block - 1) / block
-                : is_flat(ctx, s) ? (int64_t)t.size() * (ctx->flat_nodes / block)
+                : is_flat(ctx, s) ? (int64_t)t.size() * (p.flat_nodes / block)
                                   : std::min<int64_t>((int64_t)per_sm * ctx->num_sms, (int64_t)t.size());
     if (s.tma() && smem_stages(ctx->storage, s.kind - 1) == 2 && 2 * g < (int64_t)t.size()) {
         // more tiles than the CTAs' first two: the others are drawn
@@ -512,16 +531,34 @@ int apply_shape(lbm_ctx* ctx, const Shape& s) {
             g = gd;
         }
     }
-    ctx->tiles.swap(t);
-    ctx->shape = s;
-    ctx->kern = k;
-    ctx->smem = smem;
-    ctx->grid = (int)std::max<int64_t>(g, 1);
+    p.kern = k;
+    p.smem = smem;
+    p.grid = (int)std::max<int64_t>(g, 1);
+    p.ntiles = (int32_t)t.size();
+    *out = p;
+    return LBM_OK;
+}
+
+// Make shape s the context's plan, alone.
+int apply_shape(lbm_ctx* ctx, const Shape& s, int halo = 0) {
+    const int rc = make_plan(ctx, s, halo, 0, &ctx->plan);
+    if (rc != LBM_OK) return rc;
+    ctx->single.kern = nullptr;
+    ctx->plan_from = 1;
     for (int p = 0; p < 2; ++p) {
         if (ctx->graph[p]) cudaGraphExecDestroy(ctx->graph[p]);
         ctx->graph[p] = nullptr;
     }
     return LBM_OK;
+}
+
+// Shape s for single steps beside the plan; launches of `from` steps on stay
+// with the plan.  Where the tile table has no room for both the plan remains
+// alone.
+int add_single(lbm_ctx* ctx, const Shape& s, int from) {
+    const int rc = make_plan(ctx, s, 0, ctx->plan.ntiles, &ctx->single);
+    if (rc == LBM_OK) ctx->plan_from = from;
+    return rc == LBM_ERR_ARG ? LBM_OK : rc;
 }
 
 // TMA tensor maps of both population buffers: per instance a 3-D view
@@ -577,16 +614,16 @@ int build_tensor_maps(lbm_ctx* ctx, int variant) {
     return LBM_OK;
 }
 
-StepArgs step_args(const lbm_ctx* ctx, int src) {
+StepArgs step_args(const lbm_ctx* ctx, const StepPlan& p, int src) {
     StepArgs a;
     a.src = ctx->buf[src];
     a.dst = ctx->buf[1 - src];
     a.inst = ctx->d_inst;
-    a.tiles = ctx->d_tiles;
-    a.ntiles = (int32_t)ctx->tiles.size();
-    a.tw = is_flat(ctx, ctx->shape) ? ctx->flat_nodes : ctx->shape.tw;
-    a.tw_log2 = ctx->shape.tw > 0 ? ilog2(ctx->shape.tw) : 0;
-    a.th = ctx->shape.th;
+    a.tiles = ctx->d_tiles + p.tile0;
+    a.ntiles = p.ntiles;
+    a.tw = is_flat(ctx, p.shape) ? p.flat_nodes : p.shape.tw;
+    a.tw_log2 = p.shape.tw > 0 ? ilog2(p.shape.tw) : 0;
+    a.th = p.shape.th;
     a.rho0 = ctx->rho0;
     a.status = ctx->d_status;
     a.tmaps = ctx->d_tmaps + (size_t)src * 2 * ctx->count;
@@ -598,7 +635,7 @@ StepArgs step_args(const lbm_ctx* ctx, int src) {
     a.lost_tile = ctx->lost_tile;
     a.inplace = 0;
     a.steps = 1;
-    a.halo = ctx->halo;
+    a.halo = p.halo;
     return a;
 }
 
@@ -606,46 +643,46 @@ StepArgs step_args(const lbm_ctx* ctx, int src) {
 // scheduled while the previous kernel in the stream drains, and waits for its
 // completion (griddepcontrol.wait) before touching device state.
 // inplace: the (first) step collides without streaming (one-node-per-thread
-// and tube kernels only); steps: time steps of the launch (tube kernel only).
-cudaError_t launch_step(lbm_ctx* ctx, int src, cudaStream_t s, bool inplace = false, int steps = 1) {
-    StepArgs a = step_args(ctx, src);
+// and tube kernels only); steps: time steps of the launch (tube and region
+// kernels only).
+cudaError_t launch_step(lbm_ctx* ctx, const StepPlan& p, int src, cudaStream_t s, bool inplace = false,
+                        int steps = 1) {
+    StepArgs a = step_args(ctx, p, src);
     a.inplace = inplace ? 1 : 0;
     a.steps = steps;
     void* params[] = {&a};
-    const int block = block_threads(ctx, ctx->shape);
+    const int block = block_threads(ctx, p);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctx->grid);
+    cfg.gridDim = dim3(p.grid);
     cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = ctx->smem;
+    cfg.dynamicSmemBytes = p.smem;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelExC(&cfg, ctx->kern, params);
+    return cudaLaunchKernelExC(&cfg, p.kern, params);
 }
 
-// Median of three timed launches of the current shape (after one untimed
-// launch) on the rest-state buffers, in milliseconds; < 0 on a CUDA error.
-float time_current_shape(lbm_ctx* ctx, cudaEvent_t* ev) {
-    // one warm-up launch, then twice three back-to-back launches (as the
-    // step loop runs them: a launch's tail overlaps the next one's start);
-    // the faster of the two, per launch
-    const int steps = ctx->shape.block() ? ctx->halo : 1;  // of a launch
-    if (launch_step(ctx, 0, ctx->stream, false, steps) != cudaSuccess) return -1.f;
+// Time of a launch of `steps` steps of the current plan in milliseconds, on
+// the rest-state buffers: after an untimed launch twice three back-to-back
+// launches (as the step loop runs them: a launch's tail overlaps the next
+// one's start), the faster of the two; < 0 on a CUDA error.
+float time_current_shape(lbm_ctx* ctx, cudaEvent_t* ev, int steps = 1) {
+    if (launch_step(ctx, ctx->plan, 0, ctx->stream, false, steps) != cudaSuccess) return -1.f;
     int src = 1;
     float t[2];
     for (int r = 0; r < 2; ++r) {
         if (cudaEventRecord(ev[2 * r], ctx->stream) != cudaSuccess) return -1.f;
         for (int k = 0; k < 3; ++k, src ^= 1)
-            if (launch_step(ctx, src, ctx->stream, false, steps) != cudaSuccess) return -1.f;
+            if (launch_step(ctx, ctx->plan, src, ctx->stream, false, steps) != cudaSuccess) return -1.f;
         if (cudaEventRecord(ev[2 * r + 1], ctx->stream) != cudaSuccess) return -1.f;
     }
     if (cudaEventSynchronize(ev[3]) != cudaSuccess) return -1.f;
     for (int r = 0; r < 2; ++r)
         if (cudaEventElapsedTime(&t[r], ev[2 * r], ev[2 * r + 1]) != cudaSuccess) return -1.f;
-    return std::min(t[0], t[1]) / (3.f * steps);
+    return std::min(t[0], t[1]) / 3.f;
 }
 
 // The same timing through a captured graph of four launches, as the step
@@ -657,9 +694,8 @@ float time_current_shape_graph(lbm_ctx* ctx, cudaEvent_t* ev) {
     if (cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
         return -1.f;
     bool ok = true;
-    const int steps = ctx->shape.block() ? ctx->halo : 1;
     for (int k = 0; k < 4; ++k)
-        ok = ok && launch_step(ctx, k & 1, ctx->capture_stream, false, steps) == cudaSuccess;
+        ok = ok && launch_step(ctx, ctx->plan, k & 1, ctx->capture_stream) == cudaSuccess;
     if (cudaStreamEndCapture(ctx->capture_stream, &graph) != cudaSuccess || !ok) return -1.f;
     cudaGraphExec_t g = nullptr;
     const cudaError_t e = cudaGraphInstantiate(&g, graph, 0);
@@ -675,13 +711,14 @@ float time_current_shape_graph(lbm_ctx* ctx, cudaEvent_t* ev) {
     for (int r = 0; r < 2 && ok; ++r)
         ok = cudaEventElapsedTime(&t[r], ev[2 * r], ev[2 * r + 1]) == cudaSuccess;
     cudaGraphExecDestroy(g);
-    return ok ? std::min(t[0], t[1]) / (4.f * steps) : -1.f;
+    return ok ? std::min(t[0], t[1]) / 4.f : -1.f;
 }
 
 // Autotuner cache: the chosen shape per (device, lattice, types, rule,
 // boundary, instance sizes).  Kept for the life of the process, and in the
 // text file named by LBM_AUTOTUNE_CACHE when that variable is set (one line
-// per key: "<key> V tw th kind"), so that a later process -- a profiler run,
+// per key: "<key> V tw th kind"; for the region kernel also "<key>/single" with
+// the shape beside it and "<key>/from" with its shortest launch), so that a later process -- a profiler run,
 // for instance -- takes the same shape without timing anything.
 std::mutex g_tune_mu;
 std::map<std::string, Shape>& tune_cache() {
@@ -753,22 +790,26 @@ void tune_store(const std::string& key, const Shape& s) {
 
 // Keep the fastest candidate shape: each is timed over back-to-back
 // launches on the rest-state buffers (the collision's instruction stream
-// does not depend on the data); the ones within 5 % of the fastest are
-// timed again in a captured graph, which decides.  Then the buffers and
-// counters are cleared.  A shape found in the cache is applied without
+// does not depend on the data); close ones are
+// timed again in a captured graph, which decides.  Where the region kernel
+// takes less for its steps, it becomes the plan, and the fastest shape
+// with one step per launch stays beside it for calls and remainders of fewer
+// steps than pay for a region's loads and stores.  Then the buffers and
+// counters are cleared.  Shapes found in the cache are applied without
 // timing.
 int autotune(lbm_ctx* ctx) {
     const std::string key = tune_key(ctx);
-    Shape cached;
-    if (tune_lookup(key, &cached) && apply_shape(ctx, cached) == LBM_OK) return LBM_OK;
-    std::vector<Shape> cands = candidate_shapes(ctx->storage);
-    int K, rows;
-    if (ctx->storage != DT_F64 && block_plan(ctx, &K, &rows)) cands.push_back({2, K, rows, 5});
+    Shape best_s{}, one{}, from{};  // from.V: steps of the shortest launch of the region kernel
+    if (tune_lookup(key, &best_s) &&
+        (!best_s.block() || (tune_lookup(key + "/single", &one) && tune_lookup(key + "/from", &from))) &&
+        apply_shape(ctx, best_s) == LBM_OK)
+        return best_s.block() ? add_single(ctx, one, std::min(std::max(from.V, 1), ctx->plan.halo)) : LBM_OK;
+    const std::vector<Shape> cands = candidate_shapes(ctx->storage);
     if (cands.size() == 1) return apply_shape(ctx, cands[0]);
     cudaEvent_t ev[6];
     for (int i = 0; i < 6; ++i) LBM_CK(cudaEventCreate(&ev[i]));
     float best = 1e30f;
-    Shape best_s = default_shape_d2q9(ctx->storage);
+    best_s = default_shape_d2q9(ctx->storage);
     int rc = LBM_OK;
     std::vector<float> t(cands.size(), -1.f);
     for (size_t c = 0; c < cands.size(); ++c) {
@@ -781,31 +822,63 @@ int autotune(lbm_ctx* ctx) {
         t[c] = ms;
         best = std::min(best, ms);
     }
-    // The candidates within 5 % of the fastest are timed once more, after
-    // the others, through a captured graph as the step loop runs them, and
-    // that time decides between them.  Below 20 us a single launch is mostly
-    // launch (7.1 us where the graph takes 5.8), so there the margin is wider.
-    const float margin = best < 0.02f ? 1.6f : 1.05f;
-    std::vector<float> tg(cands.size(), -1.f);
-    for (size_t c = 0; c < cands.size() && rc == LBM_OK; ++c) {
-        if (t[c] < 0.f || t[c] > margin * best) continue;
-        if (apply_shape(ctx, cands[c]) != LBM_OK) continue;
-        const float ms = time_current_shape_graph(ctx, ev);
-        if (ms < 0.f) {
-            rc = LBM_ERR_CUDA;
-            break;
-        }
-        tg[c] = ms;
+    // The region kernel, unless its model leaves it no chance: a launch of k
+    // steps takes t1 + (k - 1) slope.
+    int K = 0, rows = 0;
+    double us = 0.0;
+    float tK = -1.f, t1 = -1.f;
+    if (rc == LBM_OK && block_plan(ctx, &K, &rows, &us) && us < 1e3 * best &&
+        apply_shape(ctx, Shape{2, K, rows, 5}) == LBM_OK) {
+        tK = time_current_shape(ctx, ev, K);
+        t1 = time_current_shape(ctx, ev, 1);
+        if (tK < 0.f || t1 < 0.f) rc = LBM_ERR_CUDA;
     }
-    best = 1e30f;
+    // Candidates within 5 % of the fastest are timed once more, after the
+    // others, through a captured graph as the step loop runs them, and
+    // that time decides between them; so is the fastest where the region
+    // kernel comes close (a graph takes 0.8 to 1 of single launches' time).
+    const bool close_region = tK >= 0.75f * K * best && tK < K * best;
+    int near = 0;
     for (size_t c = 0; c < cands.size(); ++c) {
-        if (getenv("LBM_DEBUG"))
-            fprintf(stderr, "liblbm: autotune kind %d V %d tw %d th %d: %.4f ms per launch, %.4f in a graph\n",
-                    cands[c].kind, cands[c].V, cands[c].tw, cands[c].th, t[c], tg[c]);
-        if (tg[c] >= 0.f && tg[c] < best) {  // only the close call's graph times compete
-            best = tg[c];
-            best_s = cands[c];
+        near += t[c] >= 0.f && t[c] <= 1.05f * best;
+        if (t[c] == best) best_s = cands[c];
+    }
+    float fastest = best;  // of one step per launch
+    if (near > 1 || close_region) {
+        fastest = 1e30f;
+        for (size_t c = 0; c < cands.size() && rc == LBM_OK; ++c) {
+            if (t[c] < 0.f || t[c] > 1.05f * best) continue;
+            if (apply_shape(ctx, cands[c]) != LBM_OK) continue;
+            const float ms = time_current_shape_graph(ctx, ev);
+            if (ms < 0.f) {
+                rc = LBM_ERR_CUDA;
+                break;
+            }
+            if (getenv("LBM_DEBUG"))
+                fprintf(stderr, "liblbm: autotune kind %d: %.4f ms in a graph\n", cands[c].kind, ms);
+            if (ms < fastest) {
+                fastest = ms;
+                best_s = cands[c];
+            }
         }
+    }
+    one = best_s;
+    if (rc == LBM_OK && tK >= 0.f && tK < K * fastest) {
+        // The region kernel takes launches of the steps from which on it is
+        // ahead by a tenth of single steps, whose time in a row is
+        // 0.8 of what was timed.
+        best_s = {2, K, rows, 5};
+        const float slope = (tK - t1) / (K - 1);
+        from = {1, 0, 0};
+        while (from.V < K && t1 + (from.V - 1) * slope > 0.9f * 0.8f * from.V * best) ++from.V;
+    }
+    if (getenv("LBM_DEBUG")) {
+        for (size_t c = 0; c < cands.size(); ++c)
+            fprintf(stderr, "liblbm: autotune kind %d V %d tw %d th %d: %.4f ms per launch\n", cands[c].kind,
+                    cands[c].V, cands[c].tw, cands[c].th, t[c]);
+        if (tK >= 0.f)
+            fprintf(stderr, "liblbm: autotune regions of %d rows: 1 step %.4f ms, %d steps %.4f ms (%.4f modelled), "
+                    "used from %d\n", rows, t1, K, tK, 1e-3 * K * us, best_s.block() ? from.V : 0);
     }
     for (int i = 0; i < 6; ++i) cudaEventDestroy(ev[i]);
     if (rc != LBM_OK) {
@@ -817,6 +890,11 @@ int autotune(lbm_ctx* ctx) {
     LBM_CK(cudaMemsetAsync(ctx->d_status, 0, sizeof(unsigned long long) * 2 * ctx->count,
                            ctx->stream));
     rc = apply_shape(ctx, best_s);
+    if (rc == LBM_OK && best_s.block()) {
+        rc = add_single(ctx, one, from.V);
+        tune_store(key + "/single", one);
+        tune_store(key + "/from", from);
+    }
     if (rc == LBM_OK) tune_store(key, best_s);
     return rc;
 }
@@ -825,7 +903,7 @@ int autotune(lbm_ctx* ctx) {
 // upload the executable graphs, so that no capture or first-launch upload
 // happens inside a later lbm_step.
 int capture_graphs(lbm_ctx* ctx) {
-    if (ctx->shape.block()) return LBM_OK;  // several steps per launch: no graph
+    if (ctx->plan.shape.block()) return LBM_OK;  // several steps per launch: no graph
     for (int p = 0; p < 2; ++p) {
         cudaGraphExec_t& g = ctx->graph[p];
         if (g) continue;
@@ -833,7 +911,7 @@ int capture_graphs(lbm_ctx* ctx) {
         LBM_CK(cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal));
         int src = p;
         for (int k = 0; k < GRAPH_STEPS; ++k) {
-            cudaError_t e = launch_step(ctx, src, ctx->capture_stream);
+            cudaError_t e = launch_step(ctx, ctx->plan, src, ctx->capture_stream);
             if (e != cudaSuccess) {
                 cudaStreamEndCapture(ctx->capture_stream, &graph);
                 LBM_CK(e);
@@ -847,6 +925,19 @@ int capture_graphs(lbm_ctx* ctx) {
         LBM_CK(cudaGraphUpload(g, ctx->stream));
     }
     return LBM_OK;
+}
+
+// The plan takes several steps per launch (tube and region kernels).
+bool takes_several(const lbm_ctx* ctx) { return ctx->lattice == 1 || ctx->plan.shape.block(); }
+
+// The next launch of a call with n steps left, of *k steps (post: the stored
+// field is post-collision).
+const StepPlan& next_launch(const lbm_ctx* ctx, bool post, int64_t n, int* k) {
+    *k = 1;
+    if (!takes_several(ctx) || (!post && ctx->lattice == 2)) return ctx->plan;
+    if (post && n < ctx->plan_from) return ctx->single;
+    *k = (int)std::min<int64_t>(n, ctx->plan.halo);
+    return ctx->plan;
 }
 
 bool parse_shape_env(Shape* s) {
@@ -1170,8 +1261,9 @@ int lbm_create_batch(lbm_ctx** out, lbm_lattice lat, int32_t count, const int64_
         // and the CTA size)
         int V = 0;
         const bool pinned = parse_shape_env(&s);
-        tube_plan(ctx, pinned ? s.V : 0, &V, &ctx->halo);
-        rc = apply_shape(ctx, pinned ? s : Shape{V, 128, 1});
+        int halo = 0;
+        tube_plan(ctx, pinned ? s.V : 0, &V, &halo);
+        rc = apply_shape(ctx, pinned ? s : Shape{V, 128, 1}, halo);
     } else if (parse_shape_env(&s)) rc = apply_shape(ctx, s);
     else if (o.autotune && !getenv("LBM_NO_AUTOTUNE")) rc = autotune(ctx);
     else rc = apply_shape(ctx, default_shape_d2q9(o.storage));
@@ -1244,51 +1336,48 @@ int lbm_step(lbm_ctx* ctx, int64_t n) {
     if (ctx->failed) return LBM_ERR_CUDA;
     if (!ctx->initialized) return LBM_ERR_STATE;
     if (n == 0) return LBM_OK;
-    if (ctx->lattice == 1) {
-        while (n > 0) {
-            const int k = (int)std::min<int64_t>(n, ctx->halo);
-            LBM_CK(launch_step(ctx, ctx->cur, ctx->stream, !ctx->post, k));
-            ctx->cur = 1 - ctx->cur;
-            ctx->post = true;
-            ctx->steps += k;
-            n -= k;
+    while (n > 0) {
+        if (ctx->lattice == 2 && ctx->post && !takes_several(ctx) && n >= GRAPH_STEPS) {
+            cudaGraphExec_t& g = ctx->graph[ctx->cur];
+            if (!g) {
+                const int rc = capture_graphs(ctx);
+                if (rc != LBM_OK) return rc;
+            }
+            LBM_CK(cudaGraphLaunch(g, ctx->stream));
+            n -= GRAPH_STEPS;
+            ctx->steps += GRAPH_STEPS;
+            continue;
         }
-        return LBM_OK;
-    }
-    if (!ctx->post) {
-        if (is_flat(ctx, ctx->shape)) {
-            LBM_CK(launch_step(ctx, ctx->cur, ctx->stream, true));
-        } else {
+        int k;
+        const StepPlan& p = next_launch(ctx, ctx->post, n, &k);
+        if (!ctx->post && ctx->lattice == 2 && !is_flat(ctx, p.shape)) {
             AuxArgs a = aux_args(ctx);
             LBM_CK(run_aux(AuxOp::CollideInPlace, a, ctx->buf[ctx->cur], ctx->buf[1 - ctx->cur],
                            nullptr, nullptr, nullptr, nullptr, nullptr, nullptr));
+        } else {
+            LBM_CK(launch_step(ctx, p, ctx->cur, ctx->stream, !ctx->post, k));
         }
         ctx->cur = 1 - ctx->cur;
         ctx->post = true;
-        ctx->steps += 1;
-        --n;
-    }
-    while (ctx->shape.block() && n > 0) {
-        const int k = (int)std::min<int64_t>(n, ctx->halo);
-        LBM_CK(launch_step(ctx, ctx->cur, ctx->stream, false, k));
-        ctx->cur = 1 - ctx->cur;
         ctx->steps += k;
         n -= k;
     }
-    while (n >= GRAPH_STEPS) {
-        cudaGraphExec_t& g = ctx->graph[ctx->cur];
-        if (!g) {
-            const int rc = capture_graphs(ctx);
-            if (rc != LBM_OK) return rc;
-        }
-        LBM_CK(cudaGraphLaunch(g, ctx->stream));
-        n -= GRAPH_STEPS;
-        ctx->steps += GRAPH_STEPS;
-    }
-    for (; n > 0; --n) {
-        LBM_CK(launch_step(ctx, ctx->cur, ctx->stream));
-        ctx->cur = 1 - ctx->cur;
-        ctx->steps += 1;
+    return LBM_OK;
+}
+
+int lbm_step_launches(lbm_ctx* ctx, int64_t n, int64_t* out) {
+    if (!ctx || n < 0 || !out) return LBM_ERR_ARG;
+    out[0] = out[1] = 0;
+    bool post = ctx->post;
+    while (n > 0) {
+        int k;
+        const StepPlan& p = next_launch(ctx, post, n, &k);
+        // the same launch again and again, but for the first one and the remainder
+        const int64_t m = post ? n / k : 1;
+        out[0] += m;
+        if (takes_several(ctx) && &p == &ctx->plan && (post || ctx->lattice == 1)) out[1] += m;
+        post = true;
+        n -= m * k;
     }
     return LBM_OK;
 }
@@ -1540,6 +1629,9 @@ int lbm_save_state(lbm_ctx* ctx, void* host_buf) {
     h.buf_bytes = ctx->cv.buf_bytes;
     char* out = static_cast<char*>(host_buf);
     std::memcpy(out, &h, sizeof h);
+    AuxArgs a = aux_args(ctx);
+    LBM_CK(run_aux(AuxOp::ClearPadding, a, nullptr, ctx->buf[ctx->cur], nullptr, nullptr, nullptr,
+                   nullptr, nullptr, nullptr));
     LBM_CK(cudaMemcpyAsync(out + sizeof h, ctx->d_status, h.status_bytes, cudaMemcpyDeviceToHost,
                            ctx->stream));
     LBM_CK(cudaMemcpyAsync(out + sizeof h + h.status_bytes, ctx->buf[ctx->cur], h.buf_bytes,
@@ -1575,11 +1667,11 @@ int lbm_load_state(lbm_ctx* ctx, const void* host_buf) {
 
 int lbm_launch_shape(lbm_ctx* ctx, int32_t* out) {
     if (!ctx || !out) return LBM_ERR_ARG;
-    out[0] = ctx->shape.V;
-    out[1] = ctx->shape.tw;
-    out[2] = ctx->shape.th;
-    out[3] = ctx->grid;
-    out[4] = ctx->shape.kind;
+    out[0] = ctx->plan.shape.V;
+    out[1] = ctx->plan.shape.tw;
+    out[2] = ctx->plan.shape.th;
+    out[3] = ctx->plan.grid;
+    out[4] = ctx->plan.shape.kind;
     return LBM_OK;
 }
 

@@ -470,6 +470,21 @@ gather_f_kernel(const S* src, const InstDesc* insts, bool pulled, double rho0, d
     }
 }
 
+// The columns [nx, pitch) of every row and plane to zero.  Nothing reads them,
+// but the TMA kernel's stores, clipped at 16 bytes, leave values there where
+// the other step kernels do not, and a saved state is to be the same whichever
+// kernels took its steps.
+template <class Lat, typename S>
+__global__ void __launch_bounds__(AUX_THREADS) clear_padding_kernel(S* dst, const InstDesc* insts) {
+    const InstDesc& in = insts[blockIdx.y];
+    const int pad = in.pitch - in.nx;
+    const int64_t n = (int64_t)pad * in.ny * Lat::Q;
+    for (int64_t k = (int64_t)blockIdx.x * AUX_THREADS + threadIdx.x; k < n; k += (int64_t)gridDim.x * AUX_THREADS) {
+        const int64_t row = k / pad, a = row / in.ny, y = row - a * in.ny;
+        dst[in.off + a * in.plane + y * in.pitch + in.nx + (k - row * pad)] = zero_value<S>();
+    }
+}
+
 // Stream function of the LDAS post-processing (Sec. IV.I) along each row of
 // each instance: psi(x, y) = - integral_0^x u_y dx in lattice units, with
 // the composite Simpson rule over pairs of unit intervals from the left
@@ -949,6 +964,12 @@ cudaError_t aux_dispatch(AuxOp op, const AuxArgs& a, const void* src, void* dst,
             gather_f_kernel<Lat, S><<<g, AUX_THREADS, 0, a.stream>>>(static_cast<const S*>(src), a.inst,
                                                                      a.pulled, a.rho0, o0, per);
             break;
+        case AuxOp::ClearPadding: {
+            const int64_t most = (int64_t)7 * a.max_ny * Lat::Q;  // rows are padded to a multiple of 8
+            const dim3 blocks((unsigned)std::min<int64_t>((most + AUX_THREADS - 1) / AUX_THREADS, 1024), (unsigned)a.count);
+            clear_padding_kernel<Lat, S><<<blocks, AUX_THREADS, 0, a.stream>>>(static_cast<S*>(dst), a.inst);
+            break;
+        }
         case AuxOp::StreamFunction:
             if constexpr (Lat::Q == 9) {
                 // a warp per row

@@ -34,7 +34,7 @@ __host__ __device__ inline int cons_split(int64_t nodes) {
 // the two counters of the TMA kernel's drawn tiles.
 constexpr int TILE_COUNTERS = 8, ERROR_WORDS = 16;
 
-enum class AuxOp { Init, SetF, CollideInPlace, Moments, GatherF, StreamFunction, Conservation };
+enum class AuxOp { Init, SetF, CollideInPlace, Moments, GatherF, StreamFunction, Conservation, ClearPadding };
 
 struct AuxArgs {
     int lattice;   // 1 = D1Q3, 2 = D2Q9
@@ -61,6 +61,7 @@ struct AuxArgs {
 // CollideInPlace: dst <- collide(src) without streaming
 // Moments:        o0, o1, o2 <- rho, ux, uy of f(t_n) read from src
 // GatherF:        o0 <- FP64 populations of f(t_n)
+// ClearPadding:   columns of dst beyond each instance's own to deviation 0
 // StreamFunction: o0 <- stream function of f(t_n) (D2Q9), [inst][y][x]
 // Conservation:   o0 <- per-instance totals (3 doubles each), o1 = partials scratch
 //                 (count * CONS_PARTIALS * 3 doubles; partial b of instance i at

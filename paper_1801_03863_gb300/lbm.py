@@ -39,7 +39,7 @@ EXPORTS = (
     "lbm_stream_function", "lbm_stream_function_device",
     "lbm_conservation_noalloc", "lbm_status",
     "lbm_status_instance",
-    "lbm_launch_shape", "lbm_destroy", "lbm_status_string",
+    "lbm_launch_shape", "lbm_step_launches", "lbm_destroy", "lbm_status_string",
     "lbm_init_batch", "lbm_moments_batch", "lbm_moments_batch_device",
     "lbm_stream_function_batch", "lbm_state_bytes", "lbm_save_state", "lbm_load_state",
 )
@@ -101,6 +101,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
             "lbm_status": (ctypes.c_int, [P, P]),
             "lbm_status_instance": (ctypes.c_int, [P, I32, P]),
             "lbm_launch_shape": (ctypes.c_int, [P, P]),
+            "lbm_step_launches": (ctypes.c_int, [P, ctypes.c_int64, P]),
             "lbm_destroy": (ctypes.c_int, [P]),
             "lbm_status_string": (ctypes.c_char_p, [ctypes.c_int]),
             "lbm_init_batch": (ctypes.c_int, [P, I32, P, P, P]),
@@ -258,6 +259,12 @@ def lbm_launch_shape(h) -> dict:
     return {"V": int(c[0]), "tw": int(c[1]), "th": int(c[2]), "grid": int(c[3]),
             "kind": {0: "chunks", 1: "smem", 2: "smem_small", 3: "smem_wide",
                      4: "smem_deep", 5: "block"}[int(c[4])]}
+
+
+def lbm_step_launches(h, n: int) -> dict:
+    c = np.zeros(2, dtype=np.int64)
+    _check(load().lbm_step_launches(h, int(n), _p(c)), "lbm_step_launches")
+    return {"launches": int(c[0]), "of_several_steps": int(c[1])}
 
 
 def lbm_init_batch(h, instance: int, rho, ux=None, uy=None) -> None:
@@ -454,6 +461,9 @@ class Lattice:
 
     def launch_shape(self) -> dict:
         return lbm_launch_shape(self._h)
+
+    def step_launches(self, n: int) -> dict:
+        return lbm_step_launches(self._h, n)
 
     def split(self, flat: np.ndarray, per_node: int = 1):
         """Split concatenated per-node arrays into per-instance [ny, nx] arrays."""
