@@ -22,7 +22,9 @@ OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "liblbm.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE]
+# --no-compress: nvcc compresses device code beyond some 10 MB a file, which
+# costs the first context of a storage type 10 ms to unpack
+NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--no-compress", "-Xcompiler", "-fPIC", "-I", INCLUDE]
 
 
 def nvcc() -> str:

@@ -374,6 +374,8 @@ int64_t block_tiles(const lbm_ctx* ctx, int K, int rows, bool* whole, std::vecto
 // time was 0.95 to 1.9 of the modelled one.  Whether the TMA kernel is ahead
 // is timed, unless the model is already behind it.
 bool block_plan(const lbm_ctx* ctx, int* K, int* rows, double* us) {
+    const int64_t most = std::min<int64_t>(4 * ctx->num_sms, ctx->layout.max_tiles);
+    if (ctx->count > most) return false;
     const int cap = block_max_rows(ctx->storage);
     const double unit = ctx->collision == LBM_MINXENT4 ? 0.41 : 0.28;
     *us = 1e30;
@@ -382,7 +384,7 @@ bool block_plan(const lbm_ctx* ctx, int* K, int* rows, double* us) {
         const double units = std::max(std::ceil(live / 4), turns > 1 ? 4 * (turns - 1) + 2.4 : 0.0);
         const double rounds = std::ceil((double)n / ctx->num_sms);
         const double t = rounds * (units * unit + 0.15 + 2.5 / steps) + 2.0 / steps;
-        if (n <= 4 * ctx->num_sms && n <= ctx->layout.max_tiles && t < *us) {
+        if (n <= most && t < *us) {
             *us = t;
             *K = steps;
             *rows = r;
@@ -392,11 +394,18 @@ bool block_plan(const lbm_ctx* ctx, int* K, int* rows, double* us) {
     const int tall = (int)std::min<int64_t>(ctx->layout.max_ny, cap);
     const int64_t n = block_tiles(ctx, 0, tall, &whole, nullptr);
     if (whole) consider(tall, BLOCK_WHOLE_STEPS, tall, n);
-    for (int k = 2; k <= 8; k += 2)
-        for (int r = 2 * k + 1; r <= cap; ++r) {
-            const int64_t cut = block_tiles(ctx, k, r, &whole, nullptr);
-            if (!whole) consider(r, k, r - k - 1, cut);  // (rows computed, on average)
+    for (int k = 2; k <= 8; k += 2) {
+        // from the highest regions down, until there are too many
+        std::vector<int64_t> cut(cap + 1, -1);  // by rows; -1: uncut or too many
+        int r = cap;
+        for (; r > 2 * k; --r) {
+            const int64_t m = block_tiles(ctx, k, r, &whole, nullptr);
+            if (m > most) break;
+            if (!whole) cut[r] = m;
         }
+        for (++r; r <= cap; ++r)
+            if (cut[r] >= 0) consider(r, k, r - k - 1, cut[r]);  // (rows computed, on average)
+    }
     return *us < 1e30;
 }
 
