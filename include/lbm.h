@@ -282,7 +282,8 @@ int lbm_status_instance(lbm_ctx* ctx, int32_t instance, int64_t* counters);
  *  0  D2Q9: register-chunk kernel; with out[0] = 1 the FP64 kernel with one
  *     node per thread (warps of 32 consecutive nodes, tw = 32, th = 1).
  *     D1Q3: the tube kernel, out[0] nodes per lane, tw x th threads a CTA,
- *     several steps per launch; both follow from the sizes.
+ *     several steps per launch; both follow from the sizes.  (With FP32
+ *     arithmetic a kernel of its own takes calls and remainders of one step.)
  *  1 to 4  the TMA-staged D2Q9 kernel, whose CTAs have one warp that only
  *     moves tiles in and out of shared memory besides the colliding warps.
  *     1: large tiles, 8-warp CTAs, 1792 nodes for 2-byte storage or 896 for

@@ -38,12 +38,14 @@ size_t dtype_bytes(int dt) { return dt == DT_F64 ? 8 : (dt == DT_F32 ? 4 : 2); }
 // regions of th rows.
 // Kind 0 with V = 1 on D2Q9 is the FP64 kernel with one node per thread
 // (warps of 32 consecutive nodes: tw = 32, th = 1).  On D1Q3 kind 0 is the
-// tube kernel: V nodes per lane, tw x th threads per CTA.
+// tube kernel: V nodes per lane, tw x th threads per CTA.  Kind 6: the
+// register-chunk kernel on D1Q3, for single steps beside the tube kernel.
 struct Shape {
     int V, tw, th;
     int kind = 0;
     bool tma() const { return kind >= 1 && kind <= 4; }
     bool block() const { return kind == 5; }
+    bool single_tube() const { return kind == 6; }
 };
 
 // A step kernel ready to launch: its shape, and its tiles' place in the
@@ -289,6 +291,7 @@ int block_threads(const lbm_ctx* ctx, const StepPlan& p) {
     const Shape& s = p.shape;
     if (s.tma()) return smem_block_threads(s.kind - 1);
     if (s.block()) return 32 * p.block_warps;
+    if (s.single_tube()) return s.tw;
     if (ctx->lattice == 1) return std::max(32, std::min(s.tw * s.th, 256) / 32 * 32);
     return is_flat(ctx, s) ? 32 : s.tw * s.th;
 }
@@ -417,7 +420,7 @@ std::vector<TileDesc> build_tiles(const lbm_ctx* ctx, const StepPlan& p) {
         block_tiles(ctx, s.tw, s.th, &whole, &t);
         return t;
     }
-    if (s.kind >= 1) {
+    if (s.tma()) {
         for (int i = 0; i < ctx->count; ++i) {
             const InstDesc& in = ctx->layout.inst[i];
             const int tn = smem_tile_nodes(ctx->storage, s.kind - 1);
@@ -430,7 +433,7 @@ std::vector<TileDesc> build_tiles(const lbm_ctx* ctx, const StepPlan& p) {
         }
         return t;
     }
-    if (ctx->lattice == 1) {
+    if (ctx->lattice == 1 && !s.single_tube()) {
         const int u = 32 * s.V - 2 * p.halo;
         for (int i = 0; i < ctx->count; ++i)
             for (int32_t x = 0; x < ctx->layout.inst[i].nx; x += u) t.push_back({(int32_t)i, x, 0, 0});
@@ -487,8 +490,13 @@ int make_plan(lbm_ctx* ctx, const Shape& s, int halo, int32_t tile0, StepPlan* o
         smem = block_smem_bytes(ctx->storage, s.th);
         p.halo = s.tw;
         LBM_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    } else if (s.single_tube()) {
+        if (ctx->lattice != 1) return LBM_ERR_ARG;
+        if (ctx->storage == DT_F32) k = step_kernel_single_tube_f32();
+        else if (ctx->storage == DT_F16) k = step_kernel_single_tube_f16();
+        else if (ctx->storage == DT_BF16) k = step_kernel_single_tube_bf16();
     } else if (s.kind >= 1) {
-        if (ctx->lattice != 2 || ctx->compute != DT_F32 || s.kind > 4) return LBM_ERR_ARG;
+        if (ctx->lattice != 2 || ctx->compute != DT_F32 || !s.tma()) return LBM_ERR_ARG;
         k = find_smem_kernel(ctx, s.kind - 1, false, &smem);
         if (!k) return LBM_ERR_ARG;
         LBM_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -526,7 +534,7 @@ int make_plan(lbm_ctx* ctx, const Shape& s, int halo, int32_t tile0, StepPlan* o
     LBM_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
     per_sm = std::max(per_sm, 1);
     int64_t g = s.block() ? (int64_t)t.size()
-                : ctx->lattice == 1 ? ((int64_t)t.size() * 32 + block - 1) / block
+                : ctx->lattice == 1 && !s.single_tube() ? ((int64_t)t.size() * 32 + block - 1) / block
                 : is_flat(ctx, s) ? (int64_t)t.size() * (p.flat_nodes / block)
                                   : std::min<int64_t>((int64_t)per_sm * ctx->num_sms, (int64_t)t.size());
     if (s.tma() && smem_stages(ctx->storage, s.kind - 1) == 2 && 2 * g < (int64_t)t.size()) {
@@ -1273,6 +1281,8 @@ int lbm_create_batch(lbm_ctx** out, lbm_lattice lat, int32_t count, const int64_
         int halo = 0;
         tube_plan(ctx, pinned ? s.V : 0, &V, &halo);
         rc = apply_shape(ctx, pinned ? s : Shape{V, 128, 1}, halo);
+        if (rc == LBM_OK && !pinned && o.compute == DT_F32)
+            rc = add_single(ctx, Shape{o.storage == DT_F32 ? 4 : 8, 128, 1, 6}, 2);
     } else if (parse_shape_env(&s)) rc = apply_shape(ctx, s);
     else if (o.autotune && !getenv("LBM_NO_AUTOTUNE")) rc = autotune(ctx);
     else rc = apply_shape(ctx, default_shape_d2q9(o.storage));

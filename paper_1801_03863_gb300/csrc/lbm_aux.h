@@ -76,6 +76,12 @@ const void* step_kernel_f32(int lattice, int collision, int V);
 const void* step_kernel_f16(int lattice, int collision, int V);
 const void* step_kernel_bf16(int lattice, int collision, int V);
 
+// D1Q3 kernels of one step per launch (4 nodes a thread for FP32 storage, 8 for
+// 2-byte storage).
+const void* step_kernel_single_tube_f32();
+const void* step_kernel_single_tube_f16();
+const void* step_kernel_single_tube_bf16();
+
 // D2Q9 step kernels that take several steps per launch on overlapping regions
 // (lbm_step_block.cuh; FP32 arithmetic): regions of 64 columns and at most
 // block_max_rows rows, CTAs of at most BLOCK_WARPS warps.

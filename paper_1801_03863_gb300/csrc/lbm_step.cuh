@@ -255,6 +255,7 @@ __global__ void __launch_bounds__(256) step_kernel(const StepArgs args) {
                 }
             }
             uint32_t st = Collide<Lat, COLL, CT, (int)sizeof(S)>::run(d, rho0v, rates, o);
+            if constexpr (Q == 3) st = bgk_suspect(st) ? bgk_status(o[0], o[1], o[2], rho0v) : 0u;
             if (cavity_edge) {
 #pragma unroll
                 for (int l = 0; l < P; ++l) {
@@ -608,6 +609,15 @@ __global__ void __launch_bounds__(256) step_tube_kernel(const StepArgs args) {
         }
     }
     if (n_unst) atomicAdd(args.status + 2 * tile.inst + 1, (unsigned long long)n_unst);
+}
+
+// The register-chunk kernel on D1Q3 (FP32 arithmetic), for single steps: a
+// launch of the tube kernel's is mostly a warp's wait for its tile's descriptor and
+// nodes, which one step does not make up for (18.0 M nodes, one step: 84 us
+// against 73 in FP32, 73 against 50 in FP16; two steps 90 against 146).  FP64
+// stays with the tube kernel (1000 tubes: 135 against 300 us).
+template <typename S, int V> const void* pick_step_single_tube_kernel() {
+    return (const void*)&step_kernel<D1Q3, S, float, V, COLL_MINXENT4>;
 }
 
 // The D2Q9 register-chunk kernel for a collision rule with storage S,

@@ -17,6 +17,8 @@ const void* step_kernel_bf16(int lattice, int collision, int V) {
     return nullptr;
 }
 
+const void* step_kernel_single_tube_bf16() { return pick_step_single_tube_kernel<__nv_bfloat16, 8>(); }
+
 const void* step_kernel_block_bf16(int collision, int rows) {
     return pick_step_block_kernel<__nv_bfloat16>(collision, rows);
 }

@@ -17,6 +17,8 @@ const void* step_kernel_f16(int lattice, int collision, int V) {
     return nullptr;
 }
 
+const void* step_kernel_single_tube_f16() { return pick_step_single_tube_kernel<__half, 8>(); }
+
 const void* step_kernel_block_f16(int collision, int rows) {
     return pick_step_block_kernel<__half>(collision, rows);
 }

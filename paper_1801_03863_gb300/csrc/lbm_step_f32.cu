@@ -18,6 +18,8 @@ const void* step_kernel_f32(int lattice, int collision, int V) {
     return nullptr;
 }
 
+const void* step_kernel_single_tube_f32() { return pick_step_single_tube_kernel<float, 4>(); }
+
 const void* step_kernel_block_f32(int collision, int rows) {
     return pick_step_block_kernel<float>(collision, rows);
 }

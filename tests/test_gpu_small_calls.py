@@ -43,3 +43,35 @@ def test_short_calls_do_not_pay_for_regions():
             assert lat.step_launches(n) == {"launches": n, "of_several_steps": 0}
         assert lat.step_launches(5 * k) == {"launches": 5, "of_several_steps": 5}
         assert lat.step_launches(5 * k + 1) == {"launches": 6, "of_several_steps": 5}
+
+@pytest.mark.parametrize("bc", ["periodic", "zero_gradient"])
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16"])
+def test_tube_calls_of_any_length_agree(bc, storage):
+    """Single steps and several steps per launch are different kernels: the same bits and counters, a
+    nearly inviscid tube's unstable nodes among them."""
+    dims = [(n, 1) for n in (1, 2, 3, 7, 64, 511, 513, 800, 4097)]
+    f0 = np.concatenate([wl.random_populations(3, 1, nx, eps=0.6, seed=nx).ravel() for nx, _ in dims])
+    got = []
+    for calls in ([30], [1] * 30, [2, 1, 5, 1, 1, 20], [29, 1]):
+        with lbm.Lattice("d1q3", dims, [1e-4] * len(dims), bc, compute="f32", storage=storage) as lat:
+            lat.set_populations(f0)
+            for k in calls:
+                lat.step(k)
+            got.append((lat.populations(), lat.status()))
+    assert got[0][1]["unstable"] > 0
+    for f, st in got[1:]:
+        assert np.array_equal(f, got[0][0]) and st == got[0][1]
+
+
+
+def test_single_steps_of_tubes_take_their_own_kernel():
+    """16 M nodes in FP16, one step: a launch of the tube kernel takes 73 us, the kernel for single steps 50;
+    in FP64 the tube kernel is ahead."""
+    for storage, several in (("f16", 0), ("f64", 1)):
+        with lbm.Lattice("d1q3", [(4000, 1)] * 64, 0.02, "zero_gradient",
+                         compute="f64" if storage == "f64" else "f32", storage=storage) as lat:
+            lat.init(np.ones(4000 * 64))
+            assert lat.step_launches(1) == {"launches": 1, "of_several_steps": 1}
+            lat.step(1)
+            assert lat.step_launches(1) == {"launches": 1, "of_several_steps": several}
+            assert lat.step_launches(2) == {"launches": 1, "of_several_steps": 1}
