@@ -602,14 +602,15 @@ __device__ __forceinline__ uint32_t mrt_d2q9(const T (&d)[9], T rho0, const Rate
 // moment fix all three populations, and BGK relaxation meets the same three
 // constraints, so both rules reduce to f + omega (f^eq - f).
 //
-// Returns a word to be passed to bgk_suspect: in FP32 the populations
-// f^post_a = W_a rho0 + out_a of all lanes or-ed as integers, which stays
-// below 2^96's pattern when every one is finite, small and not negative (a
-// sign bit, an infinity or a NaN raises it; so may a population above 2^64 or
-// a -0).  Where it is raised bgk_status decides exactly; it is not inlined, so
-// that the common path stays short (inlined: 23.2 us).  Against deciding
-// every node exactly (compares and a sum per lane) the tube kernel went from
-// 21.65 to 20.74 us a step on 18.0 M nodes in FP32, 24.87 to 23.36 in FP16.
+// Returns a word to be passed to bgk_suspect: in FP32 the largest bit pattern
+// of the populations f^post_a = W_a rho0 + out_a of all lanes, which stays
+// below 2^96's when every one is finite, not negative and below 2^96, so that their
+// sum is below 1e30 (a sign bit, an infinity or a NaN raises it; so does a -0).  Where
+// it is raised bgk_status decides exactly; it is not inlined, so that the
+// common path stays short (inlined: 23.2 us).  Against deciding every node
+// exactly (compares and a sum per lane) the tube kernel went from 21.65 to 20.74
+// us a step on 18.0 M nodes in FP32, 24.87 to 23.36 in FP16.  (The patterns or-ed
+// cost the same but mix exponents: 2 beside 1/2 looks like 2^127.)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ bool bgk_suspect(uint32_t bits) { return bits >= 0x6f800000u; }
 template <typename T> __device__ __noinline__ uint32_t bgk_status(T o0, T o1, T o2, T rho0) {
@@ -644,7 +645,7 @@ __device__ __forceinline__ uint32_t bgk_d1q3_f32(const T (&d)[3], T rho0, const 
     for (int a = 0; a < 3; ++a) {
         const T f = out[a] + T(W[a]) * rho0;
 #pragma unroll
-        for (int l = 0; l < N::LANES; ++l) bits |= __float_as_uint(N::lane(f, l));
+        for (int l = 0; l < N::LANES; ++l) bits = max(bits, __float_as_uint(N::lane(f, l)));
     }
     return bits;
 }
