@@ -902,10 +902,14 @@ __global__ void cons_final_kernel(const double* partials, const InstDesc* insts,
 }
 
 // Nodes of a block: at most 2048 (8 per thread), fewer while that leaves
-// less than 8 blocks per SM for the whole launch.
-uint32_t nodes_per_block(int64_t total) {
+// less than 8 blocks per SM for the whole launch.  Beside a large instance
+// (of max_items) the others' blocks are mostly empty ones, so an ensemble's
+// instances get at most 4096 each (one 12000 x 12000 lattice beside 5000 of 20 x
+// 20, FP16: init 179 -> 7.5 ms).
+uint32_t nodes_per_block(int64_t total, int64_t max_items, int count) {
     uint32_t per = 2048;
     while (per > AUX_THREADS && total / per < 8 * 152) per /= 2;
+    while (count > 1 && (max_items + per - 1) / per > 4096) per *= 2;
     return per;
 }
 dim3 aux_grid(int64_t max_items, int count, uint32_t per) {
@@ -916,9 +920,10 @@ template <class Lat, typename S, typename T, int COLL>
 cudaError_t collide_inplace_dispatch(const AuxArgs& a, const void* src, void* dst) {
     // node pairs of a row, rounded up per row
     const int P = std::is_same<T, float>::value ? 2 : 1;
-    const uint32_t per = nodes_per_block(a.total_nodes / P);
+    const int64_t most = a.max_nodes / P + a.max_ny;
+    const uint32_t per = nodes_per_block(a.total_nodes / P, most, a.count);
     collide_inplace_kernel<Lat, S, T, COLL>
-        <<<aux_grid(a.max_nodes / P + a.max_ny, a.count, per), AUX_THREADS, 0, a.stream>>>(
+        <<<aux_grid(most, a.count, per), AUX_THREADS, 0, a.stream>>>(
             static_cast<const S*>(src), static_cast<S*>(dst), a.inst, a.rho0, a.status, per);
     return cudaGetLastError();
 }
@@ -943,7 +948,7 @@ cudaError_t collide_inplace_by_rule(const AuxArgs& a, const void* src, void* dst
 template <class Lat, typename S>
 cudaError_t aux_dispatch(AuxOp op, const AuxArgs& a, const void* src, void* dst, const double* p0,
                          const double* p1, const double* p2, double* o0, double* o1, double* o2) {
-    const uint32_t per = nodes_per_block(a.total_nodes);
+    const uint32_t per = nodes_per_block(a.total_nodes, a.max_nodes, a.count);
     const dim3 g = aux_grid(a.max_nodes, a.count, per);
     switch (op) {
         case AuxOp::Init:
