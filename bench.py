@@ -372,12 +372,18 @@ def run_reference(args, dist):
     return 0
 
 
-def step_launches(chunks, lattice: str, shape: dict) -> int:
-    """Launches of the step kernel for lbm_step calls of these lengths: one
-    per step, but for the kernels that take several steps per launch (regions:
-    tw steps; the D1Q3 tube kernel: at most 48, counted as such)."""
-    per = 48 if lattice == "d1q3" else shape["tw"] if shape["kind"] == "block" else 1
-    return sum(-(-c // per) for c in chunks)
+def launch_figures(nodes: int, bytes_per_lu: float, steps: int, launches: int, step_ms: float,
+                   kind: str, peak: float) -> dict:
+    """Per-launch figures of the step kernel.  A launch reads and writes every
+    node once, however many steps it takes.  Only the TMA-staged kernels are
+    bound by that traffic; for the others (several steps per launch, FP64) it
+    measures nothing, so that "achieved" and "frac" are null."""
+    launch_ms = step_ms / launches
+    bound = "hbm" if kind.startswith("smem") else "arithmetic"
+    achieved = nodes * bytes_per_lu / (launch_ms * 1e-3) / 1e9 if bound == "hbm" else None
+    return {"bound": bound, "achieved": achieved, "frac": None if achieved is None else achieved / peak,
+            "algorithmic_bytes_per_launch": nodes * bytes_per_lu, "avg_launch_ms": launch_ms,
+            "steps_per_launch": steps / launches}
 
 
 def config_for(args, wk, lat):
@@ -432,6 +438,7 @@ def run_ours(args, dist):
         k -= c
     step_ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True))
                for _ in chunks]
+    launches = sum(lat.step_launches(c)["launches"] for c in chunks)
     dist.barrier()
     torch.cuda.synchronize()
     ev0.record(stream)
@@ -455,21 +462,14 @@ def run_ours(args, dist):
 
     peak, peak_kind = measured_peaks()
     bpl = wk.bytes_per_lu(args.storage)
-    launch_ms = step_ms / args.steps
-    achieved = wk.nodes * bpl / (launch_ms * 1e-3) / 1e9
     shape = lat.launch_shape()
     tpn = traffic_per_node(f"{wk.name}:{args.collision}:{args.storage}", shape["kind"])
-    # the kernels that take several steps per pass over memory, and FP64, are
-    # bound by arithmetic: their "achieved" is not a traffic figure
-    bound = "hbm" if shape["kind"].startswith("smem") else "arithmetic"
-    roofline = {"bound": bound, "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak, "peak_source": peak_kind,
+    roofline = {**launch_figures(wk.nodes, bpl, args.steps, launches, step_ms, shape["kind"], peak),
+                "peak": peak, "unit": "GB/s", "peak_source": peak_kind,
                 "traffic": None if tpn is None else tpn * wk.nodes,
-                "algorithmic_bytes_per_launch": wk.nodes * bpl,
                 "kernel": f"lbm step kernel ({shape['kind']}) {wk.lattice.upper()} "
                           f"{args.storage} storage, {args.compute} compute, "
-                          f"{args.collision.upper()}",
-                "avg_launch_ms": launch_ms}
+                          f"{args.collision.upper()}"}
 
     # the sharded path's one collective: every rank gets every member's
     # conservation totals (ensembles; single-instance runs are replicas)
@@ -487,7 +487,7 @@ def run_ours(args, dist):
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
         "dtype": args.compute, "data": "synthetic", "config": config_for(args, wk, lat),
         "roofline": roofline,
-        "gpu_launches": step_launches(chunks, wk.lattice, shape) + 2 * len(chunks),
+        "gpu_launches": launches + 2 * len(chunks),
         "clocks": sampler.summary(),
         "status": st,
         "totals": totals,
