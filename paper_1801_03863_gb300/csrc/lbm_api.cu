@@ -702,6 +702,25 @@ float time_current_shape(lbm_ctx* ctx, cudaEvent_t* ev, int steps = 1) {
     return std::min(t[0], t[1]) / 3.f;
 }
 
+// Time per step over some 12 steps of back-to-back launches of `steps` steps
+// of the current plan, the faster of two trains: long enough that the first
+// launch, which three launches are mostly, does not count.
+float time_current_train(lbm_ctx* ctx, cudaEvent_t* ev, int steps = 1) {
+    const int n = std::max(2, 12 / steps);
+    int src = 0;
+    float t[2];
+    for (int r = 0; r < 2; ++r) {
+        if (cudaEventRecord(ev[2 * r], ctx->stream) != cudaSuccess) return -1.f;
+        for (int k = 0; k < n; ++k, src ^= 1)
+            if (launch_step(ctx, ctx->plan, src, ctx->stream, false, steps) != cudaSuccess) return -1.f;
+        if (cudaEventRecord(ev[2 * r + 1], ctx->stream) != cudaSuccess) return -1.f;
+    }
+    if (cudaEventSynchronize(ev[3]) != cudaSuccess) return -1.f;
+    for (int r = 0; r < 2; ++r)
+        if (cudaEventElapsedTime(&t[r], ev[2 * r], ev[2 * r + 1]) != cudaSuccess) return -1.f;
+    return std::min(t[0], t[1]) / (float)(n * steps);
+}
+
 // The same timing through a captured graph of four launches, as the step
 // loop replays them: one warm-up replay, then the faster of two, per launch.
 // The deep ring with FP32 storage ran 5 % slower in graphs than as single
@@ -852,17 +871,14 @@ int autotune(lbm_ctx* ctx) {
     }
     // Candidates within 5 % of the fastest are timed once more, after the
     // others, through a captured graph as the step loop runs them, and
-    // that time decides between them; so is the fastest where the region
-    // kernel comes close (a graph takes 0.8 to 1 of single launches' time).
-    const bool close_region = tK >= 0.75f * K * best && tK < K * best;
+    // that time decides between them.
     int near = 0;
     for (size_t c = 0; c < cands.size(); ++c) {
         near += t[c] >= 0.f && t[c] <= 1.05f * best;
         if (t[c] == best) best_s = cands[c];
     }
-    float fastest = best;  // of one step per launch
-    if (near > 1 || close_region) {
-        fastest = 1e30f;
+    if (near > 1) {
+        float fastest = 1e30f;
         for (size_t c = 0; c < cands.size() && rc == LBM_OK; ++c) {
             if (t[c] < 0.f || t[c] > 1.05f * best) continue;
             if (apply_shape(ctx, cands[c]) != LBM_OK) continue;
@@ -880,7 +896,20 @@ int autotune(lbm_ctx* ctx) {
         }
     }
     one = best_s;
-    if (rc == LBM_OK && tK >= 0.f && tK < K * fastest) {
+    // Where the region kernel comes close to it, trains of both decide
+    // (1001 x 333 FP32 TRT: 6.1 us a step against 7.0 by three launches or a
+    // graph, and 6.1 against 5.8 in trains and in the step loop).
+    bool region = rc == LBM_OK && tK >= 0.f && tK < K * best;
+    if (region && tK >= 0.7f * K * best) {
+        float step[2] = {-1.f, -1.f};
+        if (apply_shape(ctx, Shape{2, K, rows, 5}) == LBM_OK) step[0] = time_current_train(ctx, ev, K);
+        if (apply_shape(ctx, one) == LBM_OK) step[1] = time_current_train(ctx, ev);
+        if (step[0] < 0.f || step[1] < 0.f) rc = LBM_ERR_CUDA;
+        region = step[0] < step[1];
+        if (getenv("LBM_DEBUG"))
+            fprintf(stderr, "liblbm: autotune trains: regions %.4f ms a step, kind %d %.4f\n", step[0], one.kind, step[1]);
+    }
+    if (rc == LBM_OK && region) {
         // The region kernel takes launches of the steps from which on it is
         // ahead by a tenth of single steps, whose time in a row is
         // 0.8 of what was timed.
