@@ -80,22 +80,15 @@ std::vector<Shape> candidate_shapes(int storage) {
     return out;
 }
 
-int64_t count_tiles(const std::vector<std::pair<int64_t, int64_t>>& dims, const Shape& s,
-                    int storage, bool least_padding) {
+// Tiles of the TMA kernel's geometry `variant` (kind - 1).
+int64_t count_smem_tiles(const std::vector<std::pair<int64_t, int64_t>>& dims, int variant, int storage,
+                         bool least_padding) {
     int64_t n = 0;
-    if (s.kind >= 1) {
-        for (auto& d : dims) {
-            const int tn = smem_tile_nodes(storage, s.kind - 1);
-            const int64_t X = smem_tile_width(d.first, d.second, tn, smem_threads(s.kind - 1),
-                                              least_padding);
-            const int64_t R = tn / X;
-            n += ((d.first + X - 1) / X) * ((d.second + R - 1) / R);
-        }
-        return n;
-    }
     for (auto& d : dims) {
-        const int64_t chunks = (d.first + s.V - 1) / s.V;
-        n += ((chunks + s.tw - 1) / s.tw) * ((d.second + s.th - 1) / s.th);
+        const int tn = smem_tile_nodes(storage, variant);
+        const int64_t X = smem_tile_width(d.first, d.second, tn, smem_threads(variant), least_padding);
+        const int64_t R = tn / X;
+        n += ((d.first + X - 1) / X) * ((d.second + R - 1) / R);
     }
     return n;
 }
@@ -139,9 +132,9 @@ Layout make_layout(int lattice, int storage, const std::vector<std::pair<int64_t
         bound += chunks * d.second / 128 + chunks / 4 + d.second + 1;
     }
     L.max_tiles = bound;
-    for (int kind = 1; kind <= 4; ++kind)
+    for (int variant = 0; variant < 4; ++variant)
         for (bool lp : {false, true})
-            L.max_tiles = std::max(L.max_tiles, count_tiles(dims, Shape{2, 0, 0, kind}, storage, lp));
+            L.max_tiles = std::max(L.max_tiles, count_smem_tiles(dims, variant, storage, lp));
     return L;
 }
 

@@ -51,8 +51,8 @@ __device__ __forceinline__ double widen(double v) { return v; }
 __device__ __forceinline__ double widen(__half v) { return widen(__half2float(v)); }
 __device__ __forceinline__ double widen(__nv_bfloat16 v) { return widen(__bfloat162float(v)); }
 
-// |v| of a double in FP32's normal range, as FP32 bits with `up` added below
-// the kept bits first (rounding), or -1 outside the range
+// The double with this high word lies in [2^-126, 2^127) by magnitude: FP32's
+// normal range but for its last binade, from which a rounding might overflow.
 __device__ __forceinline__ bool in_f32_range(uint32_t hi) {
     return ((hi >> 20) & 0x7ffu) - 897u < 1150u - 897u;
 }

@@ -39,8 +39,8 @@
 // each non-conserved moment k of f toward f^eq at its own rate B_k:
 //     f^post_a = f_a + sum_k T_ka B_k (m^eq_k - m_k) / d_k.
 //
-// The rules are templates over the number type T of lbm_num.cuh (double,
-// float, or F2 = two nodes at once); a[b] below always means a * b + c with
+// The rules are templates over the number type T of lbm_num.cuh (double
+// or F2 = two FP32 nodes at once); a[b] below always means a * b + c with
 // one rounding (Num<T>::mad).
 #pragma once
 #include "lbm_common.cuh"
@@ -79,17 +79,9 @@ __device__ __forceinline__ typename Num<T>::Pred finite_nonneg(const T (&out)[Q]
     typename N::Pred ok;
     if constexpr (std::is_same<T, double>::value) {
         ok = finite_nonneg_f64<Q>(out, w, rho0);
-    } else if constexpr (N::LANES == 1) {
-        ok = true;
-#pragma unroll
-        for (int a = 0; a < Q; ++a) ok = ok && (out[a] >= -T(w[a]) * rho0);
+    } else {
         // out >= c is false for NaN; a +inf population needs a non-finite input
         // and then the mass sum is not finite
-        T s = out[0];
-#pragma unroll
-        for (int a = 1; a < Q; ++a) s = s + out[a];
-        ok = ok && (fabs(s) < T(1e30));
-    } else {
         bool okx = true, oky = true;
         float sx = 0.f, sy = 0.f;
 #pragma unroll
@@ -414,11 +406,7 @@ __device__ __forceinline__ uint32_t minxent_d2q9(const T (&d)[9], T rho0, const 
         }
         rare = any != 0u;
         if (rare) {
-            if constexpr (N::LANES == 1) {
-                ok = N::lane(chk, 0) == 0.f && !neg[0];
-            } else {
-                ok = {N::lane(chk, 0) == 0.f && !neg[0], N::lane(chk, 1) == 0.f && !neg[1]};
-            }
+            ok = {N::lane(chk, 0) == 0.f && !neg[0], N::lane(chk, 1) == 0.f && !neg[1]};
             se = N::sel(ok, se, T(0.0));
             sps = N::sel(ok, sps, T(0.0));
             if constexpr (NFREE == 4) {
@@ -659,7 +647,7 @@ __device__ __forceinline__ uint32_t bgk_d1q3(const T (&d)[3], T rho0, const Rate
         // X = j u + drho / 3 - (d_1 + d_2) (the rule moves one moment and
         // conserves the others): 13 FP64 instructions with the reciprocal
         // instead of 26 (FP64 issue bounds this path; the FP32 paths keep
-        // the form below, whose rounding their results are pinned to)
+        // the form below)
         constexpr double W[3] = {2.0 / 3.0, 1.0 / 6.0, 1.0 / 6.0};
         const double n = d[1] + d[2], drho = d[0] + n, j = d[1] - d[2];
         const double u = j * N::rcp(rho0 + drho);

@@ -139,9 +139,10 @@ struct StepArgs {
     unsigned int* error;         // device error word (bounded waits that ran out)
     int32_t spin_limit;          // polls of one bounded mbarrier wait (TMA kernel)
     int32_t lost_tile;           // test hook: tile whose copies are never issued (-1: none)
-    int32_t inplace;             // collide without streaming (tube kernel: the first step)
-    int32_t steps;               // tube kernel: time steps of this launch, at most halo
-    int32_t halo;                // tube kernel: nodes carried along at either end of a segment
+    int32_t inplace;             // one-node-per-thread kernel: collide without streaming (tube
+                                 // kernel: in the first step)
+    int32_t steps;               // tube and region kernels: time steps of this launch, at most halo
+    int32_t halo;                // nodes carried along at either end of a segment or region
 };
 
 __host__ __device__ inline int64_t round_up(int64_t v, int64_t m) { return (v + m - 1) / m * m; }

@@ -2,15 +2,12 @@
 //
 // The collision rules are written once over a number type T:
 //   double  FP64 path: Newton reciprocal (below) and table logarithm (lbm_f64.cuh).
-//   float   FP32 path, one node per value.
 //   F2      FP32 path, two nodes per value: the packed FP32x2 instructions of
 //           sm_100+ (__fadd2_rn, __fmul2_rn, __ffma2_rn) do both nodes in one
 //           issue; reciprocals and logarithms run per lane on the MUFU unit.
-//   F1      FP32, one node per value (the one-off in-place collision).
 // The compiler may fuse a packed product whose only use is a following
 // packed add into one packed FMA (it does so even for the _rn forms), which
-// scalar __fmul_rn / __fadd_rn never are; so F1 and F2 agree to FP32
-// rounding, not bit for bit.  All step kernels use F2 with the same
+// scalar __fmul_rn / __fadd_rn never are.  All step kernels use F2 with the same
 // collision code and agree bit for bit with each other.
 //
 // FP32 transcendental choice: ln(p/W) is needed as log(1 + delta) with
@@ -71,22 +68,6 @@ __device__ __forceinline__ F2 operator-(F2 a, F2 b) {
 }
 __device__ __forceinline__ F2 operator*(F2 a, F2 b) { return F2(__fmul2_rn(a.v, b.v)); }
 
-// Scalar FP32: every + - * rounds separately (__fadd_rn / __fmul_rn are
-// never contracted into FMAs) and fused operations are explicit
-// (Num<F1>::mad).
-struct F1 {
-    float v;
-    F1() = default;
-    __device__ __forceinline__ constexpr F1(float a) : v(a) {}
-};
-__device__ __forceinline__ F1 operator+(F1 a, F1 b) { return F1(__fadd_rn(a.v, b.v)); }
-__device__ __forceinline__ F1 operator-(F1 a) { return F1(-a.v); }
-__device__ __forceinline__ F1 operator-(F1 a, F1 b) { return F1(__fsub_rn(a.v, b.v)); }
-__device__ __forceinline__ F1 operator*(F1 a, F1 b) { return F1(__fmul_rn(a.v, b.v)); }
-__device__ __forceinline__ bool operator>=(F1 a, F1 b) { return a.v >= b.v; }
-__device__ __forceinline__ bool operator<(F1 a, F1 b) { return a.v < b.v; }
-__device__ __forceinline__ F1 fabs(F1 a) { return F1(fabsf(a.v)); }
-
 // Per-lane predicate.
 struct B2 {
     bool x, y;
@@ -101,34 +82,6 @@ template <> struct Num<double> {
     __device__ static __forceinline__ double rcp(double x) { return rcp_f64(x); }
     __device__ static __forceinline__ double lane(double v, int) { return v; }
     __device__ static __forceinline__ void set_lane(double& v, int, double x) { v = x; }
-};
-
-template <> struct Num<float> {
-    using Pred = bool;
-    static constexpr int LANES = 1;
-    static constexpr float LOG_SCALE = 0.693147180559945309f;  // log returns log2
-    __device__ static __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-    __device__ static __forceinline__ float rcp(float x) { return rcp_approx(x); }
-    __device__ static __forceinline__ float lnp(float, float y) { return lg2_approx(y); }
-    __device__ static __forceinline__ float vmin(float a, float b) { return fminf(a, b); }
-    __device__ static __forceinline__ Pred gt(float a, float b) { return a > b; }
-    __device__ static __forceinline__ float sel(Pred p, float a, float b) { return p ? a : b; }
-    __device__ static __forceinline__ float lane(float v, int) { return v; }
-    __device__ static __forceinline__ void set_lane(float& v, int, float x) { v = x; }
-};
-
-template <> struct Num<F1> {
-    using Pred = bool;
-    static constexpr int LANES = 1;
-    static constexpr float LOG_SCALE = 0.693147180559945309f;  // log returns log2
-    __device__ static __forceinline__ F1 mad(F1 a, F1 b, F1 c) { return F1(__fmaf_rn(a.v, b.v, c.v)); }
-    __device__ static __forceinline__ F1 rcp(F1 x) { return F1(rcp_approx(x.v)); }
-    __device__ static __forceinline__ F1 lnp(F1, F1 y) { return F1(lg2_approx(y.v)); }
-    __device__ static __forceinline__ F1 vmin(F1 a, F1 b) { return F1(fminf(a.v, b.v)); }
-    __device__ static __forceinline__ Pred gt(F1 a, F1 b) { return a.v > b.v; }
-    __device__ static __forceinline__ F1 sel(Pred p, F1 a, F1 b) { return p ? a : b; }
-    __device__ static __forceinline__ float lane(F1 v, int) { return v.v; }
-    __device__ static __forceinline__ void set_lane(F1& v, int, float x) { v.v = x; }
 };
 
 template <> struct Num<F2> {
@@ -155,7 +108,6 @@ template <> struct Num<F2> {
 // Scalar type of one lane.
 template <typename T> struct LaneOf { using type = T; };
 template <> struct LaneOf<F2> { using type = float; };
-template <> struct LaneOf<F1> { using type = float; };
 
 // 4x4 symmetric positive definite solve A x = b by an LDL^T factorisation:
 // A = L D L^T with unit lower-triangular L, then L z = b, x = L^-T D^-1 z.

@@ -1,7 +1,9 @@
-// lbm_step.cuh -- the fused pull-stream + collide + boundary kernel.
+// lbm_step.cuh -- fused pull-stream + collide + boundary kernels that work in
+// registers: the register-chunk kernel (below), the FP64 kernel with one node
+// per thread and the D1Q3 kernel that takes several steps per launch.
 //
-// One launch performs one time step of Eq. (2) for every instance of a
-// context.  Populations are stored SoA (one plane per velocity, rows of
+// A launch of the register-chunk kernel performs one time step of Eq. (2) for
+// every instance of a context.  Populations are stored SoA (one plane per velocity, rows of
 // `pitch` elements, pitch a multiple of 8) as deviations from W_a rho0, and
 // the stored state is the post-collision field of the previous step, so the
 // step is a pull:
@@ -225,9 +227,7 @@ __global__ void __launch_bounds__(256) step_kernel(const StepArgs args) {
 
         // Collide nodes one at a time (FP64) or two at a time (FP32, packed
         // FP32x2 arithmetic).
-        using CT = typename std::conditional<
-            std::is_same<T, float>::value, typename std::conditional<(V % 2 == 0), F2, F1>::type,
-            T>::type;
+        using CT = typename std::conditional<std::is_same<T, float>::value, F2, T>::type;
         using N = Num<CT>;
         constexpr int P = N::LANES;
         using LT = typename LaneOf<CT>::type;
