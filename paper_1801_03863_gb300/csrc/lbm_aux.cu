@@ -497,7 +497,8 @@ __global__ void __launch_bounds__(AUX_THREADS) clear_padding_kernel(S* dst, cons
 // so that they are stored in order.  4 FP64 instructions a node besides
 // u_y's own.  8.9 M nodes in 64 lattices, FP16: 0.72 ms of moments and 0.29
 // ms of one thread per row walking its row in memory, now 0.20 ms; 257 x 257
-// FP64: 68 -> 20 us.
+// FP64: 68 -> 20 us.  Rows of up to 32 nodes share a warp (4 x 100000 FP64: 205
+// -> 22 us; with one thread per row 41 us).
 constexpr int PSI_WARPS = 4, PSI_NODES = 256;
 template <typename S>
 __global__ void __launch_bounds__(PSI_WARPS * 32)
@@ -507,6 +508,38 @@ stream_function_kernel(const S* src, const InstDesc* insts, bool pulled, double 
     const InstDesc& in = insts[blockIdx.y];
     const int nx = in.nx, lane = (int)(threadIdx.x & 31u);
     double* u = buf[threadIdx.x >> 5];
+    auto velocity = [&](int x, int y) {  // u_y
+        S raw[9];
+        node_state<D2Q9, S>(src, in, x, y, pulled, raw);
+        double m, jx, jy;
+        node_sums<D2Q9, S>(raw, m, jx, jy);
+        return jy * rcp_f64(rho0 + m);
+    };
+    if (nx <= 32) {
+        // rows that 16 lanes or fewer hold, 2 nodes each, share a warp
+        int log_lanes = 0;
+        while ((2 << log_lanes) < nx) ++log_lanes;
+        const int lanes = 1 << log_lanes, l = lane & (lanes - 1), x = 2 * l;
+        const int64_t rows = 32 >> log_lanes, all = (int64_t)gridDim.x * PSI_WARPS * rows;
+        for (int64_t y0 = ((int64_t)blockIdx.x * PSI_WARPS + (threadIdx.x >> 5)) * rows; y0 < in.ny; y0 += all) {
+            const int64_t y = y0 + (lane >> log_lanes);
+            const bool a = y < in.ny && x < nx, b = y < in.ny && x + 1 < nx;
+            const double v0 = a ? velocity(x, (int)y) : 0.0, v1 = b ? velocity(x + 1, (int)y) : 0.0;
+            const double w0 = __shfl_up_sync(0xffffffffu, v0, 1), w1 = __shfl_up_sync(0xffffffffu, v1, 1);
+            const double inc = l == 0 ? 0.0 : fma(4.0, w1, w0 + v0) * (1.0 / 3.0);
+            double sum = inc;
+            for (int d = 1; d < lanes; d <<= 1) {
+                const double o = __shfl_up_sync(0xffffffffu, sum, d);
+                if (l >= d) sum += o;
+            }
+            const double left = __shfl_up_sync(0xffffffffu, sum, 1);
+            const double e = (l == 0 ? 0.0 : left) + inc;
+            double* p = psi + (in.node0 - node_base) + y * nx + x;
+            if (a) p[0] = -e;
+            if (b) p[1] = -fma(0.5, v0 + v1, e);
+        }
+        return;
+    }
     for (int y = blockIdx.x * PSI_WARPS + (int)(threadIdx.x >> 5); y < in.ny; y += gridDim.x * PSI_WARPS) {
         double* p = psi + (in.node0 - node_base) + (int64_t)y * nx;
         double carry = 0.0;  // integral over [0, x0 - 2]
@@ -519,13 +552,7 @@ stream_function_kernel(const S* src, const InstDesc* insts, bool pulled, double 
             for (int i = 0; i < 32 * L; i += 32) {
                 const int x = x0 + i + lane;
                 double v = 0.0;
-                if (x < nx) {
-                    S raw[9];
-                    node_state<D2Q9, S>(src, in, x, y, pulled, raw);
-                    double m, jx, jy;
-                    node_sums<D2Q9, S>(raw, m, jx, jy);
-                    v = jy * rcp_f64(rho0 + m);
-                }
+                if (x < nx) v = velocity(x, y);
                 u[2 + i + lane] = v;
                 last = v;
             }
