@@ -1287,7 +1287,8 @@ int lbm_create_batch(lbm_ctx** out, lbm_lattice lat, int32_t count, const int64_
     {
         std::vector<int2> items;
         for (int i = 0; i < count; ++i)
-            for (int b = 0; b < cons_partials(ctx->layout.inst[i].nx, ctx->layout.inst[i].ny); ++b) items.push_back({i, b});
+            for (int b = 0; b < cons_partials(ctx->layout.inst[i].nx, ctx->layout.inst[i].ny, (int)dtype_bytes(o.storage)); ++b)
+                items.push_back({i, b});
         ctx->n_cons = (int)items.size();
         if (cudaMemcpyAsync(ctx->d_cons, items.data(), sizeof(int2) * items.size(),
                             cudaMemcpyHostToDevice, ctx->stream) != cudaSuccess ||

@@ -697,13 +697,17 @@ __device__ __forceinline__ bool half_sums(const float (&d)[Lat::Q], long long (&
 
 __device__ __noinline__ double add_slow(long long a, long long b) { return (double)a + (double)b; }
 
-template <class Lat, typename S>
+// CLUSTER: launched in clusters of several CTAs.  totals (null: none): every
+// instance is one partial, and pass 2 is spared (5000 tubes of 100 nodes, FP32
+// 33 us with it).
+template <class Lat, typename S, bool CLUSTER>
 __global__ void __launch_bounds__(CONS_THREADS, 3)
-cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool pulled, double* partials) {
+cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool pulled, double* partials,
+                    double rho0, double* totals) {
     constexpr int Q = Lat::Q, E = 16 / (int)sizeof(S);  // nodes per chunk
     const int2 it = items[blockIdx.x];
     const InstDesc& in = insts[it.x];
-    const int nx = in.nx, ny = in.ny, P = cons_partials(nx, ny);
+    const int nx = in.nx, ny = in.ny, P = cons_partials(nx, ny, (int)sizeof(S));
     const uint32_t C = (uint32_t)cons_split((int64_t)nx * ny), rank = blockIdx.y;
     const uint32_t chunks = (uint32_t)(nx + E - 1) / E;       // per row
     const uint64_t total = (uint64_t)((ny - it.y + P - 1) / P) * chunks;
@@ -831,8 +835,13 @@ cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool
                 }
             }
         }
-    // fixed trees: threads, then the CTAs of the cluster in order
+    // fixed trees: threads, then the CTAs of the cluster in order; the terms of
+    // threads and warps without nodes, zeros, are left out
     __shared__ double cta[3];
+    const uint64_t before = (uint64_t)rank * CONS_THREADS;
+    const uint32_t threads = rank < C && total > before ? (uint32_t)min(total - before, (uint64_t)CONS_THREADS) : 0u;
+    const uint32_t warps = (threads + 31u) / 32u, lanes = min(threads, 32u);  // with nodes
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u;
     if constexpr (std::is_same<S, __half>::value) {
         // integers add exactly within a warp; FP64 only holds nodes with non-finite values.
         // A lane has some 2^15 nodes at most (2^31 nodes of an instance, of at least 1 in 8 CTAs
@@ -840,87 +849,107 @@ cons_partial_kernel(const S* src, const InstDesc* insts, const int2* items, bool
         // 2^15 x 9 x 2^40 < 2^58.2 and those of 16 lanes below 2^62.2; those of
         // two such halves may not fit.
         __shared__ double sh[3][CONS_THREADS / 32];
-        double s[3] = {t.s0, t.s1, t.s2};
-        long long i[3] = {t.i0, t.i1, t.i2};
-        const bool in_f64 = __any_sync(0xffffffffu, !(s[0] == 0.0 && s[1] == 0.0 && s[2] == 0.0));
+        if (warp < warps) {
+            double s[3] = {t.s0, t.s1, t.s2};
+            long long i[3] = {t.i0, t.i1, t.i2};
+            const bool in_f64 = __any_sync(0xffffffffu, !(s[0] == 0.0 && s[1] == 0.0 && s[2] == 0.0));
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
+            for (int c = 0; c < (Q == 3 ? 2 : 3); ++c) {
 #pragma unroll
-            for (int h = 16; h > 1; h >>= 1) i[c] += __shfl_down_sync(0xffffffffu, i[c], h);
-            const long long o = __shfl_down_sync(0xffffffffu, i[c], 1);
-            const long long sum = (long long)((uint64_t)i[c] + (uint64_t)o);
-            if ((threadIdx.x & 31u) == 0u) {
-                const bool wraps = ((i[c] ^ sum) & (o ^ sum)) < 0;
-                s[c] += (wraps ? add_slow(i[c], o) : (double)sum) * (1.0 / 16777216.0);
+                for (int h = 16; h > 1; h >>= 1) i[c] += __shfl_down_sync(0xffffffffu, i[c], h);
+                const long long o = __shfl_down_sync(0xffffffffu, i[c], 1);
+                const long long sum = (long long)((uint64_t)i[c] + (uint64_t)o);
+                if (lane == 0u) {
+                    const bool wraps = ((i[c] ^ sum) & (o ^ sum)) < 0;
+                    s[c] += (wraps ? add_slow(i[c], o) : (double)sum) * (1.0 / 16777216.0);
+                }
+                if (in_f64) {
+#pragma unroll
+                    for (int h = 16; h > 0; h >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], h);
+                }
+                if (lane == 0u) sh[c][warp] = s[c];
             }
-            if (in_f64) {
-#pragma unroll
-                for (int h = 16; h > 0; h >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], h);
-            }
-            if ((threadIdx.x & 31u) == 0u) sh[c][threadIdx.x >> 5] = s[c];
         }
         __syncthreads();
         if (threadIdx.x < 3) {
             double v = 0.0;
-#pragma unroll
-            for (int w = 0; w < CONS_THREADS / 32; ++w) v += sh[threadIdx.x][w];
+            if (threadIdx.x < (Q == 3 ? 2 : 3))
+                for (uint32_t w = 0; w < warps; ++w) v = w == 0u ? sh[threadIdx.x][0] : v + sh[threadIdx.x][w];
             cta[threadIdx.x] = v;
         }
     } else {
         // A thread's sums in FP64, then one warp per sum adds them: 8 of every lane and a shuffle
         // tree, 36 FP64 warp instructions a CTA where a tree in each warp takes 120
         __shared__ double sh[3][CONS_THREADS];
-        double s[3] = {t.s0, t.s1, t.s2};
-        if constexpr (!std::is_same<S, double>::value) {
-            const F2 h[3] = {t.h0, t.h1, t.h2}, e[3] = {t.c0, t.c1, t.c2};
+        if (warp < warps) {
+            double s[3] = {t.s0, t.s1, t.s2};
+            if constexpr (!std::is_same<S, double>::value) {
+                const F2 h[3] = {t.h0, t.h1, t.h2}, e[3] = {t.c0, t.c1, t.c2};
 #pragma unroll
-            for (int c = 0; c < (Q == 3 ? 2 : 3); ++c) {
-                // the thread's two node lanes as one pair
-                const float x = h[c].v.x, y = h[c].v.y;
-                const float sum = __fadd_rn(x, y), bv = __fsub_rn(sum, x);
-                const float r = __fadd_rn(__fadd_rn(e[c].v.x, e[c].v.y),
-                                          __fadd_rn(__fsub_rn(x, __fsub_rn(sum, bv)), __fsub_rn(y, bv)));
-                const double v = widen(sum) + widen(r);
-                s[c] = __double_as_longlong(s[c]) == 0 ? v : s[c] + v;  // (FP64 part: nodes that are not finite)
+                for (int c = 0; c < (Q == 3 ? 2 : 3); ++c) {
+                    // the thread's two node lanes as one pair
+                    const float x = h[c].v.x, y = h[c].v.y;
+                    const float sum = __fadd_rn(x, y), bv = __fsub_rn(sum, x);
+                    const float r = __fadd_rn(__fadd_rn(e[c].v.x, e[c].v.y),
+                                              __fadd_rn(__fsub_rn(x, __fsub_rn(sum, bv)), __fsub_rn(y, bv)));
+                    const double v = widen(sum) + widen(r);
+                    s[c] = __double_as_longlong(s[c]) == 0 ? v : s[c] + v;  // (FP64 part: nodes that are not finite)
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < (Q == 3 ? 2 : 3); ++c) sh[c][threadIdx.x] = s[c];
+        }
+        __syncthreads();
+        if (warp < 3u) {
+            double v = 0.0;
+            if (warp < (Q == 3 ? 2u : 3u) && warps > 0u) {
+                v = sh[warp][lane];
+                for (uint32_t w = 1; w < warps; ++w) v += sh[warp][lane + 32u * w];
+#pragma unroll
+                for (uint32_t h = 16; h > 0; h >>= 1)
+                    if (lanes > h) v += __shfl_down_sync(0xffffffffu, v, h);
+            }
+            if (lane == 0u) cta[warp] = v;
+        }
+    }
+    double* out = partials + ((int64_t)it.x * CONS_PARTIALS + it.y) * 3;
+    if constexpr (CLUSTER) {
+        const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+        cluster.sync();
+        if (rank == 0 && threadIdx.x < 3) {
+            double v = 0.0;
+            for (uint32_t r = 0; r < C; ++r) v += *cluster.map_shared_rank(&cta[threadIdx.x], r);
+            out[threadIdx.x] = v;
+        }
+        cluster.sync();  // a CTA's shared memory stays until the first has read it
+    } else {
+        __syncthreads();
+        if (threadIdx.x < 3) {
+            const double v = cta[threadIdx.x];
+            if (totals) {  // one partial an instance: its totals
+                totals[3 * it.x + threadIdx.x] = threadIdx.x == 0 ? (double)nx * (double)ny * rho0 + v : v;
+            } else {
+                out[threadIdx.x] = v;
             }
         }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) sh[c][threadIdx.x] = s[c];
-        __syncthreads();
-        const int c = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31u);
-        if (c < 3) {
-            double v = sh[c][lane];
-#pragma unroll
-            for (int w = 1; w < CONS_THREADS / 32; ++w) v += sh[c][lane + 32 * w];
-#pragma unroll
-            for (int h = 16; h > 0; h >>= 1) v += __shfl_down_sync(0xffffffffu, v, h);
-            if (lane == 0) cta[c] = v;
-        }
     }
-    const cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
-    cluster.sync();
-    if (rank == 0 && threadIdx.x < 3) {
-        double v = 0.0;
-        for (uint32_t r = 0; r < C; ++r) v += *cluster.map_shared_rank(&cta[threadIdx.x], r);
-        partials[((int64_t)it.x * CONS_PARTIALS + it.y) * 3 + threadIdx.x] = v;
-    }
-    cluster.sync();  // a CTA's shared memory stays until the first has read it
 }
 
 // Conservation, pass 2: one warp per instance adds its partials in a fixed
 // tree; total mass = N rho0 + sum d (sum_a W_a = 1).
-__global__ void cons_final_kernel(const double* partials, const InstDesc* insts, int count,
+__global__ void cons_final_kernel(const double* partials, const InstDesc* insts, int count, int bytes,
                                   double rho0, double* out) {
     const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = (int)(threadIdx.x & 31u);
     if (i >= count) return;
-    const int P = cons_partials(insts[i].nx, insts[i].ny);
+    const int P = cons_partials(insts[i].nx, insts[i].ny, bytes);
     double s[3] = {0.0, 0.0, 0.0};
     for (int b = lane; b < P; b += 32)
         for (int c = 0; c < 3; ++c) s[c] += partials[((int64_t)i * CONS_PARTIALS + b) * 3 + c];
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
-        for (int h = 16; h > 0; h >>= 1) s[c] += __shfl_down_sync(0xffffffffu, s[c], h);
+        for (int h = 16; h > 0; h >>= 1)
+            if (P > h) s[c] += __shfl_down_sync(0xffffffffu, s[c], h);  // (others' terms are zeros)
     if (lane != 0) return;
     const double nodes = (double)insts[i].nx * (double)insts[i].ny;
     out[3 * i + 0] = nodes * rho0 + s[0];
@@ -1016,22 +1045,29 @@ cudaError_t aux_dispatch(AuxOp op, const AuxArgs& a, const void* src, void* dst,
             if (a.cons_nitems < 1 || !a.cons_items) return cudaErrorInvalidValue;
             // clusters of as many CTAs as the largest instance splits into
             const unsigned C = (unsigned)cons_split(a.max_nodes);
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 1;
-            attr[0].val.clusterDim.y = C;
-            attr[0].val.clusterDim.z = 1;
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)a.cons_nitems, C);
-            cfg.blockDim = dim3(CONS_THREADS);
-            cfg.stream = a.stream;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            const cudaError_t e = cudaLaunchKernelEx(&cfg, &cons_partial_kernel<Lat, S>,
-                                                     static_cast<const S*>(src), a.inst, a.cons_items,
-                                                     a.pulled, o1);
-            if (e != cudaSuccess) return e;
-            cons_final_kernel<<<(a.count + 3) / 4, 128, 0, a.stream>>>(o1, a.inst, a.count, a.rho0, o0);
+            const S* planes = static_cast<const S*>(src);
+            if (C == 1) {
+                cons_partial_kernel<Lat, S, false>
+                    <<<a.cons_nitems, CONS_THREADS, 0, a.stream>>>(planes, a.inst, a.cons_items, a.pulled, o1, a.rho0,
+                                                                   a.cons_nitems == a.count ? o0 : nullptr);
+                if (a.cons_nitems == a.count) break;
+            } else {
+                cudaLaunchAttribute attr[1];
+                attr[0].id = cudaLaunchAttributeClusterDimension;
+                attr[0].val.clusterDim.x = 1;
+                attr[0].val.clusterDim.y = C;
+                attr[0].val.clusterDim.z = 1;
+                cudaLaunchConfig_t cfg = {};
+                cfg.gridDim = dim3((unsigned)a.cons_nitems, C);
+                cfg.blockDim = dim3(CONS_THREADS);
+                cfg.stream = a.stream;
+                cfg.attrs = attr;
+                cfg.numAttrs = 1;
+                const cudaError_t e = cudaLaunchKernelEx(&cfg, &cons_partial_kernel<Lat, S, true>, planes, a.inst,
+                                                         a.cons_items, a.pulled, o1, a.rho0, (double*)nullptr);
+                if (e != cudaSuccess) return e;
+            }
+            cons_final_kernel<<<(a.count + 3) / 4, 128, 0, a.stream>>>(o1, a.inst, a.count, (int)sizeof(S), a.rho0, o0);
             break;
         }
         case AuxOp::CollideInPlace: {

@@ -14,12 +14,13 @@ namespace lbm {
 // on the device or on the other instances.
 constexpr int CONS_PARTIALS = 64;
 constexpr int CONS_THREADS = 256;
-// one partial per CONS_NODES nodes, at most one per row (with 64 for every
+// one partial per 1024 nodes, at most one per row (with 64 for every
 // lattice the smallest ones' CTAs are mostly tail: 121 us on 64 lattices of
-// 64^2 to 1024^2, FP16, now 93 us)
-constexpr int CONS_NODES = 1024;
-__host__ __device__ inline int cons_partials(int nx, int ny) {
-    const int64_t want = ((int64_t)nx * ny + CONS_NODES - 1) / CONS_NODES;
+// 64^2 to 1024^2, FP16, now 93 us); per 512 with FP64 storage, whose additions
+// take an SM 5 ns a node
+__host__ __device__ inline int cons_partials(int nx, int ny, int bytes) {
+    const int nodes = bytes == 8 ? 512 : 1024;
+    const int64_t want = ((int64_t)nx * ny + nodes - 1) / nodes;
     const int most = ny < CONS_PARTIALS ? ny : CONS_PARTIALS;
     return want < most ? (int)want : most;
 }
