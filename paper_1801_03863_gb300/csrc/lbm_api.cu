@@ -56,6 +56,7 @@ struct StepPlan {
     int grid = 0;
     size_t smem = 0;  // dynamic shared memory
     int32_t tile0 = 0, ntiles = 0;
+    bool draws = false;   // TMA kernel: tiles beyond the CTAs' first two are drawn
     int flat_nodes = 0;   // one-node-per-thread kernel: nodes per tile-table entry
     int halo = 0;         // tube and region kernels: halo nodes, steps per launch
     int block_warps = 0;  // region kernel: warps of a CTA
@@ -539,6 +540,7 @@ int make_plan(lbm_ctx* ctx, const Shape& s, int halo, int32_t tile0, StepPlan* o
         if (2 * gd < (int64_t)t.size()) {
             k = kd;
             g = gd;
+            p.draws = true;
         }
     }
     p.kern = k;
@@ -1114,6 +1116,7 @@ uint64_t layout_hash(const lbm_ctx* ctx) {
 // launch that timed out may leave them otherwise, so every entry point that
 // sets a state clears them (the sticky error word is another matter).
 cudaError_t clear_tile_counters(lbm_ctx* ctx) {
+    if (!ctx->plan.draws && !ctx->single.draws) return cudaSuccess;
     return cudaMemsetAsync(ctx->d_error + TILE_COUNTERS, 0, 2 * sizeof(unsigned int), ctx->stream);
 }
 
@@ -1677,9 +1680,15 @@ int lbm_save_state(lbm_ctx* ctx, void* host_buf) {
     h.buf_bytes = ctx->cv.buf_bytes;
     char* out = static_cast<char*>(host_buf);
     std::memcpy(out, &h, sizeof h);
-    AuxArgs a = aux_args(ctx);
-    LBM_CK(run_aux(AuxOp::ClearPadding, a, nullptr, ctx->buf[ctx->cur], nullptr, nullptr, nullptr,
-                   nullptr, nullptr, nullptr));
+    // Nothing reads the columns [nx, pitch), but the TMA kernel's stores,
+    // clipped at 16 bytes, leave values there where the region kernel does
+    // not, and the saved state is to be the same whichever took the steps.
+    if (ctx->plan.shape.block() && std::any_of(ctx->layout.inst.begin(), ctx->layout.inst.end(),
+                                               [](const InstDesc& in) { return in.pitch != in.nx; })) {
+        AuxArgs a = aux_args(ctx);
+        LBM_CK(run_aux(AuxOp::ClearPadding, a, nullptr, ctx->buf[ctx->cur], nullptr, nullptr, nullptr,
+                       nullptr, nullptr, nullptr));
+    }
     LBM_CK(cudaMemcpyAsync(out + sizeof h, ctx->d_status, h.status_bytes, cudaMemcpyDeviceToHost,
                            ctx->stream));
     LBM_CK(cudaMemcpyAsync(out + sizeof h + h.status_bytes, ctx->buf[ctx->cur], h.buf_bytes,
