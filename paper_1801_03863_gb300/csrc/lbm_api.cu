@@ -678,21 +678,23 @@ cudaError_t launch_step(lbm_ctx* ctx, const StepPlan& p, int src, cudaStream_t s
 }
 
 // Time of a launch of `steps` steps of the current plan in milliseconds, on
-// the rest-state buffers: after an untimed launch twice three back-to-back
-// launches (as the step loop runs them: a launch's tail overlaps the next
+// the rest-state buffers: after an untimed launch three back-to-back
+// launches, twice for single steps (as the step loop runs them: a launch's tail overlaps the next
 // one's start), the faster of the two; < 0 on a CUDA error.
 float time_current_shape(lbm_ctx* ctx, cudaEvent_t* ev, int steps = 1) {
+    // (several steps make a launch long enough for one run to do)
+    const int runs = steps == 1 ? 2 : 1;
     if (launch_step(ctx, ctx->plan, 0, ctx->stream, false, steps) != cudaSuccess) return -1.f;
     int src = 1;
-    float t[2];
-    for (int r = 0; r < 2; ++r) {
+    float t[2] = {1e30f, 1e30f};
+    for (int r = 0; r < runs; ++r) {
         if (cudaEventRecord(ev[2 * r], ctx->stream) != cudaSuccess) return -1.f;
         for (int k = 0; k < 3; ++k, src ^= 1)
             if (launch_step(ctx, ctx->plan, src, ctx->stream, false, steps) != cudaSuccess) return -1.f;
         if (cudaEventRecord(ev[2 * r + 1], ctx->stream) != cudaSuccess) return -1.f;
     }
-    if (cudaEventSynchronize(ev[3]) != cudaSuccess) return -1.f;
-    for (int r = 0; r < 2; ++r)
+    if (cudaEventSynchronize(ev[2 * runs - 1]) != cudaSuccess) return -1.f;
+    for (int r = 0; r < runs; ++r)
         if (cudaEventElapsedTime(&t[r], ev[2 * r], ev[2 * r + 1]) != cudaSuccess) return -1.f;
     return std::min(t[0], t[1]) / 3.f;
 }
@@ -861,8 +863,7 @@ int autotune(lbm_ctx* ctx) {
     if (rc == LBM_OK && block_plan(ctx, &K, &rows, &us) && us < 1e3 * best &&
         apply_shape(ctx, Shape{2, K, rows, 5}) == LBM_OK) {
         tK = time_current_shape(ctx, ev, K);
-        t1 = time_current_shape(ctx, ev, 1);
-        if (tK < 0.f || t1 < 0.f) rc = LBM_ERR_CUDA;
+        if (tK < 0.f) rc = LBM_ERR_CUDA;
     }
     // Candidates within 5 % of the fastest are timed once more, after the
     // others, through a captured graph as the step loop runs them, and
@@ -909,6 +910,8 @@ int autotune(lbm_ctx* ctx) {
         // ahead by a tenth of single steps, whose time in a row is
         // 0.8 of what was timed.
         best_s = {2, K, rows, 5};
+        if (apply_shape(ctx, best_s) == LBM_OK) t1 = time_current_shape(ctx, ev, 1);
+        if (t1 < 0.f) rc = LBM_ERR_CUDA;
         const float slope = (tK - t1) / (K - 1);
         from = {1, 0, 0};
         while (from.V < K && t1 + (from.V - 1) * slope > 0.9f * 0.8f * from.V * best) ++from.V;
