@@ -299,9 +299,9 @@ int block_threads(const lbm_ctx* ctx, const StepPlan& p) {
 // step of one segment alone on its scheduler / of one segment among many,
 // and per launch) are fits of measurements, V and halo swept over single
 // tubes of 800 to 20000 nodes and ensembles of 200 to 4096 tubes:
-//   800 nodes FP64: V 1, halo 12: 0.76 us a step (V 2, halo 8: 1.45);
+//   800 nodes FP64: V 1, halo 12: 0.78 us a step (V 2, halo 8: 1.45);
 //   800 nodes FP32: V 2, halo 24: 0.19 us (V 4, halo 8: 0.43);
-//   4096 tubes (18.0 M nodes) FP32: V 8, halo 8..16: 21.7 us (V 2: 32.2).
+//   4096 tubes (18.0 M nodes) FP32: V 8, halo 8..16: 21.0 us (V 2: 32.2).
 // V_pinned != 0 (LBM_SHAPE) fixes V.
 void tube_plan(const lbm_ctx* ctx, int V_pinned, int* V, int* halo) {
     struct Cost {
@@ -679,8 +679,9 @@ cudaError_t launch_step(lbm_ctx* ctx, const StepPlan& p, int src, cudaStream_t s
 
 // Time of a launch of `steps` steps of the current plan in milliseconds, on
 // the rest-state buffers: after an untimed launch three back-to-back
-// launches, twice for single steps (as the step loop runs them: a launch's tail overlaps the next
-// one's start), the faster of the two; < 0 on a CUDA error.
+// launches (as the step loop runs them: a launch's tail overlaps the next
+// one's start), for single steps the faster of two such runs; < 0 on a CUDA
+// error.
 float time_current_shape(lbm_ctx* ctx, cudaEvent_t* ev, int steps = 1) {
     // (several steps make a launch long enough for one run to do)
     const int runs = steps == 1 ? 2 : 1;

@@ -219,7 +219,7 @@ __device__ __forceinline__ bool finite_nonneg_f64(const double (&out)[Q], const 
 //     [ .           .          C13 + Sd     C57 - C68 ]
 //     [ .           .          .            C24 + Sd  ],
 // C = c r, X = -h r, Sa = C13 + C24, Sd = C57 + C68, q0 = 1 / y_0.
-// ~255 FP64 instructions per node (MinxEnt4), against 485 with log1p, IEEE
+// 252 FP64 instructions per node (MinxEnt4), against 485 with log1p, IEEE
 // divisions and the system in the rows of T.
 // ---------------------------------------------------------------------------
 template <int NFREE>

@@ -330,15 +330,15 @@ __global__ void __launch_bounds__(256) step_kernel(const StepArgs args) {
 //
 // The hardware deals CTAs to SMs unevenly while some still have room, so the
 // launch claims shared memory that leaves each SM room for its equal share
-// and no more (257 x 257: 37.2 -> 34.2 us a step; at most 128 registers, so
+// and no more (257 x 257: 37.2 -> 34.2 us a step, then; at most 128 registers, so
 // that 16 warps fit an SM: with more, 38.9).
 //
 // Measured, MinxEnt4, per step, against the register-chunk kernel with log1p
-// and IEEE divisions: 120 lattices of 17 x 17: 122.5 -> 18.7 us; 257 x 257:
-// 110 -> 34.2 us; 800 x 4: 50 -> 10.7 us; 2048 x 2048: 3680 -> 1900 us (250
-// FP64 instructions per node against 485; 0.88 of the FP64 issue rate).  The
-// smallest lattices are bound by one warp's instructions (250 x 64 cycles =
-// 7.7 us) and the launch.
+// and IEEE divisions: 120 lattices of 17 x 17: 122.4 -> 18.8 us; 257 x 257:
+// 110 -> 34.5 us; 800 x 4: 52.6 -> 12.2 us; 2048 x 2048: 3680 -> 1920 us (252
+// FP64 instructions per node against 485; 0.87 of the FP64 issue rate).  The
+// smallest lattices are bound by one warp's instructions (252 x 64 cycles =
+// 7.8 us) and the launch.
 //
 // inplace: the first step after a state was loaded collides f(x, t_n) itself,
 // without streaming.

@@ -24,8 +24,9 @@
 //    copies landed) and an "empty" one (every colliding warp is done with
 //    it).  One warp of the CTA only moves data: it fills every stage at the
 //    start, and whenever the colliding warps are done with a tile it writes
-//    the stage's nine planes out with one tensor store each (rows and chunks
-//    beyond the lattice are clipped by the hardware), waits for TMA to have
+//    the stage's nine planes out with one tensor store each (the hardware
+//    clips rows beyond the lattice and 16-byte words beyond its last column,
+//    so up to 16 bytes of row padding are written), waits for TMA to have
 //    read them and refills the stage with the tile NS later.  Issuing those
 //    26 copies takes a few thousand cycles per tile; a colliding warp that
 //    did it (as the last one to finish a tile) fell behind every time and
